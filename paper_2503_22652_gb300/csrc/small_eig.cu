@@ -28,8 +28,10 @@
 #include <cfloat>
 
 #include "common.cuh"
+#include "oz_digits.cuh"
 #include "oz_gemm.cuh"
 #include "prof.cuh"
+#include "tc_ptx.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -68,65 +70,60 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Two warp sums with their shuffle / add latencies interleaved.
-__device__ __forceinline__ void warp_sum2(double& a, double& b) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const double ta = __shfl_xor_sync(0xffffffffu, a, o), tb = __shfl_xor_sync(0xffffffffu, b, o);
-    a += ta;
-    b += tb;
-  }
+// What an FP64 instruction costs here (clock64): every SM sub-partition issues one warp-wide FP64
+// instruction per 64 clocks, whatever its active lanes and however independent it is of the one
+// before (16 dependent or independent DFMAs of a warp: 1000 clocks).  The kernels below therefore
+// count FP64 instructions per sub-partition: full lanes, no redundant scalar work in FP64, sums
+// across lanes and seeds in the integer and FP32 units.
+
+// Sum over the warp of one double per lane, every lane receiving it, in integer arithmetic: the
+// lanes' significands are aligned to the largest exponent (9 guard bits below its last place), cut
+// into 26-bit limbs and added with redux.sync.  The result is within 1/8 unit in the last place of
+// the largest addend plus one rounding, closer than a tree of FP64 adds, and costs one FP64
+// instruction (a conversion) instead of five.  Non-finite addends take the FP64 tree (NaN and Inf
+// propagate); a result below the normal range is 0.
+__device__ __forceinline__ double warp_sum_fx(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const uint32_t e0 = (hi >> 20) & 0x7ffu;
+  const uint32_t ex = max(e0, 1u);
+  const uint32_t top = __reduce_max_sync(0xffffffffu, ex);
+  if (top == 0x7ffu) return warp_sum(v);
+  const uint32_t sh = min(top - ex, 63u);
+  const uint32_t mh = (hi & 0xfffffu) | (e0 ? 0x100000u : 0u);
+  const unsigned long long mant = ((((unsigned long long)mh << 32) | lo) << 9) >> sh;
+  const long long f = (int32_t)hi < 0 ? -(long long)mant : (long long)mant;
+  // f = h 2^52 + m 2^26 + l with 0 <= m, l < 2^26: 32 limbs of 26 bits add up below 2^31
+  const uint32_t l = (uint32_t)f & 0x3ffffffu, m = (uint32_t)(f >> 26) & 0x3ffffffu;
+  const int h = (int)(f >> 52);
+  const uint32_t sl = __reduce_add_sync(0xffffffffu, l), sm = __reduce_add_sync(0xffffffffu, m);
+  const int sg = __reduce_add_sync(0xffffffffu, h);
+  const long long t = ((long long)sg << 47) + ((long long)sm << 21) + (long long)(sl >> 5);
+  const double d = __ll2double_rn(t);  // scaled by 2^(top - 1075 - 9 + 5) below
+  const int he = __double2hiint(d), ef = ((he >> 20) & 0x7ff) + (int)top - 1079;
+  return t != 0 && ef > 0 ? __hiloint2double(he + (((int)top - 1079) << 20), __double2loint(d)) : 0.0;
 }
 
-// The loops below walk rows in warp-uniform chunks of 32, four chunks per iteration with all loads
-// issued before the FMAs: an FP64 FMA has ~64 clocks of latency, so a load-FMA-store chain per
-// element leaves the FP64 pipe idle, while a chunk that lies past the end is skipped as a whole (on
-// this GPU a warp-wide FP64 instruction occupies the SM's FP64 pipe for ~12 clocks whatever its
-// active lanes, so the FMA count must stay that of the plain loop).
-// Lane partial of sum_{i < rr} mc[i] v[i].
-__device__ __forceinline__ double dot_part(const double* mc, const double* v, int rr, int lane) {
-  double a0 = 0.0, a1 = 0.0;
-  for (int c0 = 0; c0 < rr; c0 += 128) {
-    double m[4], x[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = c0 + 32 * u + lane;
-      m[u] = i < rr ? mc[i] : 0.0;
-      x[u] = i < rr ? v[i] : 0.0;
-    }
-    if (c0 < rr) a0 = fma(m[0], x[0], a0);
-    if (c0 + 32 < rr) a1 = fma(m[1], x[1], a1);
-    if (c0 + 64 < rr) a0 = fma(m[2], x[2], a0);
-    if (c0 + 96 < rr) a1 = fma(m[3], x[3], a1);
-  }
-  return a0 + a1;
+// 1 / sqrt(a) for a normal a > 0: FP32 seed y (22 bits), then one step of the third-order Householder
+// iteration y (1 + e / 2 + 3 e^2 / 8), e = 1 - a y^2 (error e^3): 5 FP64 instructions.
+__device__ __forceinline__ double rsqrt_h3(double a) {
+  const int hi = __double2hiint(a), lo = __double2loint(a);
+  const int eb = ((hi >> 20) & 0x7ff) - 1023, hf = eb >> 1;  // a = m 4^hf, m in [1, 4)
+  const float m = __int_as_float(((eb - 2 * hf + 127) << 23) | ((hi & 0xfffff) << 3) | (int)((uint32_t)lo >> 29));
+  const int yb = __float_as_int(rsqrtf(m));
+  const double y = __hiloint2double((((yb >> 23) - 127 + 1023 - hf) << 20) | ((yb >> 3) & 0xfffff), yb << 29);
+  const double e = fma(-a, y * y, 1.0);
+  return fma(e * y, fma(0.375, e, 0.5), y);
 }
 
-// mc[i] -= v[i] wc + w[i] vc for i < rr; with S2, also the lane partial of sum_{i >= 2} mc[i]^2 of
-// the new values.
-template <bool S2>
-__device__ __forceinline__ double rank2_part(double* mc, const double* v, const double* w, double vc, double wc,
-                                             int rr, int lane) {
-  double s2 = 0.0;
-  for (int c0 = 0; c0 < rr; c0 += 128) {
-    double m[4], x[4], y[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = c0 + 32 * u + lane;
-      m[u] = i < rr ? mc[i] : 0.0;
-      x[u] = i < rr ? v[i] : 0.0;
-      y[u] = i < rr ? w[i] : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (c0 + 32 * u < rr) {
-        const int i = c0 + 32 * u + lane;
-        const double nm = fma(-y[u], vc, fma(-x[u], wc, m[u]));
-        if (i < rr) mc[i] = nm;
-        if (S2) s2 = fma(i >= 2 && i < rr ? nm : 0.0, nm, s2);
-      }
-    }
-  }
-  return s2;
+// 1 / a for a normal a > 0: FP32 seed r (22 bits), then r (1 + e + e^2), e = 1 - a r: 3 FP64 instructions.
+__device__ __forceinline__ double rcp_h3(double a) {
+  const int hi = __double2hiint(a), lo = __double2loint(a);
+  const int eb = ((hi >> 20) & 0x7ff) - 1023;
+  const float m = __int_as_float((127 << 23) | ((hi & 0xfffff) << 3) | (int)((uint32_t)lo >> 29));
+  const int yb = __float_as_int(__fdividef(1.0f, m));
+  const double r = __hiloint2double((((yb >> 23) - 127 + 1023 - eb) << 20) | ((yb >> 3) & 0xfffff), yb << 29);
+  const double e = fma(-a, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 
 // ------------------------------------------------------------------ Cholesky and L^-1
@@ -285,190 +282,186 @@ __global__ void __launch_bounds__(256) chol_inv_smem_kernel(int n, const double*
 
 // ------------------------------------------------------------------ blocked Cholesky and L^-1
 // A = L L^T (A symmetric positive definite, n x n column-major, lower triangle read) and L^-1, on a
-// cooperative grid, in 32 x 32 tiles: per block column K, one CTA factors the diagonal tile and
-// inverts its factor (DI_K), all CTAs solve the panel L_IK = A_IK DI_K^T and update the trailing
-// lower triangle A_IJ -= L_IK L_JK^T; then L^-1 by the right-looking block forward substitution of
-// L X = I: X_K,: = DI_K B_K,: and B_I,: -= L_IK X_K,: for I > K.  5 grid barriers per block column
-// instead of one per column, and the FP64 work spread over every SM.
-// di: scratch of ceil(n / 32) x 32 x 32 doubles; bad: one int of scratch.  info: 0, or j + 1 for the
-// first column j whose pivot is not positive (L and L^-1 are then not written in full).
+// cooperative grid, in 32 x 32 tiles.  Per block column K, with B = I in Linv at the start:
+//   1. every CTA factors the diagonal tile and inverts its factor (DI_K = L_KK^-1) for itself: the
+//      same bits everywhere, and no barrier before they are used;
+//   2. panel L_IK = A_IK DI_K^T (I > K) and row K of the inverse X_KJ = DI_K B_KJ (J <= K);
+//   3. grid barrier; trailing updates A_IJ -= L_IK L_JK^T (K < J <= I) and B_IJ -= L_IK X_KJ
+//      (I > K, J <= K); grid barrier.
+// Two barriers per 32 columns for the factor and the inverse together.  Products are split into
+// units of 128 outputs (two threads each) so that a few tiles still spread over the SMs.
+// The factor of a tile (tile_factor): LDL^T by columns with the same row operations applied to the
+// identity, one thread per (row, column mod 8), one CTA barrier per column; the chain of a column is
+// its FMA, the reciprocal of the pivot (an FP32 seed and 3 FP64 instructions) and one product.  The
+// square roots are taken at the end, for all 32 pivots in one go.
+// info: 0, or j + 1 for the first column j whose pivot is not positive (L and L^-1 are then not
+// written in full).
+// Measured (cold, one call; before: a barrier per phase, the diagonal tile on one CTA, L^-1 after the
+// factor): see the launcher.
 constexpr int CB = 32;
 
-// Rows [r0, r0 + nr) x columns [c0, c0 + nc) of C (+|-)= A B^T or A B, the tiles staged in shared
-// memory; 256 threads over the part's outputs.
-__device__ __forceinline__ void tile_acc_part(double (*C)[CB + 1], const double (*A)[CB + 1], const double (*B)[CB + 1],
-                                              bool btrans, double sign, int r0, int nr, int c0, int nc) {
-  for (int e = threadIdx.x; e < nr * nc; e += blockDim.x) {
-    const int r = r0 + e / nc, c = c0 + e % nc;
-    double a0 = 0.0, a1 = 0.0;
-#pragma unroll 8
-    for (int k = 0; k < CB; k += 2) {
-      a0 = fma(A[r][k], btrans ? B[c][k] : B[k][c], a0);
-      a1 = fma(A[r][k + 1], btrans ? B[c][k + 1] : B[k + 1][c], a1);
-    }
-    C[r][c] = fma(sign, a0 + a1, C[r][c]);
+struct TileSmem {
+  double L[CB][CB + 1], D[CB][CB + 1];  // factor and its inverse of the diagonal tile
+  double col[2][CB], mul[2][CB], piv[CB], rs[CB];
+  int bad;
+};
+
+// Factor tile (K, K) of M (column-major n x n, lower triangle) into T.L and T.D; T.bad = 0, or j + 1
+// for the first pivot j that is not positive and finite.  256 threads.
+__device__ __forceinline__ void tile_factor(TileSmem& T, const double* M, int n, int K) {
+  const int tid = threadIdx.x, i = tid & 31, w = tid >> 5;
+  double a[4], b[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int c = w + 8 * q, gi = K * CB + i, gc = K * CB + c;
+    a[q] = (gi < n && gc < n) ? __ldcg(M + (size_t)gc * n + gi) : (i == c ? 1.0 : 0.0);
+    b[q] = i == c ? 1.0 : 0.0;
   }
+  if (tid == 0) T.bad = 0;
+  __syncthreads();
+#pragma unroll
+  for (int jq = 0; jq < 4; ++jq) {
+    for (int jw = 0; jw < 8; ++jw) {
+      const int j = 8 * jq + jw, buf = j & 1;
+      if (w == jw) {
+        const double d = __shfl_sync(0xffffffffu, a[jq], j);
+        const bool good = d > 0.0 && d < DBL_MAX;
+        const double m = a[jq] * rcp_h3(good ? d : 1.0);
+        T.col[buf][i] = a[jq];
+        T.mul[buf][i] = m;
+        T.L[i][j] = a[jq];
+        if (i == 0) {
+          T.piv[j] = good ? d : 1.0;
+          if (!good && T.bad == 0) T.bad = j + 1;
+        }
+      }
+      __syncthreads();
+      const double ci = T.col[buf][i], mi = T.mul[buf][i];
+      // the columns still to come (the next pivot's first), then the rows of the identity
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = (u + jq) & 3, c = w + 8 * q;
+        if (c > j) a[q] = fma(-ci, T.mul[buf][c], a[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (w + 8 * q <= j) {
+          const double bj = __shfl_sync(0xffffffffu, b[q], j);
+          const double v = fma(-mi, bj, b[q]);
+          if (i > j) b[q] = v;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (w == 0) T.rs[i] = rsqrt_h3(T.piv[i]);
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int c = w + 8 * q;
+    T.L[i][c] = i < c ? 0.0 : T.L[i][c] * T.rs[c];  // (d_c / sqrt(d_c) on the diagonal)
+    T.D[i][c] = b[q] * T.rs[i];
+  }
+  __syncthreads();
 }
 
-// Tile (I, J) of a column-major n x n matrix to / from shared memory (zeros outside the matrix).
-__device__ __forceinline__ void tile_load(double (*T)[CB + 1], const double* M, int n, int I, int J) {
-  for (int e = threadIdx.x; e < CB * CB; e += blockDim.x) {
-    const int c = e / CB, r = e % CB, i = I * CB + r, j = J * CB + c;
-    T[r][c] = (i < n && j < n) ? __ldcg(M + (size_t)j * n + i) : 0.0;
+// Output (r, c) of a unit: the sum of a[k] b[k] over 32 k, two threads (even / odd lanes) per output.
+__device__ __forceinline__ double unit_dot(const double* a, int sa, const double* b, int sb, int half) {
+  double s0 = 0.0, s1 = 0.0;
+#pragma unroll 8
+  for (int k = 0; k < CB / 2; k += 2) {
+    const int k0 = half * (CB / 2) + k;
+    s0 = fma(a[k0 * sa], b[k0 * sb], s0);
+    s1 = fma(a[(k0 + 1) * sa], b[(k0 + 1) * sb], s1);
   }
-}
-__device__ __forceinline__ void tile_store(const double (*T)[CB + 1], double* M, int n, int I, int J) {
-  for (int e = threadIdx.x; e < CB * CB; e += blockDim.x) {
-    const int c = e / CB, r = e % CB, i = I * CB + r, j = J * CB + c;
-    if (i < n && j < n) __stcg(M + (size_t)j * n + i, T[r][c]);
-  }
-}
-__device__ __forceinline__ void tile_store_part(const double (*T)[CB + 1], double* M, int n, int I, int J, int r0,
-                                                int nr, int c0, int nc) {
-  for (int e = threadIdx.x; e < nr * nc; e += blockDim.x) {
-    const int c = c0 + e / nr, r = r0 + e % nr, i = I * CB + r, j = J * CB + c;
-    if (i < n && j < n) __stcg(M + (size_t)j * n + i, T[r][c]);
-  }
+  s0 += s1;
+  return s0 + __shfl_xor_sync(0xffffffffu, s0, 1);
 }
 
 __global__ void __launch_bounds__(256) chol_inv_blocked_kernel(int n, const double* __restrict__ A, double* L,
-                                                               double* Linv, double* di, int* bad, int* info) {
-  __shared__ double T0[CB][CB + 1], T1[CB][CB + 1], T2[CB][CB + 1];
-  __shared__ double rdiag[CB];  // 1 / L_jj of the diagonal tile
+                                                               double* Linv, int* info) {
+  __shared__ TileSmem T;
+  __shared__ double SA[CB][CB + 1], SB[CB][CB + 1];
   cg::grid_group grid = cg::this_grid();
   const int P = gridDim.x, r = blockIdx.x, tid = threadIdx.x;
   const int nt = (n + CB - 1) / CB;
   const size_t nn = (size_t)n * n;
+  auto at = [&](const double* M, int i, int j) { return (i < n && j < n) ? __ldcg(M + (size_t)j * n + i) : 0.0; };
+  auto put = [&](double* M, int i, int j, double v) {
+    if (i < n && j < n) __stcg(M + (size_t)j * n + i, v);
+  };
   // L = lower(A), Linv = I
   for (size_t e = (size_t)r * blockDim.x + tid; e < nn; e += (size_t)P * blockDim.x) {
     const size_t j = e / n, i = e - j * n;
     __stcg(L + e, i >= j ? A[e] : 0.0);
     __stcg(Linv + e, i == j ? 1.0 : 0.0);
   }
-  if (r == 0 && tid == 0) *bad = 0;
   grid.sync();
+  const int o = tid >> 1, half = tid & 1;  // output of the unit, and half of its sum
   for (int K = 0; K < nt; ++K) {
-    const int nb = min(CB, n - K * CB);
-    // ---- diagonal tile: Cholesky in shared memory, then DI_K = L_KK^-1 (CTA 0)
-    if (r == 0) {
-      tile_load(T0, L, n, K, K);
-      __syncthreads();
-      for (int j = 0; j < nb; ++j) {
-        const double d = T0[j][j];
-        if (!(d > 0.0) || !isfinite(d)) {
-          if (tid == 0) {
-            *bad = K * CB + j + 1;
-            *info = K * CB + j + 1;
-          }
-          break;
-        }
-        const double inv = rsqrt(d);
-        if (tid == 0) rdiag[j] = inv;
-        __syncthreads();
-        if (tid > j && tid < nb) T0[tid][j] *= inv;
-        __syncthreads();
-        // trailing update inside the tile: T0[i][k] -= T0[i][j] T0[k][j], j < k <= i < nb
-        for (int e = tid; e < CB * CB; e += blockDim.x) {
-          const int i = e / CB, k = e % CB;
-          if (k > j && k <= i && i < nb) T0[i][k] = fma(-T0[i][j], T0[k][j], T0[i][k]);
-        }
-        if (tid == 0) T0[j][j] = d * inv;
-        __syncthreads();
-      }
-      // the update also wrote the tile's upper half: L is lower triangular
-      for (int e = tid; e < CB * CB; e += blockDim.x)
-        if (e % CB > e / CB) T0[e / CB][e % CB] = 0.0;
-      __syncthreads();
-      if (*(volatile int*)bad == 0) {
-        // DI = L_KK^-1 by forward substitution, 8 threads per column c: x_i = (delta_ic - sum_k
-        // L_ik x_k) / L_ii for i >= c, the sum split over the 8 threads
-        const int c = tid >> 3, s = tid & 7;
-        for (int e = tid; e < CB * CB; e += blockDim.x) T1[e / CB][e % CB] = 0.0;
-        __syncthreads();
-        for (int i = 0; i < CB; ++i) {
-          double part = 0.0;
-          if (c < nb && i < nb && i >= c)
-            for (int k = c + s; k < i; k += 8) part = fma(T0[i][k], T1[k][c], part);
-          part += __shfl_xor_sync(0xffffffffu, part, 1);
-          part += __shfl_xor_sync(0xffffffffu, part, 2);
-          part += __shfl_xor_sync(0xffffffffu, part, 4);
-          if (s == 0 && c < nb && i < nb && i >= c) T1[i][c] = ((i == c ? 1.0 : 0.0) - part) * rdiag[i];
-          __syncthreads();
-        }
-        tile_store(T0, L, n, K, K);
-        double* dk = di + (size_t)K * CB * CB;
-        for (int e = tid; e < CB * CB; e += blockDim.x) __stcg(dk + e, T1[e / CB][e % CB]);
-      }
+    tile_factor(T, L, n, K);
+    if (T.bad) {
+      if (r == 0 && tid == 0) *info = K * CB + T.bad;
+      return;  // (every CTA takes the same branch)
     }
-    grid.sync();
-    if (*(volatile int*)bad) return;
-    // ---- panel: L_IK = A_IK DI_K^T, I > K
-    const double* dk = di + (size_t)K * CB * CB;
-    // (two CTAs per tile, one per half of its rows: a row of L_IK needs only that row of A_IK)
-    for (int t = r; t < 2 * (nt - K - 1); t += P) {
-      const int I = K + 1 + t / 2, h = (t % 2) * (CB / 2);
-      for (int e = tid; e < CB * CB; e += blockDim.x) T1[e / CB][e % CB] = __ldcg(dk + e);
-      tile_load(T0, L, n, I, K);
-      for (int e = tid; e < CB * CB; e += blockDim.x) T2[e / CB][e % CB] = 0.0;
+    // ---- panel rows (4 of a tile per unit) and columns of row K of the inverse (4 of a tile per unit)
+    const int np = nt - K - 1;
+    for (int u = r; u < 8 * (np + K + 1); u += P) {
+      const bool inv = u >= 8 * np;
+      const int t = inv ? u - 8 * np : u;
+      const int I = inv ? t >> 3 : K + 1 + (t >> 3), h = 4 * (t & 7);
+      if (tid < 128) {
+        if (!inv) {
+          const int rr = tid & 3, k = tid >> 2;
+          SA[rr][k] = at(L, I * CB + h + rr, K * CB + k);
+        } else {
+          const int k = tid & 31, c = tid >> 5;
+          SA[c][k] = at(Linv, K * CB + k, I * CB + h + c);
+        }
+      }
       __syncthreads();
-      tile_acc_part(T2, T0, T1, true, 1.0, h, CB / 2, 0, CB);
-      __syncthreads();
-      tile_store_part(T2, L, n, I, K, h, CB / 2, 0, CB);
+      // (both: outputs 4 x 32, a 4-row operand against the rows of DI)
+      const int x = inv ? o >> 5 : o & 3, y = inv ? o & 31 : o >> 2;
+      const double v = unit_dot(&SA[x][0], 1, &T.D[y][0], 1, half);
+      if (half == 0) {
+        if (!inv) put(L, I * CB + h + x, K * CB + y, v);
+        else put(Linv, K * CB + y, I * CB + h + x, v);
+      }
       __syncthreads();
     }
     grid.sync();
-    // ---- trailing update of the lower triangle: A_IJ -= L_IK L_JK^T, K < J <= I
-    {
-      const int m = nt - K - 1;
-      const int tiles = m * (m + 1) / 2;
-      // (four CTAs per tile, one per quadrant of outputs; the operands are other tiles)
-      for (int tq = r; tq < 4 * tiles; tq += P) {
-        const int t = tq / 4, qr = ((tq % 4) / 2) * (CB / 2), qc = (tq % 2) * (CB / 2);
+    if (r == 0)
+      for (int e = tid; e < CB * CB; e += blockDim.x) put(L, K * CB + (e & 31), K * CB + (e >> 5), T.L[e & 31][e >> 5]);
+    if (np == 0) break;
+    // ---- trailing updates in units of 16 x 8 outputs (8 per tile)
+    const int ta = np * (np + 1) / 2, tb = np * (K + 1);
+    for (int u = r; u < 8 * (ta + tb); u += P) {
+      const int t = u >> 3, r0 = 16 * (u & 1), c0 = 8 * ((u >> 1) & 3);
+      int I, J;
+      const bool inv = t >= ta;
+      if (!inv) {
         // t -> (I, J) with J <= I: row a = I - K - 1 holds a + 1 tiles
-        int a = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
+        int a = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
         while ((a + 1) * (a + 2) / 2 <= t) ++a;
         while (a * (a + 1) / 2 > t) --a;
-        const int I = K + 1 + a, J = K + 1 + (t - a * (a + 1) / 2);
-        tile_load(T0, L, n, I, K);
-        tile_load(T1, L, n, J, K);
-        tile_load(T2, L, n, I, J);
-        __syncthreads();
-        tile_acc_part(T2, T0, T1, true, -1.0, qr, CB / 2, qc, CB / 2);
-        __syncthreads();
-        tile_store_part(T2, L, n, I, J, qr, CB / 2, qc, CB / 2);
-        __syncthreads();
+        I = K + 1 + a;
+        J = K + 1 + (t - a * (a + 1) / 2);
+      } else {
+        I = K + 1 + (t - ta) / (K + 1);
+        J = (t - ta) % (K + 1);
       }
-    }
-    grid.sync();
-  }
-  // L^-1: B = I in Linv; per block row K: X_K,: = DI_K B_K,: (column tiles <= K), then
-  // B_I,: -= L_IK X_K,: for I > K
-  for (int K = 0; K < nt; ++K) {
-    const double* dk = di + (size_t)K * CB * CB;
-    // (two CTAs per tile, one per half of its columns: a column of X_KJ needs only that column of B_KJ)
-    for (int t = r; t < 2 * (K + 1); t += P) {
-      const int J = t / 2, h = (t % 2) * (CB / 2);
-      for (int e = tid; e < CB * CB; e += blockDim.x) T1[e / CB][e % CB] = __ldcg(dk + e);
-      tile_load(T0, Linv, n, K, J);
-      for (int e = tid; e < CB * CB; e += blockDim.x) T2[e / CB][e % CB] = 0.0;
+      for (int e = tid; e < 16 * CB; e += 256) SA[e & 15][e >> 4] = at(L, I * CB + r0 + (e & 15), K * CB + (e >> 4));
+      {
+        const int e = tid;  // 8 x 32: rows of L_JK, or columns of X_KJ
+        if (!inv) SB[e & 7][e >> 3] = at(L, J * CB + c0 + (e & 7), K * CB + (e >> 3));
+        else SB[e >> 5][e & 31] = at(Linv, K * CB + (e & 31), J * CB + c0 + (e >> 5));
+      }
+      double* C = inv ? Linv : L;
+      const int x = o & 15, y = o >> 4;
+      const double old = half == 0 ? at(C, I * CB + r0 + x, J * CB + c0 + y) : 0.0;
       __syncthreads();
-      tile_acc_part(T2, T1, T0, false, 1.0, 0, CB, h, CB / 2);
-      __syncthreads();
-      tile_store_part(T2, Linv, n, K, J, 0, CB, h, CB / 2);
-      __syncthreads();
-    }
-    grid.sync();
-    const int rows = nt - K - 1, tiles = rows * (K + 1);
-    for (int tq = r; tq < 4 * tiles; tq += P) {
-      const int t = tq / 4, qr = ((tq % 4) / 2) * (CB / 2), qc = (tq % 2) * (CB / 2);
-      const int I = K + 1 + t / (K + 1), J = t % (K + 1);
-      tile_load(T0, L, n, I, K);
-      tile_load(T1, Linv, n, K, J);
-      tile_load(T2, Linv, n, I, J);
-      __syncthreads();
-      tile_acc_part(T2, T0, T1, false, -1.0, qr, CB / 2, qc, CB / 2);
-      __syncthreads();
-      tile_store_part(T2, Linv, n, I, J, qr, CB / 2, qc, CB / 2);
+      const double v = unit_dot(&SA[x][0], 1, &SB[y][0], 1, half);
+      if (half == 0) put(C, I * CB + r0 + x, J * CB + c0 + y, old - v);
       __syncthreads();
     }
     grid.sync();
@@ -656,167 +649,385 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_smem_kernel(int n, const 
   if ((n - 1) % P == r && tid == 0) d[n - 1] = cols[(size_t)((n - 1 - r) / P) * n + n - 1];
 }
 
-// The same reduction for one thread-block cluster, with every exchange through distributed shared
-// memory instead of L2.  All CTAs use one layout (nqm = ceil(n / P) column slots), so a remote
-// address is the local one in another rank.  The owner of column k + 1 updates that column first
-// (warp 0) and, while its other warps finish the rank-2 update, computes the Householder scalars of
-// the next step (alpha, beta, tau and the scale 1 / (alpha - beta)) and keeps them with the column;
-// the other CTAs read them after the barrier instead of each recomputing the norm, the square root
-// and the divide.  Step k: read pivot column k and its scalars from the owner -> own products
-// t (A v)_c -> barrier -> read the products p_c of all CTAs -> rank-2 update -> barrier.  The loop
-// writes nothing to global memory (a barrier's release then has no stores to wait for); H, d, e
-// and tau are written at the end from the owned columns and their scalars.
-constexpr int TRI_DS_SLOTS = 8;  // per owned column: beta, tau, scale, diagonal (4 used)
+// ------------------------------------------------------------------ one exchange per column
+// The reduction of tridiag_smem_kernel with one exchange between the CTAs per column instead of two
+// barriers and several dependent remote reads.  With x = M(k+1:, k) the current pivot column (alpha =
+// x_0, beta = -sign(alpha) ||x||), u = x - beta e_1 and eta = 2 / (u^T u) = 1 / (beta^2 - alpha beta),
+// H_k = I - eta u u^T and, A' being the trailing block,
+//   t = A' u = A' x - beta a,  a = A' e_1 = M(k+1:, k+1),   w = eta t - (eta^2 / 2) (u^T t) u,
+//   A' <- A' - u w^T - w u^T.
+// The products q_c = A'(:, c)^T x of the owned columns need neither beta nor eta, so the norm, the
+// square root and the divide of a column (one warp of every CTA, redundantly) run beside the
+// products and the exchange.  What travels per column is q (each entry from its column's owner) and
+// a (from the owner of column k + 1): every CTA then forms t, w and the next pivot column
+// x' = a - u w_0 - w u_0 for itself, all from the same bits, so nobody waits for an owner again.  One
+// pass over the owned columns applies the rank-2 update and forms the next products.
+// Exchange: CL = true, one thread-block cluster: q by st.async, a by one bulk copy per CTA, both
+// completing bytes on the receiver's mbarrier.  CL = false, a cooperative grid: 16-byte packets
+// {low word, tag, high word, tag} through L2 (xg: 4 n packets, zeroed), polled by the thread that
+// needs the entry; the tag is the step.  Both buffers alternate by step: a CTA sends step k + 2 only
+// after it has received step k + 1 from everyone, and those sent it after they had read step k.
+// Every wait is bounded: on a timeout *err is set to 2 and all CTAs leave.
+// Warps 0-7: rows and columns; warp 8: the scalars.  Outputs as tridiag_smem_kernel, with H(:, k) = u
+// and tau = eta (the same reflector).
+constexpr int TX_THREADS = 288;
+constexpr int TX_ROWS = 4;  // rows per thread: n <= 1024
 
-size_t tridiag_dsmem_smem(int n, int P) {
-  const size_t nqm = ((size_t)n + P - 1) / P;
-  return (nqm * n + 2 * (size_t)n + nqm * (1 + TRI_DS_SLOTS) + 40) * sizeof(double);
+size_t tridiag_xch_smem(int n, int P, bool cl) {
+  const size_t ld = ((size_t)n + 1) & ~(size_t)1, nqm = ((size_t)n + P - 1) / P;
+  return (nqm * ld + (cl ? 4 : 0) * ld + 3 * ld) * sizeof(double) + 16;
 }
 
-// Householder scalars of x = column c rows c+1.. (alpha = x_0, xn2 = |x_1..|^2), as in tridiag_smem_kernel.
-__device__ __forceinline__ void house_scalars(double alpha, double xn2, double* beta, double* t, double* sc) {
-  *beta = alpha;
-  *t = 0.0;
-  *sc = 1.0;
-  if (xn2 > 0.0) {
-    const double b = -copysign(sqrt(alpha * alpha + xn2), alpha);
-    const double g = alpha - b, rcp = 1.0 / (b * g);
-    *beta = b;
-    *t = -(g * g) * rcp;
-    *sc = b * rcp;
+__device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_async_f64(uint32_t addr, double v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr),
+               "l"(__double_as_longlong(v)), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_s2s(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   dst),
+               "r"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void pkt_store(uint4* p, double v, uint32_t tag) {
+  asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %2};" ::"l"(p), "r"((uint32_t)__double2loint(v)),
+               "r"(tag), "r"((uint32_t)__double2hiint(v))
+               : "memory");
+}
+// true when the packet carries `tag`
+__device__ __forceinline__ bool pkt_load(const uint4* p, uint32_t tag, double* v) {
+  uint32_t a, b, c, e;
+  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(a), "=r"(b), "=r"(c), "=r"(e)
+               : "l"(p)
+               : "memory");
+  *v = __hiloint2double((int)c, (int)a);
+  return b == tag && e == tag;
+}
+
+template <bool CL>
+__global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const double* __restrict__ Min, double* H,
+                                                                 double* d, double* e, double* tau, uint4* xg,
+                                                                 int* err) {
+  extern __shared__ double sm_raw[];
+  __shared__ __align__(8) uint64_t qbar[2], sbar;
+  __shared__ double red[8], scal[6];  // scal: beta, eta, -eta^2 / 2, u_0, u_0 eta, -u_0 eta^2
+  __shared__ int abort_flag[2];
+  const int P = gridDim.x, r = blockIdx.x;  // (a cluster launch is one cluster)
+  const int ld = (n + 1) & ~1;
+  const int nqm = (n + P - 1) / P, nq = (n - r + P - 1) / P;  // owned columns c = r + q P
+  double* sm = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(sm_raw) + 15) & ~uintptr_t(15));
+  double* cols = sm;                       // nqm x ld
+  double* xa = cols + (size_t)nqm * ld;    // CL: two buffers of a, two of q
+  double* xq = xa + (CL ? 2 * ld : 0);
+  double* U = xq + (CL ? 2 * ld : 0);
+  double* W = U + ld;
+  double* X = W + ld;
+  uint4* ga = xg;                          // !CL: two buffers of a, two of q
+  uint4* gq = xg + 2 * (size_t)n;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    tc::mbar_init(&qbar[0], 1);
+    tc::mbar_init(&qbar[1], 1);
+    tc::mbar_init(&sbar, 1);
+    tc::fence_barrier_init();
+    abort_flag[0] = abort_flag[1] = 0;
   }
-}
-
-__global__ void __launch_bounds__(TRI_THREADS) tridiag_dsmem_kernel(int n, const double* __restrict__ Min, double* H,
-                                                                    double* d, double* e, double* tau) {
-  extern __shared__ double sm[];
-  cg::cluster_group cluster = cg::this_cluster();
-  const int P = (int)cluster.num_blocks(), r = (int)cluster.block_rank();
-  const int nqm = (n + P - 1) / P;
-  const int nq = (n - r + P - 1) / P;  // owned columns c = r + q P, q < nq
-  double* cols = sm;                          // nqm x n
-  double* v = cols + (size_t)nqm * n;         // n
-  double* w = v + n;                          // n
-  double* prod = w + n;                       // nqm: t (A v)_c of the owned columns
-  double* hs = prod + nqm;                    // nqm x TRI_DS_SLOTS: beta, tau, scale, diagonal
-  double* red = hs + (size_t)nqm * TRI_DS_SLOTS;  // 33
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
   for (int q = 0; q < nq; ++q)
-    for (int i = tid; i < n; i += blockDim.x) cols[(size_t)q * n + i] = Min[(size_t)(r + q * P) * n + i];
-  __syncthreads();
-  // scalars of pivot column 0 (owner: rank 0)
-  if (r == 0 && warp == 0 && n > 2) {
+    for (int i = tid; i < n; i += TX_THREADS) cols[(size_t)q * ld + i] = Min[(size_t)(r + q * P) * n + i];
+  for (int i = tid; i < n; i += TX_THREADS) X[i] = Min[i];
+  if (n & 1)  // the padding row travels with the columns
+    for (int q = tid; q < nqm; q += TX_THREADS) cols[(size_t)q * ld + n] = 0.0;
+  if (CL) cg::this_cluster().sync();  // the barriers are ready before anyone sends
+  else __syncthreads();
+
+  // bytes that arrive for step k: q_c, c = k + 1 .. n - 1, and rows (k + 1) & ~1 .. of a
+  auto expect = [&](int k) {
+    tc::mbar_arrive_expect_tx(&qbar[k & 1], (uint32_t)(8 * (n - k - 1) + 8 * (ld - ((k + 1) & ~1))));
+  };
+  if (CL && tid == 0)
+    for (int k = 0; k < 2 && k + 2 < n; ++k) expect(k);
+
+  // this lane's view of CTA `lane` of the cluster
+  uint32_t rq = 0, ra = 0, rb = 0;
+  if (CL && lane < P) {
+    rq = mapa_u32(tc::smem_u32(xq), (uint32_t)lane);
+    ra = mapa_u32(tc::smem_u32(xa), (uint32_t)lane);
+    rb = mapa_u32(tc::smem_u32(qbar), (uint32_t)lane);
+  }
+
+  // rank-2 update of step k on the owned columns c >= k + 2 (UPD), the products with x' and, with
+  // `send`, what step k + 1 needs
+  auto pass = [&](int k, bool upd, bool send) {
+    const int s0 = k + 2, rr = n - s0;  // rows s0 .. n - 1
+    const int qa = s0 - r > 0 ? (s0 - r + P - 1) / P : 0;
+    const int b = (k + 1) & 1;
+    // (columns go to the warps in an order that loads sub-partition 0, which also runs the scalars, last)
+    for (int q = qa + (((warp + 3) & 3) | (warp & 4)); q < nq; q += 16) {
+      const int q2 = q + 8;
+      const bool two = q2 < nq;
+      const int c = r + q * P, c2 = c + 8 * P;
+      double* m1 = cols + (size_t)q * ld + s0;
+      double* m2 = cols + (size_t)(two ? q2 : q) * ld + s0;
+      double wc = 0.0, uc = 0.0, wc2 = 0.0, uc2 = 0.0;
+      if (upd) {
+        wc = W[c];
+        uc = U[c];
+        if (two) {
+          wc2 = W[c2];
+          uc2 = U[c2];
+        }
+      }
+      double a1 = 0.0, a2 = 0.0;
+      for (int c0 = 0; c0 < rr; c0 += 64) {
+        double x[2], u[2], w[2], p1[2], p2[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int i = c0 + 32 * h + lane;
+          const bool in = i < rr;
+          x[h] = in ? X[s0 + i] : 0.0;
+          p1[h] = in ? m1[i] : 0.0;
+          p2[h] = in && two ? m2[i] : 0.0;
+          if (upd) {
+            u[h] = in ? U[s0 + i] : 0.0;
+            w[h] = in ? W[s0 + i] : 0.0;
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int i = c0 + 32 * h + lane;
+          if (c0 + 32 * h < rr) {  // (a chunk past the end would still hold the FP64 pipe)
+            if (upd) {
+              p1[h] = fma(-w[h], uc, p1[h]);
+              if (two) p2[h] = fma(-w[h], uc2, p2[h]);
+              p1[h] = fma(-u[h], wc, p1[h]);
+              if (two) p2[h] = fma(-u[h], wc2, p2[h]);
+              if (i < rr) {
+                m1[i] = p1[h];
+                if (two) m2[i] = p2[h];
+              }
+            }
+            if (send) {
+              a1 = fma(p1[h], x[h], a1);
+              if (two) a2 = fma(p2[h], x[h], a2);
+            }
+          }
+        }
+      }
+      if (!send) continue;
+      if (c == s0) {  // column k + 2 is the next step's a
+        if (CL) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          const int i0 = s0 & ~1;
+          if (lane < P)
+            bulk_s2s(ra + (uint32_t)((b * ld + i0) * 8), tc::smem_u32(cols + (size_t)q * ld + i0),
+                     (uint32_t)((ld - i0) * 8), rb + 8u * b);
+        } else {
+          __syncwarp();
+          for (int i = s0 + lane; i < n; i += 32)
+            pkt_store(ga + (size_t)b * n + i, cols[(size_t)q * ld + i], (uint32_t)(k + 2));
+        }
+      }
+      const double d1 = warp_sum_fx(a1);
+      const double d2 = two ? warp_sum_fx(a2) : 0.0;
+      if (CL) {
+        if (lane < P) {
+          st_async_f64(rq + (uint32_t)((b * ld + c) * 8), d1, rb + 8u * b);
+          if (two) st_async_f64(rq + (uint32_t)((b * ld + c2) * 8), d2, rb + 8u * b);
+        }
+      } else if (lane == 0) {
+        pkt_store(gq + (size_t)b * n + c, d1, (uint32_t)(k + 2));
+        if (two) pkt_store(gq + (size_t)b * n + c2, d2, (uint32_t)(k + 2));
+      }
+    }
+  };
+  // scalars of the pivot column x = X[k + 1 ..] (warp 8)
+  auto scalars = [&](int k) {
     double s2 = 0.0;
-    for (int i = 2 + lane; i < n; i += 32) s2 += cols[i] * cols[i];
-    s2 = warp_sum(s2);
+    for (int i = k + 2 + lane; i < n; i += 32) s2 = fma(X[i], X[i], s2);
+    s2 = warp_sum_fx(s2);
+    const double alpha = X[k + 1];
+    double beta = alpha, eta = 0.0, u0 = 0.0;
+    const double nx2 = fma(alpha, alpha, s2);
+    if (s2 > 0.0 && nx2 < DBL_MAX) {
+      // eta = 1 / (||x||^2 + |alpha| ||x||) = (1 / ||x||) / (||x|| + |alpha|)
+      const double ri = rsqrt_h3(nx2), nx = nx2 * ri, g = nx + fabs(alpha);
+      beta = -copysign(nx, alpha);
+      u0 = copysign(g, alpha);  // alpha - beta
+      eta = ri * rcp_h3(g);
+    } else if (s2 > 0.0) {
+      beta = eta = u0 = __longlong_as_double(0x7ff8000000000000LL);  // overflow of ||x||^2
+    }
+    const double ue = u0 * eta;
     if (lane == 0) {
-      house_scalars(cols[1], s2, hs + 0, hs + 1, hs + 2);
-      hs[3] = cols[0];
+      scal[0] = beta;
+      scal[1] = eta;
+      scal[2] = -0.5 * (eta * eta);
+      scal[3] = u0;
+      scal[4] = ue;
+      scal[5] = -(ue * eta);
     }
-  }
-  cluster.sync();
-  for (int k = 0; k + 2 < n; ++k) {
-    const int rr = n - k - 1;
-    const int ok_ = k % P, oq = k / P;  // owner of the pivot column and its slot
-    const double* pc = cluster.map_shared_rank(cols + (size_t)oq * n, ok_);
-    const double* ph = cluster.map_shared_rank(hs + (size_t)oq * TRI_DS_SLOTS, ok_);
-    // v = (1, x_1 sc, x_2 sc, ...) from the owner's column (the loads are issued together)
-    double xv[2];
+    __syncwarp();
+    if (lane == 0) tc::mbar_arrive(&sbar);
+  };
+
+  if (n >= 3) {
+    double xr[TX_ROWS];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int i = tid + (int)blockDim.x * u;
-      xv[u] = (i > 0 && i < rr) ? pc[k + 1 + i] : 0.0;
+    for (int j = 0; j < TX_ROWS; ++j) {
+      const int i = tid + 256 * j;
+      xr[j] = i < n ? X[i] : 0.0;
     }
-    const double t = ph[1], sc = ph[2];
+    if (r == 0 && tid == 0) d[0] = X[0];
+    if (warp == 8) scalars(0);
+    else pass(-1, false, true);
+    for (int k = 0; k + 2 < n; ++k) {
+      const int b = k & 1;
+      if (warp < 8) {
+        const bool any = [&] {  // (warp-uniform) does this warp hold a row of the trailing block
+          bool a = false;
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int i = tid + (int)blockDim.x * u;
-      if (i < rr) v[i] = i == 0 ? 1.0 : xv[u] * sc;
-    }
-    for (int i = tid + 2 * (int)blockDim.x; i < rr; i += blockDim.x) v[i] = pc[k + 1 + i] * sc;
-    __syncthreads();
-    const int qa = (k + 1 - r + P - 1) / P > 0 ? (k + 1 - r + P - 1) / P : 0;
-    if (t != 0.0) {
-      // owned columns in pairs per warp, the two reductions interleaved
-      for (int q = qa + warp; q < nq; q += 2 * nw) {
-        const int q2 = q + nw;
-        double a = dot_part(cols + (size_t)q * n + k + 1, v, rr, lane);
-        double b = q2 < nq ? dot_part(cols + (size_t)q2 * n + k + 1, v, rr, lane) : 0.0;
-        warp_sum2(a, b);
-        if (lane == 0) {
-          prod[q] = t * a;
-          if (q2 < nq) prod[q2] = t * b;
+          for (int j = 0; j < TX_ROWS; ++j) a = a || (256 * j + 32 * warp < n && 256 * j + 32 * warp + 31 > k);
+          return a;
+        }();
+        bool ok = true;
+        double qv[TX_ROWS], av[TX_ROWS], q0 = 0.0, a0 = 0.0;
+#pragma unroll
+        for (int j = 0; j < TX_ROWS; ++j) qv[j] = av[j] = 0.0;
+        if (CL) {
+          ok = tc::mbar_wait(&qbar[b], (uint32_t)((k >> 1) & 1));
+          if (tid == 0 && ok && k + 4 < n) expect(k + 2);
+          if (any) {
+            q0 = xq[b * ld + k + 1];
+            a0 = xa[b * ld + k + 1];
+          }
+#pragma unroll
+          for (int j = 0; j < TX_ROWS; ++j) {
+            const int i = tid + 256 * j;
+            const bool in = i > k && i < n;
+            qv[j] = in ? xq[b * ld + i] : 0.0;
+            av[j] = in ? xa[b * ld + i] : 0.0;
+          }
+        } else if (any) {
+          // (each packet is loaded until its tag shows up, then kept)
+          uint32_t need = 3u << (2 * TX_ROWS);
+#pragma unroll
+          for (int j = 0; j < TX_ROWS; ++j) {
+            const int i = tid + 256 * j;
+            if (i > k && i < n) need |= 3u << (2 * j);
+          }
+          const long long c0 = clock64();
+          do {
+#pragma unroll
+            for (int j = 0; j <= TX_ROWS; ++j) {
+              const int i = j < TX_ROWS ? tid + 256 * j : k + 1;
+              double v;
+              if ((need >> (2 * j)) & 1u) {
+                if (pkt_load(gq + (size_t)b * n + i, (uint32_t)(k + 1), &v)) {
+                  need &= ~(1u << (2 * j));
+                  if (j < TX_ROWS) qv[j] = v;
+                  else q0 = v;
+                }
+              }
+              if ((need >> (2 * j)) & 2u) {
+                if (pkt_load(ga + (size_t)b * n + i, (uint32_t)(k + 1), &v)) {
+                  need &= ~(2u << (2 * j));
+                  if (j < TX_ROWS) av[j] = v;
+                  else a0 = v;
+                }
+              }
+            }
+          } while (need && clock64() - c0 < tc::kWaitCycles);
+          const bool done = need == 0u;
+          ok = done;
+        }
+        ok = tc::mbar_wait(&sbar, (uint32_t)(k & 1)) && ok;
+        if (!ok) abort_flag[b] = 1;
+        const double beta = scal[0], eta = scal[1], mh = scal[2], u0 = scal[3], ue = scal[4], f0 = scal[5];
+        double u[TX_ROWS], z[TX_ROWS], y[TX_ROWS], g = 0.0, e0 = 0.0;
+        if (any) {
+#pragma unroll
+          for (int j = 0; j < TX_ROWS; ++j) {
+            const int i = tid + 256 * j, base = 256 * j + 32 * warp;
+            u[j] = z[j] = y[j] = 0.0;
+            if (base < n && base + 31 > k) {
+              u[j] = i == k + 1 ? u0 : i > k ? xr[j] : 0.0;
+              z[j] = fma(-beta, av[j], qv[j]);  // t
+              g = fma(u[j], z[j], g);
+            }
+          }
+          g = warp_sum_fx(g);
+          // beside the sum: eta t, a - u_0 eta t, eta t_0
+#pragma unroll
+          for (int j = 0; j < TX_ROWS; ++j) {
+            const int base = 256 * j + 32 * warp;
+            if (base < n && base + 31 > k) {
+              y[j] = fma(-ue, z[j], av[j]);
+              z[j] *= eta;
+            }
+          }
+          e0 = eta * fma(-beta, a0, q0);
+        }
+        if (lane == 0) red[warp] = g;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (any) {
+          const double gam = n <= 64 ? red[0] + red[1] : warp_sum_fx(lane < 8 ? red[lane] : 0.0);
+          // w = eta t + kappa u, kappa = -eta^2 gam / 2;  x' = a - u w_0 - w u_0
+          //   = (a - u_0 eta t) - u (eta t_0 + 2 kappa u_0)
+          const double c0 = fma(f0, gam, e0), kap = mh * gam;
+#pragma unroll
+          for (int j = 0; j < TX_ROWS; ++j) {
+            const int i = tid + 256 * j, base = 256 * j + 32 * warp;
+            if (base < n && base + 31 > k) {
+              const double x = fma(-u[j], c0, y[j]);
+              const double w = fma(kap, u[j], z[j]);
+              if (i > k && i < n) {
+                U[i] = u[j];
+                W[i] = w;
+                X[i] = x;
+                xr[j] = x;
+                if (k % P == r) {
+                  H[(size_t)k * n + i] = u[j];
+                  if (i == k + 1) {
+                    d[k + 1] = x;  // a_0 - 2 u_0 w_0: the next diagonal entry
+                    e[k] = beta;
+                    tau[k] = eta;
+                  }
+                  if (k + 3 == n && i == n - 1) e[n - 2] = x;
+                }
+              }
+            }
+          }
         }
       }
-    }
-    cluster.sync();
-    // the owner of column k + 1 computes the next scalars; its warp 0 updates only that column
-    const bool next_owner = (k + 1) % P == r && k + 3 < n;
-    if (t != 0.0) {
-      for (int i = tid; i < rr; i += blockDim.x) {
-        const int c = k + 1 + i;
-        w[i] = cluster.map_shared_rank(prod, c % P)[c / P];
+      __syncthreads();
+      if (abort_flag[b]) {
+        if (tid == 0) atomicExch(err, 2);
+        break;
       }
-      __syncthreads();
-      double pv = 0.0;
-      for (int i = tid; i < rr; i += blockDim.x) pv += w[i] * v[i];
-      const double K = -0.5 * t * block_sum(pv, red);
-      for (int i = tid; i < rr; i += blockDim.x) w[i] += K * v[i];
-      __syncthreads();
-      if (next_owner && warp == 0) {
-        const int q = qa;  // column k + 1
-        double* col = cols + (size_t)q * n;
-        double s2 = rank2_part<true>(col + k + 1, v, w, v[0], w[0], rr, lane);
-        s2 = warp_sum(s2);
-        __syncwarp();
-        if (lane == 0) {
-          double* h = hs + (size_t)q * TRI_DS_SLOTS;
-          house_scalars(col[k + 2], s2, h + 0, h + 1, h + 2);
-          h[3] = col[k + 1];
-        }
+      const bool more = k + 3 < n;
+      if (warp == 8) {
+        if (more) scalars(k + 1);
       } else {
-        const int q0 = next_owner ? qa + 1 : qa, w0 = next_owner ? 1 : 0, ws = nw - w0;
-        for (int q = q0 + (warp - w0); q < nq; q += ws) {
-          const int c = r + q * P;
-          rank2_part<false>(cols + (size_t)q * n + k + 1, v, w, v[c - k - 1], w[c - k - 1], rr, lane);
-        }
-      }
-    } else if (next_owner && warp == 0) {
-      // no update this step: column k + 1 as it stands
-      const int q = qa;
-      const double* col = cols + (size_t)q * n;
-      double s2 = 0.0;
-      for (int i = k + 3 + lane; i < n; i += 32) s2 += col[i] * col[i];
-      s2 = warp_sum(s2);
-      if (lane == 0) {
-        double* h = hs + (size_t)q * TRI_DS_SLOTS;
-        house_scalars(col[k + 2], s2, h + 0, h + 1, h + 2);
-        h[3] = col[k + 1];
+        pass(k, true, more);
       }
     }
-    cluster.sync();
-  }
-  // outputs of the owned pivot columns k < n - 2: d, e, tau and H(:, k) = (1, x sc)
-  for (int q = 0; q < nq; ++q) {
-    const int k = r + q * P;
-    if (k + 2 >= n) break;
-    const double* col = cols + (size_t)q * n;
-    const double* h = hs + (size_t)q * TRI_DS_SLOTS;
-    const double sc = h[2];
-    for (int i = k + 1 + tid; i < n; i += blockDim.x) H[(int64_t)k * n + i] = i == k + 1 ? 1.0 : col[i] * sc;
-    if (tid == 0) {
-      d[k] = h[3];
-      e[k] = h[0];
-      tau[k] = h[1];
+    __syncthreads();
+    if ((n - 1) % P == r && tid == 0) d[n - 1] = cols[(size_t)((n - 1 - r) / P) * ld + n - 1];
+  } else if (r == 0 && tid == 0) {
+    d[0] = Min[0];
+    if (n == 2) {
+      e[0] = Min[1];
+      d[1] = Min[3];
     }
   }
-  // last 2 x 2 block
-  if (n >= 2 && (n - 2) % P == r && tid == 0) {
-    const double* mc = cols + (size_t)((n - 2 - r) / P) * n;
-    d[n - 2] = mc[n - 2];
-    e[n - 2] = mc[n - 1];
-  }
-  if ((n - 1) % P == r && tid == 0) d[n - 1] = cols[(size_t)((n - 1 - r) / P) * n + n - 1];
+  if (CL) cg::this_cluster().sync();  // nobody leaves while another CTA may still send to it
 }
 
 // ------------------------------------------------------------------ tridiagonal eigenvalues
@@ -989,6 +1200,338 @@ __global__ void __launch_bounds__(32) bisect_kernel(int n, const double* __restr
   }
 }
 
+// ------------------------------------------------------------------ eigenpairs of T, one warp each
+// Eigenvalue j of T = tridiag(e, d, e) and its eigenvector, one warp per eigenvalue, four per CTA.  An
+// FP64 instruction takes 64 clocks of its SM sub-partition, so the time is the number of FP64
+// instructions per Sturm step times the number of passes over T; bisect_kernel needs 3 and 11-12.
+//   * Search: 4 passes of 32 trial points in FP32 narrow Gershgorin's interval by 33^4; the result
+//     and a margin bracket the FP64 search (the first FP64 pass counts at both ends and widens the
+//     bracket on the side that turns out wrong).  Once a bracket between neighbouring points holds
+//     one eigenvalue, the secant of the last minor through them estimates it, and the next 32
+//     points lie at distances w 4^-i (i = 0 .. 15) on both sides of the estimate: the bracket shrinks
+//     to about four times the secant's error without that error being known, so 3-4 FP64 passes
+//     reach round-off.  Clusters go on by multisection (5 bits a pass).
+//   * Sturm step in FP64, 2 instructions: the minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} as
+//     p_i = c_i q_i with c_i = e_{i-1}^2 c_{i-2}: q_i = a_i q_{i-1} - q_{i-2}, a_i = (d_i - x) g_i,
+//     g_i = c_{i-1} / c_i = 1 / (e_{i-1}^2 g_{i-1}), one FMA each for a_i and q_i.  c restarts every
+//     8 steps (q_{i-2} is multiplied by the last g) with a power-of-two rescaling.  |e| is kept
+//     >= 2^-100 ||T|| so that no g overflows (a change far below the rounding of T).
+//   * Vector: the rows of (T - x) z = 0 solved forwards from z_0 = 1 (lane 0) and backwards from
+//     z_{n-1} = 1 (lane 1), both rescaled by powers of two, joined at the index k with the largest
+//     |f_k b_k|, which is proportional to the k-th diagonal entry of (T - x)^-1 (the twisted
+//     factorisation of Fernando and Parlett): every row but k holds to rounding and row k's
+//     residual is the smallest possible.
+// Vectors of numerically equal eigenvalues (gap <= 1e-9 ||T||) are replaced by inviter_kernel.
+constexpr int TE_WARPS = 4;
+constexpr int TE_MAX_N = 1408;
+
+size_t tri_eig_smem(int n) {
+  const size_t ng = ((size_t)n + 7) / 8 + 1;
+  return (size_t)n * (7 + 2 * TE_WARPS) * sizeof(double) + (size_t)n * 2 * sizeof(float) +
+         2 * TE_WARPS * ng * sizeof(int) + 16;
+}
+
+// x 2^k, 0 when the result leaves the normal range downwards (x normal or 0, the result does not overflow).
+__device__ __forceinline__ double scale2(double x, int k) {
+  const int hi = __double2hiint(x), ef = (hi >> 20) & 0x7ff;
+  const int nf = ef + k;
+  return ef != 0 && nf > 0 ? __hiloint2double(hi + (k << 20), __double2loint(x)) : 0.0;
+}
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// FP32 Sturm count of T / ||T|| at x.
+__device__ __forceinline__ int sturm_count_f32(int n, const float* d, const float* e2, float x) {
+  float pm = 1.f, p = d[0] - x;
+  uint32_t hp = __float_as_uint(p);
+  int cnt = (int)(hp >> 31);
+  int i = 1;
+  for (; i + 4 <= n; i += 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float pn = fmaf(d[i + u] - x, p, -(e2[i + u] * pm));
+      const uint32_t hn = __float_as_uint(pn);
+      cnt += (int)((hn ^ hp) >> 31);
+      pm = p;
+      p = pn;
+      hp = hn;
+    }
+    const int ef = (int)max((hp >> 23) & 0xffu, (__float_as_uint(pm) >> 23) & 0xffu);
+    const float sc = __int_as_float((254 - min(max(ef, 1), 253)) << 23);  // 2^-(exponent)
+    p *= sc;
+    pm *= sc;
+  }
+  for (; i < n; ++i) {
+    const float pn = fmaf(d[i] - x, p, -(e2[i] * pm));
+    const uint32_t hn = __float_as_uint(pn);
+    cnt += (int)((hn ^ hp) >> 31);
+    pm = p;
+    p = pn;
+    hp = hn;
+  }
+  return cnt;
+}
+
+// FP64 Sturm count at x (scaled), and the last minor as q 2^qe (up to a factor common to all x).
+__device__ __forceinline__ int sturm_count_g(int n, double d0, const double* g, const double* dg, double x, double* q,
+                                             int* qe) {
+  double pm = 1.0, p = d0 - x;
+  uint32_t hp = (uint32_t)__double2hiint(p);
+  int cnt = (int)(hp >> 31), ee = 0;
+  int i = 1;
+  for (; i + 8 <= n; i += 8) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const double pn = fma(fma(-x, g[i + u], dg[i + u]), p, -pm);
+      const uint32_t hn = (uint32_t)__double2hiint(pn);
+      cnt += (int)((hn ^ hp) >> 31);
+      pm = p;
+      p = pn;
+      hp = hn;
+    }
+    pm *= g[i + 7];
+    const int ex = max(exp_field(p), exp_field(pm)) - 1023;
+    p = scale2(p, -ex);
+    pm = scale2(pm, -ex);
+    hp = (hp & 0x80000000u) | ((uint32_t)__double2hiint(p) & 0x7fffffffu);
+    ee += ex;
+  }
+  for (; i < n; ++i) {
+    const double pn = fma(fma(-x, g[i], dg[i]), p, -pm);
+    const uint32_t hn = (uint32_t)__double2hiint(pn);
+    cnt += (int)((hn ^ hp) >> 31);
+    pm = p;
+    p = pn;
+    hp = hn;
+  }
+  *q = p;
+  *qe = ee;
+  return cnt;
+}
+
+__global__ void __launch_bounds__(32 * TE_WARPS) tri_eig_kernel(int n, const double* __restrict__ d,
+                                                                const double* __restrict__ e, double* lam,
+                                                                double* tnorm_out, double* Z) {
+  extern __shared__ double sm[];
+  __shared__ double rmin[TE_WARPS], rmax[TE_WARPS];
+  const int ng = (n + 7) / 8 + 1;
+  double* g = sm;          // g_i, (d_i) g_i: row i of the Sturm recurrence
+  double* dg = g + n;
+  double* rf = dg + n;     // e_{i-1} / e_i and d_i / e_i, 1 / e_i: forward solve, row i
+  double* df = rf + n;
+  double* ie = df + n;
+  double* rb = ie + n;     // e_i / e_{i-1} and d_i / e_{i-1}: backward solve, row i
+  double* db = rb + n;
+  double* vec = db + n;    // per warp: n forward, n backward values
+  float* d32 = reinterpret_cast<float*>(vec + (size_t)2 * TE_WARPS * n);
+  float* e32 = d32 + n;
+  int* vex = reinterpret_cast<int*>(e32 + n);  // per warp: exponents of every 8 values, both directions
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // Gershgorin's interval
+  double glo = DBL_MAX, ghi = -DBL_MAX;
+  for (int i = tid; i < n; i += 32 * TE_WARPS) {
+    const double r = (i + 1 < n ? fabs(e[i]) : 0.0) + (i > 0 ? fabs(e[i - 1]) : 0.0);
+    glo = fmin(glo, d[i] - r);
+    ghi = fmax(ghi, d[i] + r);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
+    ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
+  }
+  if (lane == 0) {
+    rmin[warp] = glo;
+    rmax[warp] = ghi;
+  }
+  __syncthreads();
+  for (int w = 0; w < TE_WARPS; ++w) {
+    glo = fmin(glo, rmin[w]);
+    ghi = fmax(ghi, rmax[w]);
+  }
+  const double tnorm = fmax(fabs(glo), fabs(ghi));
+  const double inv = tnorm > 0.0 ? 1.0 / tnorm : 1.0;
+  // scaled off-diagonal entry, kept away from zero
+  auto es = [&](int i) {
+    const double v = e[i] * inv;
+    return fabs(v) < 0x1p-100 ? 0x1p-100 : v;
+  };
+  for (int i = tid; i < n; i += 32 * TE_WARPS) {
+    const double ds = d[i] * inv;
+    const double ec = i + 1 < n ? es(i) : 1.0, ep = i > 0 ? es(i - 1) : 0.0;
+    const double ic = rcp_h3(ec < 0.0 ? -ec : ec) * (ec < 0.0 ? -1.0 : 1.0);
+    const double ip = i > 0 ? rcp_h3(ep < 0.0 ? -ep : ep) * (ep < 0.0 ? -1.0 : 1.0) : 0.0;
+    ie[i] = ic;
+    rf[i] = ep * ic;
+    df[i] = ds * ic;
+    rb[i] = i + 1 < n ? ec * ip : 0.0;
+    db[i] = ds * ip;
+    d32[i] = (float)ds;
+    e32[i] = (float)(ep * ep);
+  }
+  for (int t = tid; 1 + 8 * t < n; t += 32 * TE_WARPS) {
+    double gp = 1.0;
+    for (int i = 1 + 8 * t; i < min(n, 9 + 8 * t); ++i) {
+      const double ev = es(i - 1);
+      gp = rcp_h3(ev * ev * gp);
+      g[i] = gp;
+      dg[i] = d[i] * inv * gp;
+    }
+  }
+  __syncthreads();
+  const int j = blockIdx.x * TE_WARPS + warp;
+  if (j >= n) return;
+  const double d0 = d[0] * inv;
+  glo = glo * inv - 4.0 * DBL_EPSILON;
+  ghi = ghi * inv + 4.0 * DBL_EPSILON;
+  // ---- FP32 multisection
+  float flo = (float)glo, fhi = (float)ghi;
+  for (int it = 0; it < 4; ++it) {
+    const float w = (fhi - flo) * (1.f / 33.f);
+    const int cnt = sturm_count_f32(n, d32, e32, flo + w * (float)(lane + 1));
+    const unsigned ge = __ballot_sync(0xffffffffu, cnt > j);
+    const int q = ge ? __ffs(ge) - 1 : 32;
+    const float a = flo + w * (float)q;
+    fhi = q < 32 ? flo + w * (float)(q + 1) : fhi;
+    flo = q > 0 ? a : flo;
+  }
+  // ---- FP64
+  double lo = fmax(glo, (double)flo - 3e-6), hi = fmin(ghi, (double)fhi + 3e-6);
+  bool lo_ok = false, hi_ok = false, sec = false;
+  double xs = 0.0;
+  for (int it = 0; it < 80; ++it) {
+    const double w = hi - lo;
+    if (lo_ok && hi_ok && w <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + 0.5 * DBL_EPSILON) break;
+    double x;
+    if (sec) {
+      const int i = lane < 16 ? lane : 31 - lane;
+      const double o = scale2(w, -2 * i);
+      x = fmin(fmax(lane < 16 ? xs - o : xs + o, lo), hi);
+    } else if (lo_ok && hi_ok) {
+      x = fma(w, (double)(lane + 1) * (1.0 / 33.0), lo);
+    } else {
+      x = lane == 31 ? hi : fma(w, (double)lane * (1.0 / 31.0), lo);
+    }
+    double qv;
+    int qe;
+    const int cnt = sturm_count_g(n, d0, g, dg, x, &qv, &qe);
+    const unsigned ge = __ballot_sync(0xffffffffu, cnt > j);
+    const int q = ge ? __ffs(ge) - 1 : 32;
+    sec = false;
+    if (q == 0) {
+      const double x0 = __shfl_sync(0xffffffffu, x, 0);
+      hi = x0;
+      hi_ok = true;
+      if (!lo_ok) {
+        lo = fmax(glo, x0 - 8.0 * w);
+        lo_ok = lo == glo;
+      }
+    } else if (q == 32) {
+      const double x1 = __shfl_sync(0xffffffffu, x, 31);
+      lo = x1;
+      lo_ok = true;
+      if (!hi_ok) {
+        hi = fmin(ghi, x1 + 8.0 * w);
+        hi_ok = hi == ghi;
+      }
+    } else {
+      const double xl = __shfl_sync(0xffffffffu, x, q - 1), xh = __shfl_sync(0xffffffffu, x, q);
+      const int cl = __shfl_sync(0xffffffffu, cnt, q - 1), ch = __shfl_sync(0xffffffffu, cnt, q);
+      const double ql = __shfl_sync(0xffffffffu, qv, q - 1), qh = __shfl_sync(0xffffffffu, qv, q);
+      const int el = __shfl_sync(0xffffffffu, qe, q - 1), eh = __shfl_sync(0xffffffffu, qe, q);
+      lo = xl;
+      hi = xh;
+      lo_ok = hi_ok = true;
+      if (ch - cl == 1) {
+        // zero of the line through (xl, ql) and (xh, qh), opposite signs
+        const int de = eh - el;
+        const double a = fabs(de > 0 ? scale2(ql, -de) : ql), b = fabs(de < 0 ? scale2(qh, de) : qh);
+        const double t = a + b;
+        if (t > 0.0 && t < DBL_MAX) {
+          xs = fma(xh - xl, a / t, xl);
+          sec = true;
+        }
+      }
+    }
+  }
+  const double xl = 0.5 * (lo + hi);
+  if (lane == 0) {
+    lam[j] = xl * tnorm;
+    if (j == 0) *tnorm_out = tnorm;
+  }
+  // ---- vector: lane 0 forwards, lane 1 backwards
+  double* F = vec + (size_t)warp * 2 * n;
+  double* B = F + n;
+  int* eF = vex + warp * 2 * ng;
+  int* eB = eF + ng;
+  if (lane < 2) {
+    const bool fw = lane == 0;
+    const int st = fw ? 1 : -1;
+    int i = fw ? 0 : n - 1;
+    const double* pa = fw ? ie : ie - 1;  // 1 / e_i, or 1 / e_{i-1}
+    const double* pd = fw ? df : db;
+    const double* pr = fw ? rf : rb;
+    double* out = fw ? F : B;
+    int* oe = fw ? eF : eB;
+    double zm = 0.0, z = 1.0;
+    int ee = 0;
+    for (int s0 = 0; s0 < n; s0 += 8) {
+      // values s0 .. s0 + 7 of this direction share the exponent ee
+      oe[s0 >> 3] = ee;
+      const int m = min(8, n - s0);
+      for (int u = 0; u < m; ++u) {
+        out[i] = z;
+        if (s0 + u + 1 < n) {
+          // z_next = -((d_i - x) z + e_prev zm) / e_next
+          const double zn = fma(fma(xl, pa[i], -pd[i]), z, -(pr[i] * zm));
+          zm = z;
+          z = zn;
+        }
+        i += st;
+      }
+      const int ex = max(exp_field(z), exp_field(zm)) - 1023;
+      z = scale2(z, -ex);
+      zm = scale2(zm, -ex);
+      ee += ex;
+    }
+  }
+  __syncwarp();
+  // the joining index: largest |f_k b_k|, compared by exponent, then by the product of significands
+  int be = -2000000000, bk = 0;
+  double bm = -1.0;
+  for (int k = lane; k < n; k += 32) {
+    const double f = F[k], b = B[k];
+    const int ff = exp_field(f), bf = exp_field(b);
+    if (ff == 0 || bf == 0) continue;
+    const int ex = eF[k >> 3] + eB[(n - 1 - k) >> 3] + ff + bf;
+    const double m = fabs(scale2(f, 1023 - ff) * scale2(b, 1023 - bf));
+    if (ex > be || (ex == be && m > bm)) {
+      be = ex;
+      bm = m;
+      bk = k;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const int oe = __shfl_xor_sync(0xffffffffu, be, o), ok = __shfl_xor_sync(0xffffffffu, bk, o);
+    const double om = __shfl_xor_sync(0xffffffffu, bm, o);
+    if (oe > be || (oe == be && (om > bm || (om == bm && ok < bk)))) {
+      be = oe;
+      bm = om;
+      bk = ok;
+    }
+  }
+  const double fk = F[bk], bkv = B[bk];
+  const int fe = eF[bk >> 3], bee = eB[(n - 1 - bk) >> 3];
+  const double sf = 1.0 / fk, sb = 1.0 / bkv;
+  __syncwarp();
+  double nr = 0.0;
+  for (int k = lane; k < n; k += 32) {
+    const double z = k <= bk ? scale2(F[k] * sf, eF[k >> 3] - fe) : scale2(B[k] * sb, eB[(n - 1 - k) >> 3] - bee);
+    F[k] = z;
+    nr = fma(z, z, nr);
+  }
+  const double sc = rsqrt_h3(warp_sum_fx(nr));
+  double* zj = Z + (size_t)j * n;
+  for (int k = lane; k < n; k += 32) zj[k] = F[k] * sc;
+}
+
 // ------------------------------------------------------------------ tridiagonal eigenvectors
 // LU factorisation with partial pivoting of T - lam I (one thread).  Row i of U holds u0 (diagonal),
 // u1, u2 (first and second superdiagonals); mult/sw record the elimination of row i + 1.
@@ -1059,7 +1602,7 @@ __device__ void tri_solve(int n, const double* u0, const double* u1, const doubl
 // eigenvectors of T.  A cluster larger than maxc sets *flag (the caller then uses another solver).
 __global__ void __launch_bounds__(32) inviter_kernel(int n, const double* __restrict__ d, const double* __restrict__ e,
                                                      const double* __restrict__ lam, const double* __restrict__ tnorm_p,
-                                                     double* Z, int maxc, int* flag) {
+                                                     double* Z, int maxc, int clusters_only, int* flag) {
   extern __shared__ double sm[];
   const int j = blockIdx.x;
   const int lane = threadIdx.x & 31;
@@ -1069,6 +1612,7 @@ __global__ void __launch_bounds__(32) inviter_kernel(int n, const double* __rest
   if (j > 0 && lam[j] - lam[j - 1] <= ortol) return;  // not the first member of its cluster
   int k = j + 1;
   while (k < n && lam[k] - lam[k - 1] <= ortol) ++k;
+  if (clusters_only && k == j + 1) return;
   if (k - j > maxc) {
     if (lane == 0) atomicExch(flag, 1);
     return;
@@ -1160,13 +1704,16 @@ __global__ void __launch_bounds__(64) backtransform_reg_kernel(int n, const doub
       }
     }
     const double tk = tau[k];
+    // (rows up to k are not touched: their chunks are skipped, an FP64 instruction costs the same
+    // with zeros; likewise the chunks past n of a wider instantiation)
     double s = 0.0;
 #pragma unroll
-    for (int t = 0; t < R; ++t) s += hc[t] * z[t];
-    s = warp_sum(s) * tk;
+    for (int t = 0; t < R; ++t)
+      if (32 * t + 31 > k && 32 * t < n) s = fma(hc[t], z[t], s);
+    s = warp_sum_fx(s) * tk;
 #pragma unroll
     for (int t = 0; t < R; ++t) {
-      z[t] -= s * hc[t];
+      if (32 * t + 31 > k && 32 * t < n) z[t] = fma(-s, hc[t], z[t]);
       hc[t] = hn[t];
     }
   }
@@ -1314,43 +1861,44 @@ bool launch_resident(cudaStream_t s, void (*kc)(Args...), void (*kg)(Args...), i
   return true;
 }
 
-// Above this order the tridiagonalisation runs on a cooperative grid of one CTA per SM: its rank-2
-// updates, O(n^2) FP64 work per column, then outweigh the grid barrier's cost over the cluster's
-// (measured per Rayleigh-Ritz step: n = 240 cluster 4.10 ms / grid 4.52 ms, n = 600 18.8 / 16.3 ms;
-// a n^3 + b n fits put the crossover near 380).
-constexpr int kTriClusterMaxN = 384;
+// tridiag_xch_kernel: one cluster up to this order, above it a cooperative grid (a grid's exchange
+// through L2 costs ~1 us more per column, but spreads the FP64 work over more SMs).  Measured (us),
+// cluster of 16 / grid of 96: n = 240 1036 / 1237, 300 1607 / 1704, 384 2573 / 2338, 480 4016 / 3220.
+constexpr int kTriClusterMaxN = 320;
 
-// tridiag_smem_kernel on a cooperative grid of one CTA per SM when the owned columns fit in shared
-// memory; false otherwise.
-bool launch_tridiag_grid(cudaStream_t s, int n, int num_sms, const double* M, double* H, double* d, double* e,
-                         double* tau, double* xch, double* p) {
-  const int P = num_sms;
-  const size_t smem = resident_smem(n, P);
+// The workspace tridiag_xch_kernel needs on a grid, in doubles (4 n packets of 16 bytes).
+size_t tridiag_xch_ws(int n) { return 8 * (size_t)n + 2; }
+
+// False when the matrix does not fit (n > 1024, or no shared memory for the owned columns).
+bool launch_tridiag_xch(cudaStream_t s, int n, int num_sms, const double* M, double* H, double* d, double* e,
+                        double* tau, double* xg, int* err) {
+  if (n > 256 * TX_ROWS) return false;
+  if (n <= kTriClusterMaxN) {
+    static const int csz = cluster_size_for(reinterpret_cast<const void*>(tridiag_xch_kernel<true>), TX_THREADS,
+                                            tridiag_xch_smem(kTriClusterMaxN, 16, true));
+    // 8 CTAs reach the floor of the exchange for small orders (n = 60: 158 us, 4: 166, 16: 164)
+    const int P = std::min(csz, n <= 96 ? 8 : 16);
+    const size_t smem = P > 0 ? tridiag_xch_smem(n, P, true) : 0;
+    if (P > 0 && smem <= SMEM_CAP) {
+      cudaLaunchAttribute at[1];
+      cudaLaunchConfig_t cfg = cluster_cfg(P, TX_THREADS, smem, s, at);
+      RC_CUDA(cudaLaunchKernelEx(&cfg, tridiag_xch_kernel<true>, n, M, H, d, e, tau, (uint4*)nullptr, err));
+      RC_LAUNCH();
+      return true;
+    }
+  }
+  const int P = std::min(num_sms, n <= 512 ? 96 : 128);
+  const size_t smem = tridiag_xch_smem(n, P, false);
   if (smem > SMEM_CAP) return false;
-  static const bool attr = [] {
-    RC_CUDA(cudaFuncSetAttribute(reinterpret_cast<const void*>(tridiag_smem_kernel<false>),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_CAP));
-    return true;
-  }();
-  (void)attr;
+  set_smem_limit(reinterpret_cast<const void*>(tridiag_xch_kernel<false>), (int)SMEM_CAP);
   int per_sm = 0;
-  RC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tridiag_smem_kernel<false>, TRI_THREADS, smem));
+  RC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tridiag_xch_kernel<false>, TX_THREADS, smem));
   if (per_sm < 1) return false;
-  int nn = n;
-  void* argv[] = {(void*)&nn, (void*)&M, (void*)&H, (void*)&d, (void*)&e, (void*)&tau, (void*)&xch, (void*)&p};
-  RC_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(tridiag_smem_kernel<false>), dim3(P),
-                                      dim3(TRI_THREADS), argv, smem, s));
-  RC_LAUNCH();
-  return true;
-}
-
-// One cluster of tridiag_dsmem_kernel when its CTAs hold the owned columns; false otherwise.
-bool launch_tridiag_dsmem(cudaStream_t s, int n, const double* M, double* H, double* d, double* e, double* tau) {
-  static const int csz = cluster_size_for(reinterpret_cast<const void*>(tridiag_dsmem_kernel), TRI_THREADS, SMEM_CAP);
-  if (csz <= 0 || tridiag_dsmem_smem(n, csz) > SMEM_CAP) return false;
-  cudaLaunchAttribute at[1];
-  cudaLaunchConfig_t cfg = cluster_cfg(csz, TRI_THREADS, tridiag_dsmem_smem(n, csz), s, at);
-  RC_CUDA(cudaLaunchKernelEx(&cfg, tridiag_dsmem_kernel, n, M, H, d, e, tau));
+  uint4* pk = reinterpret_cast<uint4*>((reinterpret_cast<uintptr_t>(xg) + 15) & ~uintptr_t(15));
+  RC_CUDA(cudaMemsetAsync(pk, 0, 64 * (size_t)n, s));  // no packet carries a tag yet
+  void* argv[] = {(void*)&n, (void*)&M, (void*)&H, (void*)&d, (void*)&e, (void*)&tau, (void*)&pk, (void*)&err};
+  RC_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(tridiag_xch_kernel<false>), dim3(P),
+                                      dim3(TX_THREADS), argv, smem, s));
   RC_LAUNCH();
   return true;
 }
@@ -1366,18 +1914,15 @@ void launch_backtransform(cudaStream_t s, int n, const double* H, const double* 
 int cholesky_inverse_f64(cudaStream_t s, int n, double* A, double* L, double* Linv, int* d_info, int num_sms,
                          DevBuf<double>& scratch) {
   RC_CHECK(n >= 1 && n <= 6144, RCHFSI_ERR_UNSUPPORTED, "cholesky_inverse: order out of [1, 6144]");
-  // blocked on a cooperative grid (5 grid barriers per 32 columns, FP64 work on every SM)
   {
     const int nt = (n + CB - 1) / CB;
-    const size_t need = (size_t)nt * CB * CB + 8;
-    double* di = scratch.ensure(std::max(need, 3 * (size_t)n));
-    int* bad = reinterpret_cast<int*>(di + (size_t)nt * CB * CB);
     int per_sm = 0;
     RC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chol_inv_blocked_kernel, 256, 0));
     if (per_sm >= 1) {
+      // no more CTAs than the largest phase has units (a barrier costs more with more CTAs)
       const int P = std::max(1, std::min(num_sms, 2 * nt * (nt + 1)));
       const double* Ac = A;
-      void* argv[] = {(void*)&n, (void*)&Ac, (void*)&L, (void*)&Linv, (void*)&di, (void*)&bad, (void*)&d_info};
+      void* argv[] = {(void*)&n, (void*)&Ac, (void*)&L, (void*)&Linv, (void*)&d_info};
       RC_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(chol_inv_blocked_kernel), dim3(P), dim3(256),
                                           argv, 0, s));
       RC_LAUNCH();
@@ -1396,9 +1941,9 @@ int cholesky_inverse_f64(cudaStream_t s, int n, double* A, double* L, double* Li
 bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, DevBuf<double>& ws, int* d_flag,
                  int num_sms, const OzScratch* oz) {
   if (n < 1 || n > 3072) return false;
-  // workspace: H, S, V2 (n^2 each), d, e, tau, p (n each), xch (n + 8), tnorm
+  // workspace: H, S, V2 (n^2 each), d, e, tau, p (n each), xch (n + 8), tnorm, exchange packets
   const size_t nn = (size_t)n * n;
-  double* H = ws.ensure(3 * nn + 6 * (size_t)n + 16);
+  double* H = ws.ensure(3 * nn + 6 * (size_t)n + 16 + tridiag_xch_ws(n));
   double* S = H + nn;
   double* V2 = S + nn;
   double* d = V2 + nn;
@@ -1407,6 +1952,7 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
   double* p = tau + n;
   double* xch = p + n;
   double* tnorm = xch + n + 8;
+  double* pkts = tnorm + 8;
   if (n == 1) {
     RC_CUDA(cudaMemcpyAsync(evals, M, sizeof(double), cudaMemcpyDeviceToDevice, s));
     const double one = 1.0;
@@ -1416,23 +1962,28 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
   }
   RC_CUDA(cudaMemsetAsync(e, 0, sizeof(double) * n, s));
   RC_CUDA(cudaMemsetAsync(tau, 0, sizeof(double) * n, s));
+  RC_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
   // 1. Q^T M Q = T
-  if (!(n <= kTriClusterMaxN ? launch_tridiag_dsmem(s, n, M, H, d, e, tau)
-                             : launch_tridiag_grid(s, n, num_sms, M, H, d, e, tau, xch, p)) &&
+  if (!launch_tridiag_xch(s, n, num_sms, M, H, d, e, tau, pkts, d_flag) &&
       !launch_resident(s, tridiag_smem_kernel<true>, tridiag_smem_kernel<false>, n, num_sms, n, (const double*)M, H,
                        d, e, tau, xch, p))
     launch_multi(s, tridiag_kernel<true>, tridiag_kernel<false>, n, num_sms, n, M, H, d, e, tau, p);
-  // 2. eigenvalues of T
-  bisect_kernel<<<n, 32, 2 * (size_t)n * sizeof(double), s>>>(n, d, e, evals, tnorm);
+  // 2. eigenvalues and eigenvectors of T (into V2), 3. the vectors of clusters
+  const bool pairs = n <= TE_MAX_N;
+  if (pairs) {
+    set_smem_limit(reinterpret_cast<const void*>(tri_eig_kernel), (int)SMEM_CAP);
+    tri_eig_kernel<<<cdiv(n, TE_WARPS), 32 * TE_WARPS, tri_eig_smem(n), s>>>(n, d, e, evals, tnorm, V2);
+  } else {
+    bisect_kernel<<<n, 32, 2 * (size_t)n * sizeof(double), s>>>(n, d, e, evals, tnorm);
+  }
   RC_LAUNCH();
-  // 3. eigenvectors of T (into V2)
-  RC_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
   set_smem_limit(reinterpret_cast<const void*>(inviter_kernel), (int)SMEM_CAP);
-  inviter_kernel<<<n, 32, inviter_smem(n), s>>>(n, d, e, evals, tnorm, V2, INV_MAX_CLUSTER, d_flag);
+  inviter_kernel<<<n, 32, inviter_smem(n), s>>>(n, d, e, evals, tnorm, V2, INV_MAX_CLUSTER, pairs ? 1 : 0, d_flag);
   RC_LAUNCH();
   int flag = 0;
   RC_CUDA(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
   RC_CUDA(cudaStreamSynchronize(s));
+  RC_CHECK(flag != 2, RCHFSI_ERR_TIMEOUT, "a bounded wait in the tridiagonalisation ran out");
   if (flag) return false;
   // 4. one Newton-Schulz step towards the orthogonal factor: Z <- Z (3 I - Z^T Z) / 2
   if (oz) {
