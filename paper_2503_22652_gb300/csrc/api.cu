@@ -856,8 +856,10 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
   // G_B = L L^T and L^-1 (one cluster / cooperative kernel); G_B is kept in Zt for a retry
   auto factor = [&]() {
     prof::Scope ps(c.s, RCHFSI_KERNEL_SMALL_DENSE, 2.0 * N * N * N / 3.0, 8.0 * N * N * 3);
-    symmetrize_f64(c.s, N, w.GA.p, N);
-    symmetrize_f64(c.s, N, w.GB.p, N);
+    if (!(emu && Na == N)) {  // (the emulated Gram matrices of a real problem are mirrored: exactly symmetric)
+      symmetrize_f64(c.s, N, w.GA.p, N);
+      symmetrize_f64(c.s, N, w.GB.p, N);
+    }
     RC_CUDA(cudaMemcpyAsync(w.Zt.p, w.GB.p, sizeof(double) * N * N, cudaMemcpyDeviceToDevice, c.s));
     cholesky_inverse_f64(c.s, N, w.GB.p, w.Lb.p, w.Li.p, w.info.p, c.num_sms, w.eigws);
     int inf = 0;
@@ -891,7 +893,13 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
   if (info != 0) return RCHFSI_ERR_ILL_CONDITIONED;
   // M = L^-1 G_A L^-T: two FP64-accurate products (BF16 slices on the tensor cores, the Gram
   // slices no longer needed) or two FP64 GEMMs on all SMs
-  if (emu) {
+  // (small N: FP64 products, see kSmallGemmMaxN; above it, slices on the tensor cores.  Measured per
+  // product with its slicings, N = 128: 15 us against 35 us; N = 240: 31 against 40 us)
+  const bool small = emu && N <= kSmallGemmMaxN;
+  if (small) {
+    gemm_small_f64(c.s, N, w.Li.p, 1, N, w.GA.p, 1, N, 1.0, 0.0, w.Zt.p, RCHFSI_KERNEL_SMALL_DENSE);
+    gemm_small_f64(c.s, N, w.Zt.p, 1, N, w.Li.p, N, 1, 1.0, 0.0, w.Z.p, RCHFSI_KERNEL_SMALL_DENSE);
+  } else if (emu) {
     oz_slice(c.s, N, N, w.Li.p, 1, N, w.ozR);   // L^-1, row i = L^-1(i, :)
     oz_slice(c.s, N, N, w.GA.p, N, 1, w.ozE);   // column j of G_A as row j
     oz_gemm(c.s, c.num_sms, w.ozR, w.ozE, w.Zt.p, N, w.ozws, eflag);
@@ -930,7 +938,9 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
   }
   // E = L^-T V
   double* Ep = vec == w.Z.p ? w.Zt.p : w.Z.p;
-  if (emu) {
+  if (small) {
+    gemm_small_f64(c.s, N, w.Li.p, N, 1, vec, 1, N, 1.0, 0.0, Ep, RCHFSI_KERNEL_SMALL_DENSE);
+  } else if (emu) {
     oz_slice(c.s, N, N, w.Li.p, N, 1, w.ozR);  // L^-T, row i = column i of L^-1
     oz_slice(c.s, N, N, vec, N, 1, w.ozE);     // column j of V as row j
     oz_gemm(c.s, c.num_sms, w.ozR, w.ozE, Ep, N, w.ozws, eflag);

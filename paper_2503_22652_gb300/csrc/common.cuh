@@ -130,6 +130,10 @@ struct EpiArgs {
 
 void gemm_f64(cudaStream_t s, int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, bool a_kcontig,
               const double* B, int64_t ldb, bool b_kcontig, const EpiArgs& epi);
+// N x N products at small N: C(i, j) = alpha sum_k A[i ai + k ak] B[k bk + j bj] + diag [i == j], C column-major.
+constexpr int kSmallGemmMaxN = 128;
+void gemm_small_f64(cudaStream_t s, int n, const double* A, int ai, int ak, const double* B, int bk, int bj,
+                    double alpha, double diag, double* C, int prof_cls);
 void gemm_f32(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, bool a_kcontig,
               const float* B, int64_t ldb, bool b_kcontig, const EpiArgs& epi);
 

@@ -180,6 +180,39 @@ __global__ void __launch_bounds__(256) gemv_kernel(int64_t M, int N, int64_t K, 
   }
 }
 
+// C(i, j) = alpha sum_k A(i, k) B(k, j) + diag [i == j] for the N x N products of Rayleigh-Ritz at small N
+// (element (i, k) of A at A[i * ai + k * ak], (k, j) of B at B[k * bk + j * bj], C column-major with
+// leading dimension n): 16 x 16 outputs per CTA, one per thread, so that even N = 48 spreads over 9
+// SMs.  The time is a thread's FMA chain on the FP64 pipe (two warps per sub-partition: 128 clocks
+// per k), against two slicings and a product on the tensor cores, whose cost at these sizes is their
+// launches and fills.
+__global__ void __launch_bounds__(256) gemm_small_f64_kernel(int n, const double* __restrict__ A, int ai, int ak,
+                                                             const double* __restrict__ B, int bk, int bj,
+                                                             double alpha, double diag, double* __restrict__ C) {
+  __shared__ double As[16][65], Bs[16][65];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int i0 = blockIdx.x * 16, j0 = blockIdx.y * 16;
+  double a0 = 0.0;
+  for (int k0 = 0; k0 < n; k0 += 64) {
+    // the inner index of the loads follows the contiguous one
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + 256 * u;
+      const int r = ak == 1 ? e >> 6 : e & 15, k = ak == 1 ? e & 63 : e >> 4;
+      As[r][k] = (i0 + r < n && k0 + k < n) ? A[(size_t)(i0 + r) * ai + (size_t)(k0 + k) * ak] : 0.0;
+      const int c = bk == 1 ? e >> 6 : e & 15, kb = bk == 1 ? e & 63 : e >> 4;
+      Bs[c][kb] = (j0 + c < n && k0 + kb < n) ? B[(size_t)(k0 + kb) * bk + (size_t)(j0 + c) * bj] : 0.0;
+    }
+    __syncthreads();
+    const int kn = min(64, n - k0);
+#pragma unroll 8
+    for (int k = 0; k < kn; ++k) a0 = fma(As[tx][k], Bs[ty][k], a0);
+    __syncthreads();
+  }
+  const int i = i0 + tx, j = j0 + ty;
+  if (i < n && j < n) C[(size_t)j * n + i] = fma(alpha, a0, i == j ? diag : 0.0);
+}
+
 template <typename T>
 __global__ void splitk_sum_kernel(int64_t M, int64_t N, int nsplit, const T* __restrict__ partial, EpiDev<T> epi) {
   const int64_t total = M * N;
@@ -265,6 +298,13 @@ void gemm_dispatch(cudaStream_t s, int64_t M, int64_t N, int64_t K, const T* A, 
 }
 
 }  // namespace
+
+void gemm_small_f64(cudaStream_t s, int n, const double* A, int ai, int ak, const double* B, int bk, int bj,
+                    double alpha, double diag, double* C, int prof_cls) {
+  prof::Scope ps(s, prof_cls, 2.0 * n * n * n, 8.0 * 3 * n * n);
+  gemm_small_f64_kernel<<<dim3(cdiv(n, 16), cdiv(n, 16)), 256, 0, s>>>(n, A, ai, ak, B, bk, bj, alpha, diag, C);
+  RC_LAUNCH();
+}
 
 void gemm_f64(cudaStream_t s, int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, bool a_kcontig,
               const double* B, int64_t ldb, bool b_kcontig, const EpiArgs& epi) {

@@ -45,7 +45,7 @@ constexpr uint32_t kTmemCols = 512;          // 8 level blocks x 64 columns
 // ---------------------------------------------------------------- slicing
 // Row exponents, K-contiguous rows: one warp per (row, K slice), the K range split over
 // blockIdx.y so that a few hundred rows still fill the GPU; slices meet in ex by atomicMax (ex
-// preset to INT_MIN), rowexp_fix maps rows without a nonzero element to 0.
+// preset to INT_MIN), slice_kernel maps rows without a nonzero element to 0.
 __global__ void rowexp_kcontig(int64_t R, int64_t K, const double* __restrict__ X, int64_t rs, int* ex) {
   const int64_t r = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
@@ -60,7 +60,7 @@ __global__ void rowexp_kcontig(int64_t R, int64_t K, const double* __restrict__ 
 
 // Row exponents, rows contiguous across threads (element (r, k) at X[r + k * ks]): 32 rows per
 // block (coalesced), the K range split over the block's 8 warps and over blockIdx.y.  Partial maxima
-// meet in ex by atomicMax (ex preset to INT_MIN); rowexp_fix then maps rows without a nonzero
+// meet in ex by atomicMax (ex preset to INT_MIN); slice_kernel maps rows without a nonzero
 // element to 0.
 __global__ void __launch_bounds__(256) rowexp_rcontig(int64_t R, int64_t K, const double* __restrict__ X, int64_t ks,
                                                       int* ex) {
@@ -79,14 +79,9 @@ __global__ void __launch_bounds__(256) rowexp_rcontig(int64_t R, int64_t K, cons
   }
 }
 
-__global__ void rowexp_fix(int64_t R, int* ex) {
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < R && ex[r] <= -100000) ex[r] = 0;
-}
-
 // Slices of a 32-row x 64-k tile.  Block (32, 8).
 __global__ void slice_kernel(int64_t R, int64_t Rp, int64_t K, int64_t Kp, const double* __restrict__ X, int64_t rs,
-                             int64_t ks, const int* __restrict__ ex, __nv_bfloat16* __restrict__ out) {
+                             int64_t ks, int* __restrict__ ex, __nv_bfloat16* __restrict__ out) {
   __shared__ double tile[32][KC + 1];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int64_t r0 = (int64_t)blockIdx.y * 32, k0 = (int64_t)blockIdx.x * KC;
@@ -106,7 +101,13 @@ __global__ void slice_kernel(int64_t R, int64_t Rp, int64_t K, int64_t Kp, const
   for (int rr = ty; rr < 32; rr += 8) {
     const int64_t r = r0 + rr;
     if (r >= R) continue;
-    const int e = ex[r];
+    // a row without a nonzero element has the exponent 0 (the blocks of the row agree on it; the one
+    // at k0 = 0 stores it, and another block reads either value)
+    int e = ex[r];
+    if (e <= -100000) {
+      e = 0;
+      if (k0 == 0 && tx == 0) ex[r] = 0;
+    }
     // digits t_s of x 2^(-e) = sum_s t_s 2^(-8(s+1)), rounded to nearest: |t_0| <= 256, |t_s| <= 128,
     // each exact in BF16; two neighbouring k per thread, stored as one 4-byte pair per slice
     long long f0 = fixed56(tile[rr][2 * tx], e), f1 = fixed56(tile[rr][2 * tx + 1], e);
@@ -123,6 +124,75 @@ __global__ void slice_kernel(int64_t R, int64_t Rp, int64_t K, int64_t Kp, const
       }
       // digits fit in 32 bits (|t| <= 256): an int conversion stays off the FP64 pipe, which a
       // 64-bit integer conversion occupies (a few DFMA per clock per SM on this GPU)
+      o2[(int64_t)s * Rp * Kp / 2] = __floats2bfloat162_rn((float)(int)t0, (float)(int)t1);
+    }
+  }
+}
+
+// Exponents and slices of RB rows in one pass, the rows held in shared memory between the two: one
+// read of X instead of two and one launch instead of four (preset, exponents, fix, slices).  Rows
+// R .. Rp - 1 are written as zeros.  256 threads.
+template <bool KCONTIG>
+__global__ void __launch_bounds__(256) slice_rows_kernel(int RB, int64_t R, int64_t Rp, int64_t K, int64_t Kp,
+                                                         const double* __restrict__ X, int64_t rs, int64_t ks, int* ex,
+                                                         __nv_bfloat16* __restrict__ out) {
+  extern __shared__ double tile[];  // RB x (K + 1)
+  __shared__ int rex[32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t r0 = (int64_t)blockIdx.x * RB, ld = K + 1;
+  if (tid < RB) rex[tid] = -100000;
+  __syncthreads();
+  if (KCONTIG) {
+    // a warp per run of 128 elements of a row, four loads in flight per lane
+    const int runs = (int)((K + 127) / 128);
+    for (int t = warp; t < RB * runs; t += 8) {
+      const int rr = t / runs;
+      const int64_t k0 = (int64_t)(t - rr * runs) * 128 + lane, r = r0 + rr;
+      if (r >= R) continue;
+      double v[4];
+      int e = -100000;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = k0 + 32 * u < K ? X[r * rs + k0 + 32 * u] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (k0 + 32 * u < K) tile[rr * ld + k0 + 32 * u] = v[u];
+        e = max(e, exp_of(v[u]));
+      }
+      e = __reduce_max_sync(0xffffffffu, e);
+      if (lane == 0) atomicMax(&rex[rr], e);
+    }
+  } else {
+    // RB consecutive rows (a power of two) by 256 / RB k per step
+    const int rr = tid & (RB - 1);
+    const int kst = 256 / RB;
+    const int64_t r = r0 + rr;
+    int e = -100000;
+    for (int64_t k0 = tid / RB; k0 < K; k0 += 4 * kst) {
+      double v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = r < R && k0 + u * kst < K ? X[r + (k0 + u * kst) * ks] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (k0 + u * kst < K) tile[rr * ld + k0 + u * kst] = v[u];
+        e = max(e, exp_of(v[u]));
+      }
+    }
+    atomicMax(&rex[rr], e);
+  }
+  __syncthreads();
+  if (tid < RB && r0 + tid < R) ex[r0 + tid] = rex[tid] == -100000 ? 0 : rex[tid];
+  const int segs = (int)(Kp / KC);
+  for (int t = warp; t < RB * segs; t += 8) {
+    const int rr = t / segs, k = (t - rr * segs) * KC + 2 * lane;
+    const int64_t r = r0 + rr;
+    if (r >= Rp) break;
+    __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(out + r * Kp + k);
+    const int e = rex[rr] == -100000 ? 0 : rex[rr];
+    long long f0 = r < R && k < K ? fixed56(tile[rr * ld + k], e) : 0;
+    long long f1 = r < R && k + 1 < K ? fixed56(tile[rr * ld + k + 1], e) : 0;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const long long t0 = next_digit(f0, s), t1 = next_digit(f1, s);
       o2[(int64_t)s * Rp * Kp / 2] = __floats2bfloat162_rn((float)(int)t0, (float)(int)t1);
     }
   }
@@ -478,24 +548,46 @@ void oz_slice(cudaStream_t s, int64_t R, int64_t K, const double* X, int64_t rs,
   op.sl.ensure((size_t)S * op.Rp * op.Kp);
   op.ex.ensure((size_t)R);
   prof::Scope ps(s, RCHFSI_KERNEL_RR_AUX, 0.0, 8.0 * R * K + 2.0 * S * op.Rp * op.Kp);
+  // One pass with the rows in shared memory, when RB rows of K fit (64 KB: three CTAs per SM) and
+  // there are CTAs for most of the SMs; RB is 8 (16) rows where rows are contiguous across threads, so
+  // that a load covers whole 64-byte runs, and down to 1 for few K-contiguous rows.  Measured against
+  // the separate passes (us, exponents + fix + slices -> one pass, without the launches in between):
+  // 60 x 60 18 -> 4.2, 240 x 240 19 -> 8, 4000 x 240 by rows 23 -> 11.6, 262144 x 600 by rows 1120 -> 943.
+  int rb = 0;
+  const size_t row = ((size_t)K + 1) * sizeof(double);
+  if (ks == 1) {
+    for (int c : {8, 4, 2, 1})
+      if (rb == 0 && c * row <= 66 * 1024 && (c == 1 || (int64_t)cdiv(R, c) >= sm_count() / 2)) rb = c;
+    if ((int64_t)R * 4 < sm_count()) rb = K <= 1024 ? rb : 0;  // few long rows: split along K instead
+  } else if (8 * row <= 66 * 1024) {
+    rb = 8;
+  }
+  if (rb > 0) {
+    const unsigned g = cdiv(op.Rp, rb);
+    const size_t smem = rb * row;
+    if (ks == 1) {
+      set_smem_limit(reinterpret_cast<const void*>(slice_rows_kernel<true>), 68 * 1024);
+      slice_rows_kernel<true><<<g, 256, smem, s>>>(rb, R, op.Rp, K, op.Kp, X, rs, ks, op.ex.p, op.sl.p);
+    } else {
+      set_smem_limit(reinterpret_cast<const void*>(slice_rows_kernel<false>), 68 * 1024);
+      slice_rows_kernel<false><<<g, 256, smem, s>>>(rb, R, op.Rp, K, op.Kp, X, rs, ks, op.ex.p, op.sl.p);
+    }
+    RC_LAUNCH();
+    return;
+  }
   if (op.Rp > R) RC_CUDA(cudaMemsetAsync(op.sl.p, 0, sizeof(__nv_bfloat16) * S * op.Rp * op.Kp, s));
+  RC_CUDA(cudaMemsetAsync(op.ex.p, 0x80, sizeof(int) * R, s));  // 0x80808080: below every exponent
   if (ks == 1) {
     // K slices of >= 256 elements, enough (row, slice) warps for ~16 per SM
-    const unsigned rb = cdiv(R, 8);
+    const unsigned rw = cdiv(R, 8);
     const unsigned kb = (unsigned)std::max<int64_t>(
         1, std::min<int64_t>(cdiv(K, 256), (int64_t)(sm_count() * 16 * 8) / std::max<int64_t>(R, 1)));
-    RC_CUDA(cudaMemsetAsync(op.ex.p, 0x80, sizeof(int) * R, s));  // 0x80808080: below every exponent
-    rowexp_kcontig<<<dim3(rb, kb), 256, 0, s>>>(R, K, X, rs, op.ex.p);
-    RC_LAUNCH();
-    rowexp_fix<<<cdiv(R, 256), 256, 0, s>>>(R, op.ex.p);
+    rowexp_kcontig<<<dim3(rw, kb), 256, 0, s>>>(R, K, X, rs, op.ex.p);
   } else {
     // enough blocks to fill the GPU a few times over, each warp walking at least 8 k
-    const unsigned rb = cdiv(R, 32);
-    const unsigned kb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(cdiv(K, 64), (int64_t)(sm_count() * 16) / rb));
-    RC_CUDA(cudaMemsetAsync(op.ex.p, 0x80, sizeof(int) * R, s));  // 0x80808080: below every exponent
-    rowexp_rcontig<<<dim3(rb, kb), dim3(32, 8), 0, s>>>(R, K, X, ks, op.ex.p);
-    RC_LAUNCH();
-    rowexp_fix<<<cdiv(R, 256), 256, 0, s>>>(R, op.ex.p);
+    const unsigned rw = cdiv(R, 32);
+    const unsigned kb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(cdiv(K, 64), (int64_t)(sm_count() * 16) / rw));
+    rowexp_rcontig<<<dim3(rw, kb), dim3(32, 8), 0, s>>>(R, K, X, ks, op.ex.p);
   }
   RC_LAUNCH();
   RC_CHECK(cdiv(R, 32) <= 65535u, RCHFSI_ERR_INVALID_ARG, "oz_slice: too many rows");

@@ -1986,7 +1986,11 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
   RC_CHECK(flag != 2, RCHFSI_ERR_TIMEOUT, "a bounded wait in the tridiagonalisation ran out");
   if (flag) return false;
   // 4. one Newton-Schulz step towards the orthogonal factor: Z <- Z (3 I - Z^T Z) / 2
-  if (oz) {
+  if (oz && n <= kSmallGemmMaxN) {
+    // S = 1.5 I - 0.5 Z^T Z, V = Z S
+    gemm_small_f64(s, n, V2, n, 1, V2, 1, n, -0.5, 1.5, S, RCHFSI_KERNEL_EIG);
+    gemm_small_f64(s, n, V2, 1, n, S, 1, n, 1.0, 0.0, V, RCHFSI_KERNEL_EIG);
+  } else if (oz) {
     // FP64-accurate products from BF16 slices: G = Z^T Z (symmetric), S = 1.5 I - 0.5 G, V = Z S
     oz_slice(s, n, n, V2, n, 1, *oz->a);  // row i = column i of Z
     oz_gemm(s, oz->num_sms, *oz->a, *oz->a, S, n, *oz->ws, oz->err, true);
