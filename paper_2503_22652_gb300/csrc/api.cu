@@ -34,8 +34,8 @@ void Work::ensure(int64_t m_, int N_) {
   GA.ensure((size_t)N * N); GB.ensure((size_t)N * N); Z.ensure((size_t)N * N); Zt.ensure((size_t)N * N);
   Lb.ensure((size_t)N * N); Li.ensure((size_t)N * N);
   evals.ensure(N); nrm.ensure(N); rabs.ensure(N); xnrm.ensure(N);
-  info.ensure(4);
-  RC_CUDA(cudaMemset(info.p, 0, 4 * sizeof(int)));
+  info.ensure(8);
+  RC_CUDA(cudaMemset(info.p, 0, 8 * sizeof(int)));
 }
 
 bool has_B(const rchfsi_ctx& c) {
@@ -782,23 +782,9 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
   Work& w = c.w;
   // column scaling to unit 2-norm (span unchanged)
   {
-    prof::Scope ps(c.s, RCHFSI_KERNEL_RR_AUX, 2.0 * m * N, 8.0 * m * N);
-    col_norms_f64(c.s, m, N, Y, m, w.nrm.p);
-  }
-  // invert norms on device: reuse scale kernel through a tiny copy
-  {
-    std::vector<double> hn(N);
-    RC_CUDA(cudaMemcpyAsync(hn.data(), w.nrm.p, N * sizeof(double), cudaMemcpyDeviceToHost, c.s));
-    RC_CUDA(cudaStreamSynchronize(c.s));
-    for (int j = 0; j < N; ++j) {
-      RC_CHECK(std::isfinite(hn[j]), RCHFSI_ERR_NUMERIC, "non-finite column in the filtered block");
-      RC_CHECK(hn[j] > 0.0, RCHFSI_ERR_ILL_CONDITIONED, "zero column in the filtered block");
-      hn[j] = 1.0 / hn[j];
-    }
-    RC_CUDA(cudaMemcpyAsync(w.nrm.p, hn.data(), N * sizeof(double), cudaMemcpyHostToDevice, c.s));
-    prof::Scope ps(c.s, RCHFSI_KERNEL_RR_AUX, (double)m * N, 16.0 * m * N);
-    scale_cols_f64(c.s, m, N, Y, m, w.nrm.p);
-    RC_CUDA(cudaStreamSynchronize(c.s));
+    prof::Scope ps(c.s, RCHFSI_KERNEL_RR_AUX, 3.0 * m * N, 24.0 * m * N);
+    col_norms_inv_f64(c.s, m, N, Y, m, w.nrm.p, w.info.p + 4);
+    scale_cols_f64(c.s, m, N, Y, m, w.nrm.p);  // (a bad column is reported with the Cholesky status)
   }
   double* AY = w.AY.p;
   double* BY = w.BY.p;
@@ -862,10 +848,14 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
     }
     RC_CUDA(cudaMemcpyAsync(w.Zt.p, w.GB.p, sizeof(double) * N * N, cudaMemcpyDeviceToDevice, c.s));
     cholesky_inverse_f64(c.s, N, w.GB.p, w.Lb.p, w.Li.p, w.info.p, c.num_sms, w.eigws);
-    int inf = 0;
-    RC_CUDA(cudaMemcpyAsync(&inf, w.info.p, sizeof(int), cudaMemcpyDeviceToHost, c.s));
+    int st[6] = {0};
+    RC_CUDA(cudaMemcpyAsync(st, w.info.p, sizeof(st), cudaMemcpyDeviceToHost, c.s));
     RC_CUDA(cudaStreamSynchronize(c.s));
-    return inf;
+    if (std::min(st[4], st[5]) < N) {
+      RC_CHECK(st[4] > st[5], RCHFSI_ERR_NUMERIC, "non-finite column in the filtered block");
+      throw Error(RCHFSI_ERR_ILL_CONDITIONED, "zero column in the filtered block");
+    }
+    return st[0];
   };
   grams();
   int info = factor();
@@ -917,6 +907,7 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
   }
   // eigenpairs of the projected matrix M (in Z, destroyed); eigenvectors land in `vec`
   double* vec = w.Z.p;
+  bool own_eig = false;  // sym_eig_f64 enqueued: its status is read with the final synchronisation
   {
     prof::Scope ps(c.s, RCHFSI_KERNEL_EIG, 4.0 * N * N * N, 8.0 * N * N * 2);
     if (c.p.eig_mode == RCHFSI_EIG_JACOBI) {
@@ -928,6 +919,7 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
       const OzScratch oz{&w.ozR, &w.ozE, &w.ozws, eflag, c.num_sms};
       if (sym_eig_f64(c.s, N, w.Z.p, w.Zt.p, evals, w.eigws, w.info.p + 3, c.num_sms, emu ? &oz : nullptr)) {
         vec = w.Zt.p;
+        own_eig = true;
       } else {
         RC_CUDA(cudaMemcpyAsync(w.Z.p, w.Lb.p, sizeof(double) * N * N, cudaMemcpyDeviceToDevice, c.s));
         syevd(c, N, w.Z.p, evals);
@@ -936,104 +928,121 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
       syevd(c, N, w.Z.p, evals);
     }
   }
-  // E = L^-T V
-  double* Ep = vec == w.Z.p ? w.Zt.p : w.Z.p;
-  if (small) {
-    gemm_small_f64(c.s, N, w.Li.p, N, 1, vec, 1, N, 1.0, 0.0, Ep, RCHFSI_KERNEL_SMALL_DENSE);
-  } else if (emu) {
-    oz_slice(c.s, N, N, w.Li.p, N, 1, w.ozR);  // L^-T, row i = column i of L^-1
-    oz_slice(c.s, N, N, vec, N, 1, w.ozE);     // column j of V as row j
-    oz_gemm(c.s, c.num_sms, w.ozR, w.ozE, Ep, N, w.ozws, eflag);
-  } else {
-    EpiArgs e3 = epi_store(Ep, N);
-    e3.prof_cls = RCHFSI_KERNEL_SMALL_DENSE;
-    gemm_f64(c.s, N, N, N, w.Li.p, N, true, vec, N, true, e3);
-  }
-  // X = Y E, AX = AY E, BX = BY E.  Complex problems: each complex Ritz pair appears twice; when
-  // every cluster of equal Ritz values is a pair, the first member of each is kept and only those
-  // Nc columns are rotated, then completed by J ([X_s, J X_s]); otherwise all columns are rotated
-  // and the caller selects (with complex Gram-Schmidt inside larger clusters).
-  int ncol = N;
-  const double* Erot = Ep;
-  c.rr_paired = false;
-  if (c.cplx) {
-    std::vector<double> ev(N);
-    RC_CUDA(cudaMemcpyAsync(ev.data(), evals, N * sizeof(double), cudaMemcpyDeviceToHost, c.s));
+  // From the eigenvectors `vec` of M to X, AX, BX.  Returns the device status (after synchronising):
+  // [1] library eigensolver, [2] bounded waits of the products, [3] sym_eig_f64.
+  int st[4] = {0, 0, 0, 0};
+  auto read_status = [&]() {
+    RC_CUDA(cudaMemcpyAsync(st, w.info.p, sizeof(st), cudaMemcpyDeviceToHost, c.s));
     RC_CUDA(cudaStreamSynchronize(c.s));
-    double scale = 1e-300;
-    for (double v : ev) scale = std::max(scale, std::fabs(v));
-    const double thr = 1e-9 * scale;
-    std::vector<int> sel;
-    bool pairs = true;
-    for (int k = 0; k < N && pairs;) {
-      int e = k + 1;
-      while (e < N && std::fabs(ev[e] - ev[k]) <= thr) ++e;
-      if (e - k == 2) sel.push_back(k);
-      else pairs = false;
-      k = e;
+  };
+  auto finish = [&](double* vec) {
+    // E = L^-T V
+    double* Ep = vec == w.Z.p ? w.Zt.p : w.Z.p;
+    if (small) {
+      gemm_small_f64(c.s, N, w.Li.p, N, 1, vec, 1, N, 1.0, 0.0, Ep, RCHFSI_KERNEL_SMALL_DENSE);
+    } else if (emu) {
+      oz_slice(c.s, N, N, w.Li.p, N, 1, w.ozR);  // L^-T, row i = column i of L^-1
+      oz_slice(c.s, N, N, vec, N, 1, w.ozE);     // column j of V as row j
+      oz_gemm(c.s, c.num_sms, w.ozR, w.ozE, Ep, N, w.ozws, eflag);
+    } else {
+      EpiArgs e3 = epi_store(Ep, N);
+      e3.prof_cls = RCHFSI_KERNEL_SMALL_DENSE;
+      gemm_f64(c.s, N, N, N, w.Li.p, N, true, vec, N, true, e3);
     }
-    if (pairs && (int)sel.size() == c.Nc) {
-      int* dcols = c.ccols.ensure(c.Nc);
-      RC_CUDA(cudaMemcpyAsync(dcols, sel.data(), sizeof(int) * c.Nc, cudaMemcpyHostToDevice, c.s));
-      double* Es = (Ep == w.Z.p) ? w.Zt.p : w.Z.p;  // the eigenvectors V are no longer needed
-      gather_cols_f64(c.s, N, c.Nc, Ep, dcols, Es);
-      std::vector<double> e2(N);
-      for (int j = 0; j < c.Nc; ++j) e2[j] = e2[c.Nc + j] = ev[sel[j]];
-      RC_CUDA(cudaMemcpyAsync(evals, e2.data(), N * sizeof(double), cudaMemcpyHostToDevice, c.s));
-      RC_CUDA(cudaStreamSynchronize(c.s));  // sel and e2 must outlive their copies
-      ncol = c.Nc;
-      Erot = Es;
-      c.rr_paired = true;
+    // X = Y E, AX = AY E, BX = BY E.  Complex problems: each complex Ritz pair appears twice; when
+    // every cluster of equal Ritz values is a pair, the first member of each is kept and only those
+    // Nc columns are rotated, then completed by J ([X_s, J X_s]); otherwise all columns are rotated
+    // and the caller selects (with complex Gram-Schmidt inside larger clusters).
+    int ncol = N;
+    const double* Erot = Ep;
+    c.rr_paired = false;
+    if (c.cplx) {
+      std::vector<double> ev(N);
+      RC_CUDA(cudaMemcpyAsync(ev.data(), evals, N * sizeof(double), cudaMemcpyDeviceToHost, c.s));
+      RC_CUDA(cudaStreamSynchronize(c.s));
+      double scale = 1e-300;
+      for (double v : ev) scale = std::max(scale, std::fabs(v));
+      const double thr = 1e-9 * scale;
+      std::vector<int> sel;
+      bool pairs = true;
+      for (int k = 0; k < N && pairs;) {
+        int e = k + 1;
+        while (e < N && std::fabs(ev[e] - ev[k]) <= thr) ++e;
+        if (e - k == 2) sel.push_back(k);
+        else pairs = false;
+        k = e;
+      }
+      if (pairs && (int)sel.size() == c.Nc) {
+        int* dcols = c.ccols.ensure(c.Nc);
+        RC_CUDA(cudaMemcpyAsync(dcols, sel.data(), sizeof(int) * c.Nc, cudaMemcpyHostToDevice, c.s));
+        double* Es = (Ep == w.Z.p) ? w.Zt.p : w.Z.p;  // the eigenvectors V are no longer needed
+        gather_cols_f64(c.s, N, c.Nc, Ep, dcols, Es);
+        std::vector<double> e2(N);
+        for (int j = 0; j < c.Nc; ++j) e2[j] = e2[c.Nc + j] = ev[sel[j]];
+        RC_CUDA(cudaMemcpyAsync(evals, e2.data(), N * sizeof(double), cudaMemcpyHostToDevice, c.s));
+        RC_CUDA(cudaStreamSynchronize(c.s));  // sel and e2 must outlive their copies
+        ncol = c.Nc;
+        Erot = Es;
+        c.rr_paired = true;
+      }
     }
-  }
-  // FE operators: A X and B X are applied directly (a cell product costs 2 n_c^2 C per column,
-  // below the 2 m N of rotating A Y and B Y, and gives the residual of X itself); dense operators
-  // rotate A Y and B Y (2 m N per column against 2 m^2)
-  bool direct = false;
-  if (c.op_kind == RCHFSI_OP_FE_CELL) {
-    // per column: a (complex: four) cell product(s), 2 n_c^2 C each, against the rotation's 2 m N
-    const double cell = (double)c.fe->nc * c.fe->nc * (double)c.fe->n_cells * (c.fe->cplx ? 4.0 : 1.0);
-    direct = cell < (double)m * N;
-  }
-  if (emu) {
-    // E^T as ncol logical rows (row j = column j of E, contiguous); blocks as m logical rows (dofs)
-    oz_slice(c.s, ncol, N, Erot, N, 1, w.ozE);
-    oz_slice(c.s, m, N, Y, 1, m, w.ozL);
-    oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, X, m, w.ozws, eflag);
-    if (!direct) {
-      oz_slice(c.s, m, N, AY, 1, m, w.ozL);
-      oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, AX, m, w.ozws, eflag);
-      oz_slice(c.s, m, N, BY, 1, m, w.ozL);
-      oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, BX, m, w.ozws, eflag);
+    // FE operators: A X and B X are applied directly (a cell product costs 2 n_c^2 C per column,
+    // below the 2 m N of rotating A Y and B Y, and gives the residual of X itself); dense operators
+    // rotate A Y and B Y (2 m N per column against 2 m^2)
+    bool direct = false;
+    if (c.op_kind == RCHFSI_OP_FE_CELL) {
+      // per column: a (complex: four) cell product(s), 2 n_c^2 C each, against the rotation's 2 m N
+      const double cell = (double)c.fe->nc * c.fe->nc * (double)c.fe->n_cells * (c.fe->cplx ? 4.0 : 1.0);
+      direct = cell < (double)m * N;
     }
-    int flag = 0;
-    RC_CUDA(cudaMemcpyAsync(&flag, eflag, sizeof(int), cudaMemcpyDeviceToHost, c.s));
-    RC_CUDA(cudaStreamSynchronize(c.s));
-    if (flag) {
-      RC_CUDA(cudaMemsetAsync(eflag, 0, sizeof(int), c.s));
-      throw Error(RCHFSI_ERR_TIMEOUT, "a bounded wait in the emulated FP64 GEMM ran out");
+    if (emu) {
+      // E^T as ncol logical rows (row j = column j of E, contiguous); blocks as m logical rows (dofs)
+      oz_slice(c.s, ncol, N, Erot, N, 1, w.ozE);
+      oz_slice(c.s, m, N, Y, 1, m, w.ozL);
+      oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, X, m, w.ozws, eflag);
+      if (!direct) {
+        oz_slice(c.s, m, N, AY, 1, m, w.ozL);
+        oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, AX, m, w.ozws, eflag);
+        oz_slice(c.s, m, N, BY, 1, m, w.ozL);
+        oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, BX, m, w.ozws, eflag);
+      }
+    } else {
+      gemm_f64(c.s, m, ncol, N, Y, m, false, Erot, N, true, epi_store(X, m));
+      if (!direct) {
+        gemm_f64(c.s, m, ncol, N, AY, m, false, Erot, N, true, epi_store(AX, m));
+        gemm_f64(c.s, m, ncol, N, BY, m, false, Erot, N, true, epi_store(BX, m));
+      }
     }
-  } else {
-    gemm_f64(c.s, m, ncol, N, Y, m, false, Erot, N, true, epi_store(X, m));
-    if (!direct) {
-      gemm_f64(c.s, m, ncol, N, AY, m, false, Erot, N, true, epi_store(AX, m));
-      gemm_f64(c.s, m, ncol, N, BY, m, false, Erot, N, true, epi_store(BX, m));
-    }
-  }
-  if (c.rr_paired) jcomplete(X);
-  if (direct) {
-    apply_AB_f64(c, X, AX, BX, ncol);
-    if (c.rr_paired) {
+    if (c.rr_paired) jcomplete(X);
+    if (direct) {
+      apply_AB_f64(c, X, AX, BX, ncol);
+      if (c.rr_paired) {
+        jcomplete(AX);
+        jcomplete(BX);
+      }
+    } else if (c.rr_paired) {
       jcomplete(AX);
       jcomplete(BX);
     }
-  } else if (c.rr_paired) {
-    jcomplete(AX);
-    jcomplete(BX);
+    read_status();
+  };
+  finish(vec);
+  if (own_eig && st[3] == 1) {
+    // a cluster too large for inverse iteration: the same from the library's eigenvectors
+    RC_CUDA(cudaMemcpyAsync(w.Z.p, w.Lb.p, sizeof(double) * N * N, cudaMemcpyDeviceToDevice, c.s));
+    {
+      prof::Scope ps(c.s, RCHFSI_KERNEL_EIG, 4.0 * N * N * N, 8.0 * N * N * 2);
+      syevd(c, N, w.Z.p, evals);
+    }
+    finish(w.Z.p);
+    st[3] = 0;
   }
-  RC_CUDA(cudaMemcpyAsync(&info, w.info.p + 1, sizeof(int), cudaMemcpyDeviceToHost, c.s));
-  RC_CUDA(cudaStreamSynchronize(c.s));
-  if (info != 0) return RCHFSI_ERR_NUMERIC;
+  if (st[2] || (own_eig && st[3])) {
+    RC_CUDA(cudaMemsetAsync(eflag, 0, sizeof(int), c.s));
+    throw Error(RCHFSI_ERR_TIMEOUT, st[2] ? "a bounded wait in the emulated FP64 GEMM ran out"
+                                          : "a bounded wait in the tridiagonalisation ran out");
+  }
+  if (st[1] != 0) return RCHFSI_ERR_NUMERIC;
   return RCHFSI_OK;
 }
 

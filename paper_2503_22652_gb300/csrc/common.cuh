@@ -141,7 +141,8 @@ void gemm_f32(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, i
 void transpose_f64(cudaStream_t s, int64_t rows, int64_t cols, const double* in, int64_t ldin, double* out,
                    int64_t ldout);  // out(j,i) = in(i,j), both row-major views
 void scale_cols_f64(cudaStream_t s, int64_t m, int64_t n, double* X, int64_t ld, const double* scale);
-void col_norms_f64(cudaStream_t s, int64_t m, int64_t n, const double* X, int64_t ld, double* out);
+// out[j] = 1 / ||X(:,j)||; bad[0], bad[1]: the first column with a non-finite / zero norm (0x7f7f7f7f: none)
+void col_norms_inv_f64(cudaStream_t s, int64_t m, int64_t n, const double* X, int64_t ld, double* out, int* bad);
 void scale_rows_f64(cudaStream_t s, int64_t m, int64_t n, const double* in, double* out, const double* d,
                     bool cols);  // out = diag(d)*in (cols=false) or in*diag(d) (cols=true); row-major m x n
 // o1 = (float)(s1 W), o2 = (float)(s2 W) as row-major m x n blocks, W column-major (leading dim m)
@@ -184,7 +185,9 @@ int cholesky_inverse_f64(cudaStream_t s, int n, double* A, double* L, double* Li
                          DevBuf<double>& scratch);
 // Symmetric eigensolver (small_eig.cu: Householder tridiagonalisation, bisection, inverse iteration):
 // M destroyed; V (column-major eigenvectors) and evals ascending.  Returns false when it declines the
-// problem (order > 3072 or a cluster of close eigenvalues too large for inverse iteration).
+// problem (order > 3072).  Enqueues only: *d_flag, read by the caller once the stream is synchronised, is
+// 0, 1 (V and evals are not valid: a cluster of close eigenvalues too large for inverse iteration) or 2
+// (a bounded wait ran out).
 // oz: when set, the N x N products of its orthogonalisation step run FP64-accurate on the tensor
 // cores (oz_gemm.cuh) instead of as FP64 GEMMs.
 struct OzScratch;

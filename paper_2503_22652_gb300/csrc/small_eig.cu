@@ -1953,6 +1953,7 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
   double* xch = p + n;
   double* tnorm = xch + n + 8;
   double* pkts = tnorm + 8;
+  RC_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
   if (n == 1) {
     RC_CUDA(cudaMemcpyAsync(evals, M, sizeof(double), cudaMemcpyDeviceToDevice, s));
     const double one = 1.0;
@@ -1962,7 +1963,6 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
   }
   RC_CUDA(cudaMemsetAsync(e, 0, sizeof(double) * n, s));
   RC_CUDA(cudaMemsetAsync(tau, 0, sizeof(double) * n, s));
-  RC_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
   // 1. Q^T M Q = T
   if (!launch_tridiag_xch(s, n, num_sms, M, H, d, e, tau, pkts, d_flag) &&
       !launch_resident(s, tridiag_smem_kernel<true>, tridiag_smem_kernel<false>, n, num_sms, n, (const double*)M, H,
@@ -1980,11 +1980,6 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
   set_smem_limit(reinterpret_cast<const void*>(inviter_kernel), (int)SMEM_CAP);
   inviter_kernel<<<n, 32, inviter_smem(n), s>>>(n, d, e, evals, tnorm, V2, INV_MAX_CLUSTER, pairs ? 1 : 0, d_flag);
   RC_LAUNCH();
-  int flag = 0;
-  RC_CUDA(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-  RC_CUDA(cudaStreamSynchronize(s));
-  RC_CHECK(flag != 2, RCHFSI_ERR_TIMEOUT, "a bounded wait in the tridiagonalisation ran out");
-  if (flag) return false;
   // 4. one Newton-Schulz step towards the orthogonal factor: Z <- Z (3 I - Z^T Z) / 2
   if (oz && n <= kSmallGemmMaxN) {
     // S = 1.5 I - 0.5 Z^T Z, V = Z S
