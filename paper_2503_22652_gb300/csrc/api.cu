@@ -261,8 +261,17 @@ static void dense_step_lowp(rchfsi_ctx& c, bool chfsi, int prec, const void* Ry,
   }
 }
 
+// Tables of the one-launch degree loop (tc_loop.cu), behind the Lambda table in the same upload: the
+// coefficients and Lambda values of each step in FP32 and the zeroed counters.
+struct LoopTables {
+  const float* coef = nullptr;
+  const float* lam = nullptr;
+  int* counters = nullptr;
+};
+
 static void filter_dense(rchfsi_ctx& c, const double* X, const double* W, int p, const double* lamtab, double e,
-                         double cc, double s1, const std::vector<Coef>& co, double* Y, bool chfsi) {
+                         double cc, double s1, const std::vector<Coef>& co, double* Y, bool chfsi,
+                         const TcLoopPlan& loop, const LoopTables& ls) {
   const int64_t m = c.p.m;
   const int N = c.p.block;
   const size_t blk = (size_t)m * N;
@@ -358,17 +367,29 @@ static void filter_dense(rchfsi_ctx& c, const double* X, const double* W, int p,
     if (bf) reconstruct_bf16(c.s, m, N, (const __nv_bfloat16*)R, mp, dv, X, lam, out);
     else reconstruct_f32(c.s, m, N, (const float*)R, mp, dv, X, lam, out);
   };
-  if (!chfsi) {
-    cast(W, RY, s1 / e);
-    cast(W, Wl, 1.0);
+  if (loop.ok) {
+    // every product in one launch (Algorithm 2 starts from R_1 = X, one step more)
+    void *R0 = chfsi ? RX : RY, *R1 = chfsi ? RY : RX;
+    cast(chfsi ? X : W, R0, chfsi ? 1.0 : s1 / e);
+    if (!chfsi) cast(W, Wl, 1.0);
+    const int steps = (int)co.size() + (chfsi ? 1 : 0);
+    const void* op = bf ? (const void*)dense_op16(c, chfsi) : (const void*)dense_op32(c, chfsi, true);
+    tc_loop(c.s, loop, m, N, bf, op, mp, R0, R1, chfsi ? nullptr : Wl, ls.coef, ls.lam, steps, c.w.split.p,
+            ls.counters, c.w.info.p + 2);
+    RY = steps % 2 ? R1 : R0;
   } else {
-    cast(X, RX, 1.0);
-    dense_step_lowp(c, true, prec, RX, nullptr, nullptr, nullptr, Coef{s1 / e, -(s1 / e) * cc, 0.0}, RY);
-  }
-  for (size_t k = 0; k < co.size(); ++k) {
-    dense_step_lowp(c, chfsi, prec, RY, (chfsi || k > 0) ? RX : nullptr, chfsi ? nullptr : Wl,
-                    chfsi ? nullptr : lamtab + (k + 1) * N, co[k], RX);
-    std::swap(RX, RY);
+    if (!chfsi) {
+      cast(W, RY, s1 / e);
+      cast(W, Wl, 1.0);
+    } else {
+      cast(X, RX, 1.0);
+      dense_step_lowp(c, true, prec, RX, nullptr, nullptr, nullptr, Coef{s1 / e, -(s1 / e) * cc, 0.0}, RY);
+    }
+    for (size_t k = 0; k < co.size(); ++k) {
+      dense_step_lowp(c, chfsi, prec, RY, (chfsi || k > 0) ? RX : nullptr, chfsi ? nullptr : Wl,
+                      chfsi ? nullptr : lamtab + (k + 1) * N, co[k], RX);
+      std::swap(RX, RY);
+    }
   }
   if (chfsi) {
     recon(RY, nullptr, c.w.nrm.p, Y);  // nrm holds zeros: plain upcast
@@ -489,12 +510,54 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam_host, con
   } else {
     tab.assign((size_t)(p + 1) * N, 0.0);
   }
+  // The degree loop of a dense TF32 / BF16 filter runs as one launch where the operator has at most a
+  // quarter as many row tiles as the GPU has SMs (see tc_loop_plan) and its workspace fits the budget.
+  TcLoopPlan loop;
+  LoopTables ls;
+  size_t coef_at = 0, cnt_at = 0;
+  const int loop_steps = p - 1 + (chfsi ? 1 : 0);
+  if (c.op_kind == RCHFSI_OP_DENSE && (c.p.precision == RCHFSI_TF32 || c.p.precision == RCHFSI_BF16) &&
+      loop_steps > 0) {
+    const bool bf = c.p.precision == RCHFSI_BF16;
+    if (c.w.loop.M != c.p.m || c.w.loop.N != N || c.w.loop.bf16 != bf)
+      c.w.loop = tc_loop_plan(c.num_sms, c.p.m, N, bf);
+    loop = c.w.loop;
+    if (loop.ok && c.p.hbm_budget_bytes && c.w.split.n < loop.ws_floats &&
+        device_bytes(c) - c.w.split.bytes() + loop.ws_floats * sizeof(float) > c.p.hbm_budget_bytes)
+      loop.ok = false;
+    if (loop.ok) {
+      coef_at = tab.size();
+      const size_t floats = 3 * (size_t)loop_steps + (chfsi ? 0 : (size_t)loop_steps * N);
+      cnt_at = (coef_at + (floats + 1) / 2 + 15) / 16 * 16;  // counters on 128-byte lines
+      tab.resize(cnt_at + loop.counters / 2, 0.0);
+      float* f = reinterpret_cast<float*>(tab.data() + coef_at);
+      int o = 0;
+      if (chfsi) {
+        f[o++] = (float)(s1 / e);
+        f[o++] = (float)(-(s1 / e) * cc);
+        f[o++] = 0.f;
+      }
+      for (const Coef& q : co) {
+        f[o++] = (float)q.a;
+        f[o++] = (float)q.b;
+        f[o++] = (float)q.c;
+      }
+      if (!chfsi)
+        for (size_t t = 0; t < (size_t)loop_steps * N; ++t) f[o + t] = (float)tab[(size_t)N + t];
+      c.w.split.ensure(loop.ws_floats);
+    }
+  }
   double* dtab = c.w.lamtab.ensure(tab.size());
+  if (loop.ok) {
+    ls.coef = reinterpret_cast<const float*>(dtab + coef_at);
+    ls.lam = ls.coef + 3 * (size_t)loop_steps;
+    ls.counters = reinterpret_cast<int*>(dtab + cnt_at);
+  }
   RC_CUDA(cudaMemcpyAsync(dtab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, c.s));
   // zero "lambda" vector used by reconstructions that only upcast
   RC_CUDA(cudaMemsetAsync(c.w.nrm.p, 0, sizeof(double) * N, c.s));
   if (c.op_kind == RCHFSI_OP_DENSE)
-    filter_dense(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi);
+    filter_dense(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi, loop, ls);
   else
     filter_fe(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi);
   // the host table must outlive the async copy; then read the kernels' timeout flag

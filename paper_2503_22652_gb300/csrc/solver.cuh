@@ -8,6 +8,7 @@
 #include "fe.cuh"
 #include "oz_gemm.cuh"
 #include "prof.cuh"
+#include "tc_loop.cuh"
 
 struct rchfsi_ctx;
 
@@ -25,6 +26,7 @@ struct Work {
   DevBuf<float> R32a, R32b, W32;               // low-precision filter buffers (col-major or row-major)
   DevBuf<__nv_bfloat16> R16a, R16b, W16;
   DevBuf<float> split;                         // split-K partial sums of the tensor-core product
+  TcLoopPlan loop;                             // launch shape of the dense degree loop, for its (M, N, bf16)
   DevBuf<int> info;
   DevBuf<double> lz_v, lz_w, lz_vp, lz_t, lz_ab;  // Lanczos vectors and scalars
   DevBuf<double> syev_work;
