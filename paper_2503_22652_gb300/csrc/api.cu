@@ -199,14 +199,14 @@ static void lambda_table(const double* lam, int N, double e, double cc, double s
   }
 }
 
-// Scales s_k of the iterates S_k = s_k R_k of the fused FE step (s_1 = s_2 = 1, s_k = s_{k-2} / c_k,
-// so that S_{k-2} enters step k with coefficient 1); false when one leaves [2^-60, 2^60] (the
-// unfused step is used then).
-static bool fused_scales(const std::vector<Coef>& co, std::vector<double>& sc) {
+// Scales s_k of the iterates S_k = s_k R_k of the fused FE step (s_1 = s_2 = e / sigma_1, so that S_1 = W, and
+// s_k = s_{k-2} / c_k, so that S_{k-2} enters step k with coefficient 1); false when one leaves
+// [2^-60, 2^60] (the unfused step is used then).
+static bool fused_scales(const std::vector<Coef>& co, double e_over_s1, std::vector<double>& sc) {
   const int p = (int)co.size() + 1;
-  sc.assign((size_t)p + 1, 1.0);
-  for (int k = 3; k <= p; ++k) {
-    sc[k] = sc[k - 2] / co[k - 2].c;
+  sc.assign((size_t)p + 1, e_over_s1);
+  for (int k = 1; k <= p; ++k) {
+    if (k >= 3) sc[k] = sc[k - 2] / co[k - 2].c;
     if (!std::isfinite(sc[k]) || std::fabs(sc[k]) > 0x1p60 || std::fabs(sc[k]) < 0x1p-60) return false;
   }
   return true;
@@ -271,7 +271,7 @@ struct LoopTables {
 
 static void filter_dense(rchfsi_ctx& c, const double* X, const double* W, int p, const double* lamtab, double e,
                          double cc, double s1, const std::vector<Coef>& co, double* Y, bool chfsi,
-                         const TcLoopPlan& loop, const LoopTables& ls) {
+                         const TcLoopPlan& loop, const LoopTables& ls, bool rows) {
   const int64_t m = c.p.m;
   const int N = c.p.block;
   const size_t blk = (size_t)m * N;
@@ -358,20 +358,35 @@ static void filter_dense(rchfsi_ctx& c, const double* X, const double* W, int p,
     }
   }
   check_budget(c);
-  // column-major m x N (pitch m) -> pitch mp: N "rows" of m contiguous entries
-  auto cast = [&](const double* in, void* out, double scale) {
-    if (bf) cast2d_f64_to_bf16(c.s, N, m, in, m, (__nv_bfloat16*)out, mp, scale);
-    else cast2d_f64_to_f32(c.s, N, m, in, m, (float*)out, mp, scale, 0);
+  // FP64 block -> column-major storage of pitch mp (times s1, and unscaled into o2 when given); from
+  // column-major blocks: N "rows" of m contiguous entries
+  auto enter = [&](const double* in, double scale, void* o1, void* o2) {
+    if (rows) {
+      if (bf) rows_to_cols_lowp_bf16(c.s, m, N, in, scale, (__nv_bfloat16*)o1, (__nv_bfloat16*)o2, mp);
+      else rows_to_cols_lowp_f32(c.s, m, N, in, scale, (float*)o1, (float*)o2, mp);
+      return;
+    }
+    for (void* out : {o1, o2}) {
+      if (!out) continue;
+      const double f = out == o1 ? scale : 1.0;
+      if (bf) cast2d_f64_to_bf16(c.s, N, m, in, m, (__nv_bfloat16*)out, mp, f);
+      else cast2d_f64_to_f32(c.s, N, m, in, m, (float*)out, mp, f, 0);
+    }
   };
   auto recon = [&](const void* R, const double* dv, const double* lam, double* out) {
-    if (bf) reconstruct_bf16(c.s, m, N, (const __nv_bfloat16*)R, mp, dv, X, lam, out);
-    else reconstruct_f32(c.s, m, N, (const float*)R, mp, dv, X, lam, out);
+    if (rows) {
+      if (bf) cols_to_rows_recon_bf16(c.s, m, N, (const __nv_bfloat16*)R, mp, dv, X, lam, out);
+      else cols_to_rows_recon_f32(c.s, m, N, (const float*)R, mp, dv, X, lam, out);
+    } else if (bf) {
+      reconstruct_bf16(c.s, m, N, (const __nv_bfloat16*)R, mp, dv, X, lam, out);
+    } else {
+      reconstruct_f32(c.s, m, N, (const float*)R, mp, dv, X, lam, out);
+    }
   };
   if (loop.ok) {
     // every product in one launch (Algorithm 2 starts from R_1 = X, one step more)
     void *R0 = chfsi ? RX : RY, *R1 = chfsi ? RY : RX;
-    cast(chfsi ? X : W, R0, chfsi ? 1.0 : s1 / e);
-    if (!chfsi) cast(W, Wl, 1.0);
+    enter(chfsi ? X : W, chfsi ? 1.0 : s1 / e, R0, chfsi ? nullptr : Wl);
     const int steps = (int)co.size() + (chfsi ? 1 : 0);
     const void* op = bf ? (const void*)dense_op16(c, chfsi) : (const void*)dense_op32(c, chfsi, true);
     tc_loop(c.s, loop, m, N, bf, op, mp, R0, R1, chfsi ? nullptr : Wl, ls.coef, ls.lam, steps, c.w.split.p,
@@ -379,10 +394,9 @@ static void filter_dense(rchfsi_ctx& c, const double* X, const double* W, int p,
     RY = steps % 2 ? R1 : R0;
   } else {
     if (!chfsi) {
-      cast(W, RY, s1 / e);
-      cast(W, Wl, 1.0);
+      enter(W, s1 / e, RY, Wl);
     } else {
-      cast(X, RX, 1.0);
+      enter(X, 1.0, RX, nullptr);
       dense_step_lowp(c, true, prec, RX, nullptr, nullptr, nullptr, Coef{s1 / e, -(s1 / e) * cc, 0.0}, RY);
     }
     for (size_t k = 0; k < co.size(); ++k) {
@@ -409,8 +423,9 @@ static void filter_dense(rchfsi_ctx& c, const double* X, const double* W, int p,
   c.last_applies = (int64_t)co.size() + (chfsi ? 1 : 0);
 }
 
+// rows: X, W and Y are row-major, as callers hold them, instead of column-major (not with FP64).
 static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, const double* lamtab, double e,
-                      double cc, double s1, const std::vector<Coef>& co, double* Y, bool chfsi) {
+                      double cc, double s1, const std::vector<Coef>& co, double* Y, bool chfsi, bool rows) {
   const int64_t m = c.p.m;
   const int N = c.p.block;
   const size_t blk = (size_t)m * N;
@@ -444,16 +459,25 @@ static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, co
   }
   RC_CHECK(prec == RCHFSI_FP32 || prec == RCHFSI_TF32 || prec == RCHFSI_BF16, RCHFSI_ERR_INVALID_ARG,
            "bad precision");
+  // FP64 block -> row-major FP32 (times s, and unscaled), and D^-1 rs R + X Lambda -> Y
+  auto enter = [&](const double* in, double sc1, float* o1, float* o2) {
+    if (rows) rows_f32x2(c.s, m, N, in, sc1, 1.0, o1, o2);
+    else cols_to_rows_f32x2(c.s, m, N, in, sc1, 1.0, o1, o2);
+  };
+  auto leave = [&](const float* R, double rs, const double* dinv, const double* lam) {
+    if (rows) rows_recon(c.s, m, N, R, rs, dinv, X, lam, Y);
+    else rows_to_cols_recon(c.s, m, N, R, rs, dinv, X, lam, Y);
+  };
   std::vector<double> sc;
-  if (!chfsi && fe_step_supported(f, N, prec) && fused_scales(co, sc)) {
+  if (!chfsi && fe_step_supported(f, N, prec) && fused_scales(co, e / s1, sc)) {
     // fused degree steps on scaled iterates: one tensor-core launch per step does the cell products,
     // the recurrence terms and the update of R_X
     float* RX = c.w.R32a.ensure(blk);
     float* RY = c.w.R32b.ensure(blk);
     float* Wl = c.w.W32.ensure(blk);
     check_budget(c);
-    // S_1 = R_1 = (sigma_1 / e) W and W, row-major FP32, in one pass over the column-major W
-    cols_to_rows_f32x2(c.s, m, N, W, s1 / e, 1.0, RY, Wl);
+    // S_1 = W and W, row-major FP32, in one pass over W
+    enter(W, 1.0, RY, Wl);
     fill_zero(c.s, RX, blk * sizeof(float));  // S_0 = R_0 = 0
     if (!co.empty()) {
       float* lamf = c.w.lamtab_f.ensure((size_t)(p + 1) * N);  // the Lambda table in FP32 for the kernel
@@ -469,8 +493,8 @@ static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, co
         std::swap(RX, RY);
       }
     }
-    // Y = D^-1 R_p + X Lambda_p with R_p = S_p / s_p, in one pass back to column-major
-    rows_to_cols_recon(c.s, m, N, RY, 1.0 / sc[p], f.Dinv.p, X, lamtab + (size_t)p * N, Y);
+    // Y = D^-1 R_p + X Lambda_p with R_p = S_p / s_p, in one pass
+    leave(RY, 1.0 / sc[p], f.Dinv.p, lamtab + (size_t)p * N);
     c.last_applies = (int64_t)co.size();
     return;
   }
@@ -479,9 +503,9 @@ static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, co
   float* Wl = c.w.W32.ensure(blk);
   check_budget(c);
   if (!chfsi) {
-    cols_to_rows_f32x2(c.s, m, N, W, s1 / e, 1.0, RY, Wl);
+    enter(W, s1 / e, RY, Wl);
   } else {
-    cols_to_rows_f32x2(c.s, m, N, X, 1.0, 1.0, RX, RX);
+    enter(X, 1.0, RX, RX);
     recur_terms_rows_f32(c.s, m, N, RX, RY, nullptr, nullptr, 0.0, -(s1 / e) * cc, 0.0);
     fe_filter_product_f32(c.s, f, prec, RX, RY, N, (float)(s1 / e), 2);
   }
@@ -493,12 +517,16 @@ static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, co
     std::swap(RX, RY);
   }
   // Y = D^-1 R_p + X Lambda_p (Algorithm 3), or Y = R_p (Algorithm 2: no D^-1, zero Lambda)
-  rows_to_cols_recon(c.s, m, N, RY, 1.0, chfsi ? nullptr : f.Dinv.p, X, chfsi ? c.w.nrm.p : lamtab + (size_t)p * N, Y);
+  leave(RY, 1.0, chfsi ? nullptr : f.Dinv.p, chfsi ? c.w.nrm.p : lamtab + (size_t)p * N);
   c.last_applies = (int64_t)co.size() + (chfsi ? 1 : 0);
 }
 
+bool filter_takes_rows(const rchfsi_ctx& c) {
+  return !c.cplx && c.p.precision != RCHFSI_FP64 && !(c.op_kind == RCHFSI_OP_DENSE && c.dense.has_dinv_dense);
+}
+
 void filter_internal(rchfsi_ctx& c, const double* X, const double* lam_host, const double* W, double lmin, double lT,
-                     double lmax, int p, double* Y, bool chfsi) {
+                     double lmax, int p, double* Y, bool chfsi, bool rows) {
   check_bounds(lmin, lT, lmax, p);
   const int N = c.p.block;
   double e, cc, s1;
@@ -557,9 +585,9 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam_host, con
   // zero "lambda" vector used by reconstructions that only upcast
   RC_CUDA(cudaMemsetAsync(c.w.nrm.p, 0, sizeof(double) * N, c.s));
   if (c.op_kind == RCHFSI_OP_DENSE)
-    filter_dense(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi, loop, ls);
+    filter_dense(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi, loop, ls, rows);
   else
-    filter_fe(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi);
+    filter_fe(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi, rows);
   // the host table must outlive the async copy; then read the kernels' timeout flag
   int flag = 0;
   RC_CUDA(cudaMemcpyAsync(&flag, c.w.info.p + 2, sizeof(int), cudaMemcpyDeviceToHost, c.s));
@@ -657,7 +685,7 @@ void filter_fe_batch(cudaStream_t s, int num_sms, std::vector<FeFilterJob>& jobs
     const int n = c.cplx ? c.Nc : c.p.block;
     double e, cc, s1;
     filter_scalars(jobs[q].lmin, jobs[q].lT, jobs[q].lmax, p, e, cc, s1, cos[q]);
-    fused = fused && fe_step_supported(*c.fe, n, prec) && fused_scales(cos[q], scales[q]);
+    fused = fused && fe_step_supported(*c.fe, n, prec) && fused_scales(cos[q], e / s1, scales[q]);
   }
   // 1. per problem: scalars, Lambda table and coefficient table on the device, initial blocks
   for (int q = 0; q < nj; ++q) {
@@ -690,7 +718,7 @@ void filter_fe_batch(cudaStream_t s, int num_sms, std::vector<FeFilterJob>& jobs
     RX[q] = c.w.R32a.ensure(blk);
     RY[q] = c.w.R32b.ensure(blk);
     WL[q] = c.w.W32.ensure(blk);
-    cols_to_rows_f32x2(s, m, n, J.W, s1 / e, 1.0, RY[q], WL[q]);
+    cols_to_rows_f32x2(s, m, n, J.W, fused ? 1.0 : s1 / e, 1.0, RY[q], WL[q]);
     fill_zero(s, RX[q], blk * sizeof(float));
     if (fused) {
       fe_step_prepare(s, *c.fe);

@@ -151,6 +151,20 @@ void cols_to_rows_f32x2(cudaStream_t s, int64_t m, int64_t n, const double* W, d
 // Y = dinv .* (rs R) + X diag(lam), R row-major float m x n, X and Y column-major (leading dim m)
 void rows_to_cols_recon(cudaStream_t s, int64_t m, int64_t n, const float* R, double rs, const double* dinv,
                         const double* X, const double* lam, double* Y);
+// The same two with W, X and Y row-major (Y may be X).
+void rows_f32x2(cudaStream_t s, int64_t m, int64_t n, const double* W, double s1, double s2, float* o1, float* o2);
+void rows_recon(cudaStream_t s, int64_t m, int64_t n, const float* R, double rs, const double* dinv, const double* X,
+                const double* lam, double* Y);
+// Dense filter with row-major callers' blocks: o1 = s1 W and o2 = W (may be null) column-major of pitch ld; and
+// Y = dinv .* R + X diag(lam), R column-major of pitch ldr, X and Y row-major (Y may be X).
+void rows_to_cols_lowp_f32(cudaStream_t s, int64_t m, int64_t n, const double* W, double s1, float* o1, float* o2,
+                           int64_t ld);
+void rows_to_cols_lowp_bf16(cudaStream_t s, int64_t m, int64_t n, const double* W, double s1, __nv_bfloat16* o1,
+                            __nv_bfloat16* o2, int64_t ld);
+void cols_to_rows_recon_f32(cudaStream_t s, int64_t m, int64_t n, const float* R, int64_t ldr, const double* dinv,
+                            const double* X, const double* lam, double* Y);
+void cols_to_rows_recon_bf16(cudaStream_t s, int64_t m, int64_t n, const __nv_bfloat16* R, int64_t ldr,
+                             const double* dinv, const double* X, const double* lam, double* Y);
 void cast_f64_to_f32(cudaStream_t s, int64_t n, const double* in, float* out, double scale, int round_tf32);
 void cast_f64_to_bf16(cudaStream_t s, int64_t n, const double* in, __nv_bfloat16* out, double scale);
 void cast_f32_to_f64(cudaStream_t s, int64_t n, const float* in, double* out, double scale = 1.0);
@@ -172,7 +186,7 @@ void cast2d_f64_to_bf16(cudaStream_t s, int64_t rows, int64_t cols, const double
 // Recurrence update without a product (for FE: Rx = b*Ry + c*Rx + a*W*lam), generic storage
 void recur_axpby_f32(cudaStream_t s, int64_t m, int64_t n, const float* Ry, float* Rx, const float* W,
                      const double* lam, double a, double b, double c);
-// Residual-norm helpers
+// Column 2-norms of W and, when given, of X
 void resid_rel_norms(cudaStream_t s, int64_t m, int64_t n, const double* W, const double* X, double* out_abs,
                      double* out_xnorm);
 

@@ -1,11 +1,14 @@
-"""The one-launch degree loop of the dense filter at the sizes where its tiles and shares have edges, against the
-oracle on equally rounded operands.  Tolerances are those of the reduced-precision parity tests (FP32 accumulation
-and storage amplified over the degree)."""
+"""The one-launch degree loop of the dense filter and the row-major entry of the filters, at the sizes where
+their tiles and shares have edges, against the oracle on equally rounded operands.  Tolerances are
+those of the reduced-precision parity tests (FP32 accumulation and storage amplified over the degree)."""
 import numpy as np
 import pytest
 
+import workloads as wl
 from gpu_helpers import dense_case, ensure_built, lowp_reference, make_solver
 from oracle.filters import lambda_p
+
+from paper_2503_22652_gb300 import Solver
 
 pytestmark = pytest.mark.gpu
 
@@ -32,3 +35,49 @@ def test_loop_matches_reference(m, N, prec, p):
     for _ in range(2):  # the second call finds used workspaces
         got = s.filter(case["X"], case["L"], case["W"], lmin, lT, lmax, p)
         assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref - base)
+
+
+def _overlaps(s, X, L, W, args):
+    """The result written over X, over W and over an array that overlaps X shifted by a row."""
+    torch = pytest.importorskip("torch")
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    ref = s.filter(dev(X), dev(L), dev(W), *args).cpu().numpy()
+    for which in ("X", "W", "shifted"):
+        x, w = dev(X), dev(W)
+        out = {"X": x, "W": w}.get(which)
+        if out is None:
+            both = torch.empty((X.shape[0] + 1, X.shape[1]), dtype=torch.float64, device="cuda")
+            x = both[:-1].copy_(x)
+            out = both[1:]
+        s.filter(x, dev(L), w, *args, out=out)
+        yield ref, out.cpu().numpy()
+
+
+def test_output_may_overlap_inputs_dense():
+    case = dense_case(m=200, N=23)
+    s = make_solver(case, 23, precision="tf32")
+    for ref, got in _overlaps(s, case["X"], case["L"], case["W"], (*case["bounds"], 6)):
+        assert np.array_equal(ref, got)
+
+
+# (tolerances of the reduced-precision FE filter parity tests; two runs differ in the order of the cell sums, and
+# a TF32 or BF16 rounding that flips is no smaller than that of a single product)
+@pytest.mark.parametrize("N,prec,tol", [(24, "tf32", 5e-3), (41, "tf32", 5e-3), (130, "tf32", 5e-3), (41, "bf16", 5e-2)])
+def test_output_may_overlap_inputs_fe(N, prec, tol):
+    from oracle import fe as ofe, filters
+    q = wl.fe_problem(2)
+    A = ofe.assemble(q["cell_dofs"], q["A_cells"], q["m"])
+    B = ofe.assemble(q["cell_dofs"], q["B_cell"], q["m"])
+    d = q["Dinv"]
+    rng = np.random.default_rng(5)
+    X = rng.standard_normal((q["m"], N))
+    L = np.sort(rng.uniform(-20.0, 30.0, N))
+    W = A @ X - (B @ X) * L[None, :]
+    args = (-25.0, 40.0, 2500.0, 8)
+    exact = filters.rchfsi_filter(lambda R: A @ (d[:, None] * R), lambda R: d[:, None] * R, X, L, W, *args)
+    base = X * lambda_p(L, *args)[None, :]
+    s = Solver(q["m"], nev=N // 2, block=N, precision=prec)
+    s.set_fe(q["cell_dofs"], q["A_cells"], q["B_cell"], q["Dinv"])
+    for ref, got in _overlaps(s, X, L, W, args):
+        for y in (ref, got):
+            assert np.linalg.norm(y - exact) <= tol * np.linalg.norm(exact - base)
