@@ -112,28 +112,37 @@ __global__ void pack_slices_kernel(int64_t n_cells, int nc, const double* __rest
     const int r = (int)((e / kNCP) % kNCP), k = (int)(e % kNCP);
     int ea = rexp[c * kNCP + r];
     if (ea == -100000) ea = 0;
-    long long f = (r < nc && k < nc) ? fixed56(A[(c * nc + r) * nc + k], ea) : 0;
+    float t[S];
+    digits7((r < nc && k < nc) ? fixed56(A[(c * nc + r) * nc + k], ea) : 0, t);
     uint8_t* base = img + c * (int64_t)S * kASlice + sw_off2(r, k, kNCP);
 #pragma unroll
     for (int s = 0; s < S; ++s)
-      *reinterpret_cast<__nv_bfloat16*>(base + (size_t)s * kASlice) = __float2bfloat16_rn((float)(int)next_digit(f, s));
+      *reinterpret_cast<__nv_bfloat16*>(base + (size_t)s * kASlice) = __float2bfloat16_rn(t[s]);
   }
 }
 
 // Column exponents of a column-major m x n block X (leading dimension m): one block per column,
-// cexp[j] = the largest exponent in column j (-100000 for a zero column).
-__global__ void __launch_bounds__(256) colexp_cols_kernel(int64_t m, const double* __restrict__ X, int* cexp) {
-  __shared__ int red[8];
+// cexp[j] = the largest exponent in column j (-100000 for a zero column).  1024 threads with four loads
+// each in flight: with 256 threads and one load, 203 columns of 64000 took 78 us, latency-bound.
+__global__ void __launch_bounds__(1024) colexp_cols_kernel(int64_t m, const double* __restrict__ X, int* cexp) {
+  __shared__ int red[32];
   const double* col = X + (int64_t)blockIdx.x * m;
   int e = -100000;
-  for (int64_t i = threadIdx.x; i < m; i += blockDim.x) e = max(e, exp_of(col[i]));
+  int64_t i = threadIdx.x;
+  for (; i + 3 * 1024 < m; i += 4 * 1024) {
+    double v[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    for (int u = 0; u < 4; ++u) v[u] = col[i + u * 1024];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) e = max(e, exp_of(v[u]));
+  }
+  for (; i < m; i += 1024) e = max(e, exp_of(col[i]));
+  e = __reduce_max_sync(0xffffffffu, e);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) e = max(e, red[w]);
-    cexp[blockIdx.x] = e;
+  if (threadIdx.x < 32) {
+    e = __reduce_max_sync(0xffffffffu, red[threadIdx.x]);
+    if (threadIdx.x == 0) cexp[blockIdx.x] = e;
   }
 }
 
@@ -187,35 +196,37 @@ __global__ void __launch_bounds__(256) fixed_to_cols_kernel(int64_t m, int n, in
 
 // The 7 slice planes of a column-major m x n block X (leading dimension m): plane t holds the
 // digits u_t as BF16, row-major with np >= n columns (np a multiple of 64, columns n .. np-1 zero),
-// so that every dof row of a column tile is one aligned 128-byte run.  32 x 32 tiles through shared
-// memory: reads coalesced along the rows of X, writes along the columns of the planes.
+// so that every dof row of a column tile is one aligned 128-byte run.  Tiles of 32 rows x 64 columns
+// through shared memory: reads coalesced along the rows of X, writes of whole 128-byte runs.
 __global__ void __launch_bounds__(256) xslice_cols_kernel(int64_t m, int n, int np, const double* __restrict__ X,
                                                           const int* __restrict__ cexp,
                                                           __nv_bfloat16* __restrict__ planes) {
-  __shared__ double tile[32][33];
+  __shared__ double tile[64][33];
   const int64_t i0 = (int64_t)blockIdx.x * 32;
-  const int j0 = blockIdx.y * 32;
+  const int j0 = blockIdx.y * 64;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-  for (int c = ty; c < 32; c += 8) {
-    const int j = j0 + c;
+#pragma unroll
+  for (int c = 0; c < 64; c += 8) {
+    const int j = j0 + c + ty;
     const int64_t i = i0 + tx;
-    tile[c][tx] = (j < n && i < m) ? X[(int64_t)j * m + i] : 0.0;
+    tile[c + ty][tx] = (j < n && i < m) ? X[(int64_t)j * m + i] : 0.0;
   }
   __syncthreads();
-  const int j = j0 + tx;
-  int e = (j < n) ? cexp[j] : 0;
-  if (e == -100000) e = 0;
+  const int j = j0 + 2 * tx;
+  int e0 = (j < n) ? cexp[j] : 0, e1 = (j + 1 < n) ? cexp[j + 1] : 0;
+  if (e0 == -100000) e0 = 0;
+  if (e1 == -100000) e1 = 0;
   const int64_t pstride = m * (int64_t)np;
-  for (int r = ty; r < 32; r += 8) {
-    const int64_t i = i0 + r;
-    if (i >= m) break;
-    long long f = fixed56(tile[tx][r], e);
-    __nv_bfloat16* dst = planes + i * np + j;
 #pragma unroll
-    for (int t = 0; t < S; ++t) {
-      // |digit| <= 256: converted through int (a 64-bit integer conversion uses the FP64 pipe)
-      dst[(int64_t)t * pstride] = __float2bfloat16_rn((float)(int)next_digit(f, t));
-    }
+  for (int rr = 0; rr < 32; rr += 8) {
+    const int64_t i = i0 + rr + ty;
+    if (i >= m) break;
+    float t0[S], t1[S];
+    digits7(fixed56(tile[2 * tx][rr + ty], e0), t0);
+    digits7(fixed56(tile[2 * tx + 1][rr + ty], e1), t1);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(planes + i * np + j);
+#pragma unroll
+    for (int t = 0; t < S; ++t) dst[(int64_t)t * (pstride / 2)] = bf16_pair(t0[t], t1[t]);
   }
 }
 
@@ -679,9 +690,9 @@ void fe_apply_f64_cols_tc(cudaStream_t s, const FeOp& op, const double* X, doubl
   __nv_bfloat16* planes = op.ozplanes.ensure((size_t)S * total);
   {
     prof::Scope ps(s, RCHFSI_KERNEL_RR_AUX, 0.0, 16.0 * m * n + 14.0 * (double)total);
-    colexp_cols_kernel<<<(unsigned)n, 256, 0, s>>>(m, X, cexp);
+    colexp_cols_kernel<<<(unsigned)n, 1024, 0, s>>>(m, X, cexp);
     RC_LAUNCH();
-    xslice_cols_kernel<<<dim3(cdiv(m, 32), (unsigned)(np / 32)), 256, 0, s>>>(m, n, np, X, cexp, planes);
+    xslice_cols_kernel<<<dim3(cdiv(m, 32), (unsigned)(np / 64)), 256, 0, s>>>(m, n, np, X, cexp, planes);
     RC_LAUNCH();
   }
   const int64_t mrow = op.cplx ? op.mc : m;

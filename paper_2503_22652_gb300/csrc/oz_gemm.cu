@@ -108,24 +108,14 @@ __global__ void slice_kernel(int64_t R, int64_t Rp, int64_t K, int64_t Kp, const
       e = 0;
       if (k0 == 0 && tx == 0) ex[r] = 0;
     }
-    // digits t_s of x 2^(-e) = sum_s t_s 2^(-8(s+1)), rounded to nearest: |t_0| <= 256, |t_s| <= 128,
-    // each exact in BF16; two neighbouring k per thread, stored as one 4-byte pair per slice
-    long long f0 = fixed56(tile[rr][2 * tx], e), f1 = fixed56(tile[rr][2 * tx + 1], e);
-    __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(out + (int64_t)r * Kp + k0 + 2 * tx);
+    // digits t_s of x 2^(-e) = sum_s t_s 2^(-8(s+1)): |t_0| <= 256, |t_s| <= 128, each exact in BF16; two
+    // neighbouring k per thread, stored as one 4-byte pair per slice
+    float t0[S], t1[S];
+    digits7(fixed56(tile[rr][2 * tx], e), t0);
+    digits7(fixed56(tile[rr][2 * tx + 1], e), t1);
+    uint32_t* o2 = reinterpret_cast<uint32_t*>(out + (int64_t)r * Kp + k0 + 2 * tx);
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const int sh = 48 - 8 * s;
-      long long t0 = f0, t1 = f1;
-      if (sh > 0) {
-        t0 = (f0 + (1LL << (sh - 1))) >> sh;
-        t1 = (f1 + (1LL << (sh - 1))) >> sh;
-        f0 -= t0 << sh;
-        f1 -= t1 << sh;
-      }
-      // digits fit in 32 bits (|t| <= 256): an int conversion stays off the FP64 pipe, which a
-      // 64-bit integer conversion occupies (a few DFMA per clock per SM on this GPU)
-      o2[(int64_t)s * Rp * Kp / 2] = __floats2bfloat162_rn((float)(int)t0, (float)(int)t1);
-    }
+    for (int s = 0; s < S; ++s) o2[(int64_t)s * Rp * Kp / 2] = bf16_pair(t0[s], t1[s]);
   }
 }
 
@@ -186,15 +176,13 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(int RB, int64_t R, int6
     const int rr = t / segs, k = (t - rr * segs) * KC + 2 * lane;
     const int64_t r = r0 + rr;
     if (r >= Rp) break;
-    __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(out + r * Kp + k);
+    uint32_t* o2 = reinterpret_cast<uint32_t*>(out + r * Kp + k);
     const int e = rex[rr] == -100000 ? 0 : rex[rr];
-    long long f0 = r < R && k < K ? fixed56(tile[rr * ld + k], e) : 0;
-    long long f1 = r < R && k + 1 < K ? fixed56(tile[rr * ld + k + 1], e) : 0;
+    float t0[S], t1[S];
+    digits7(r < R && k < K ? fixed56(tile[rr * ld + k], e) : 0, t0);
+    digits7(r < R && k + 1 < K ? fixed56(tile[rr * ld + k + 1], e) : 0, t1);
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const long long t0 = next_digit(f0, s), t1 = next_digit(f1, s);
-      o2[(int64_t)s * Rp * Kp / 2] = __floats2bfloat162_rn((float)(int)t0, (float)(int)t1);
-    }
+    for (int s = 0; s < S; ++s) o2[(int64_t)s * Rp * Kp / 2] = bf16_pair(t0[s], t1[s]);
   }
 }
 
