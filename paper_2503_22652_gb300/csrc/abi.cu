@@ -604,7 +604,7 @@ void run_begin(SolveRun& r) {
   lanczos(c, c.w.Y.p, p.lanczos_steps, p.fixed_bounds ? nullptr : &r.lmax, &r.normA);
   RC_CHECK(r.normA > 0.0 && std::isfinite(r.normA), RCHFSI_ERR_NUMERIC, "||A|| estimate is not positive");
   const auto tr = std::chrono::steady_clock::now();
-  r.rc = rayleigh_ritz(c, c.w.Y.p, c.w.X.p, c.w.AX.p, c.w.BX.p, c.w.evals.p);
+  r.rc = rayleigh_ritz(c, c.w.Y.p, c.w.X.p, true, c.w.evals.p);
   r.retries += c.rr_retries;
   pair_after_rr(r);
   r.t_rr += ms_since(tr);
@@ -673,7 +673,7 @@ void run_filter_single(SolveRun& r) {
 void run_rr(SolveRun& r) {
   rchfsi_ctx& c = *r.h;
   const auto tr = std::chrono::steady_clock::now();
-  r.rc = rayleigh_ritz(c, c.w.Y.p, c.w.X.p, c.w.AX.p, c.w.BX.p, c.w.evals.p);
+  r.rc = rayleigh_ritz(c, c.w.Y.p, c.w.X.p, true, c.w.evals.p);
   r.retries += c.rr_retries;
   pair_after_rr(r);
   r.t_rr += ms_since(tr);
@@ -1063,7 +1063,7 @@ int rchfsi_rayleigh_ritz(rchfsi_ctx* h, const double* Y, double* X, double* eval
     need_op(h);
     rchfsi_ctx& c = *h;
     load_any(c, Y, c.w.Y.p);
-    const int rc = rayleigh_ritz(c, c.w.Y.p, c.w.X.p, c.w.AX.p, c.w.BX.p, c.w.evals.p);
+    const int rc = rayleigh_ritz(c, c.w.Y.p, c.w.X.p, false, c.w.evals.p);
     if (rc != RCHFSI_OK) return rc;
     if (c.cplx && !c.rr_paired) {
       std::vector<double> ev = host_vec(c, c.w.evals.p, c.p.block);

@@ -867,7 +867,7 @@ void filter_fe_batch(cudaStream_t s, int num_sms, std::vector<FeFilterJob>& jobs
            RCHFSI_ERR_CUDA, "syevd failed");
 }
 
-int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, double* evals) {
+int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* evals) {
   const int64_t m = c.p.m;
   const int N = c.p.block;
   Work& w = c.w;
@@ -877,6 +877,7 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
     col_norms_inv_f64(c.s, m, N, Y, m, w.nrm.p, w.info.p + 4);
     scale_cols_f64(c.s, m, N, Y, m, w.nrm.p);  // (a bad column is reported with the Cholesky status)
   }
+  double *AX = w.AX.p, *BX = w.BX.p;
   double* AY = w.AY.p;
   double* BY = w.BY.p;
   const bool emu = c.p.rr_mode == RCHFSI_RR_FP64_EMULATED;
@@ -1080,6 +1081,8 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
     // FE operators: A X and B X are applied directly (a cell product costs 2 n_c^2 C per column,
     // below the 2 m N of rotating A Y and B Y, and gives the residual of X itself); dense operators
     // rotate A Y and B Y (2 m N per column against 2 m^2)
+    // (complex vectors not yet paired: the caller's selection inside clusters needs B X)
+    const bool want = products || (c.cplx && !c.rr_paired);
     bool direct = false;
     if (c.op_kind == RCHFSI_OP_FE_CELL) {
       // per column: a (complex: four) cell product(s), 2 n_c^2 C each, against the rotation's 2 m N
@@ -1091,7 +1094,7 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
       oz_slice(c.s, ncol, N, Erot, N, 1, w.ozE);
       oz_slice(c.s, m, N, Y, 1, m, w.ozL);
       oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, X, m, w.ozws, eflag);
-      if (!direct) {
+      if (want && !direct) {
         oz_slice(c.s, m, N, AY, 1, m, w.ozL);
         oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, AX, m, w.ozws, eflag);
         oz_slice(c.s, m, N, BY, 1, m, w.ozL);
@@ -1099,19 +1102,19 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, d
       }
     } else {
       gemm_f64(c.s, m, ncol, N, Y, m, false, Erot, N, true, epi_store(X, m));
-      if (!direct) {
+      if (want && !direct) {
         gemm_f64(c.s, m, ncol, N, AY, m, false, Erot, N, true, epi_store(AX, m));
         gemm_f64(c.s, m, ncol, N, BY, m, false, Erot, N, true, epi_store(BX, m));
       }
     }
     if (c.rr_paired) jcomplete(X);
-    if (direct) {
+    if (want && direct) {
       apply_AB_f64(c, X, AX, BX, ncol);
       if (c.rr_paired) {
         jcomplete(AX);
         jcomplete(BX);
       }
-    } else if (c.rr_paired) {
+    } else if (want && c.rr_paired) {
       jcomplete(AX);
       jcomplete(BX);
     }

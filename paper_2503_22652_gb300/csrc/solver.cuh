@@ -101,8 +101,9 @@ bool filter_takes_rows(const rchfsi_ctx& c);
 void filter_internal(rchfsi_ctx& c, const double* X, const double* lam_host, const double* W, double lmin,
                      double lT, double lmax, int p, double* Y, bool chfsi, bool rows = false);
 
-// Rayleigh-Ritz on column-major Y (scaled in place): X, AX, BX, evals (device) are outputs.
-int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, double* AX, double* BX, double* evals);
+// Rayleigh-Ritz on column-major Y (scaled in place): X and evals (device) are outputs, and with `products`
+// also A X and B X in c.w.AX and c.w.BX (a solve's residuals; a single call has no use for them).
+int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* evals);
 
 // Lanczos bounds (host results).
 void lanczos(rchfsi_ctx& c, const double* v0_dev, int k, double* lmax, double* normA);
