@@ -1043,6 +1043,20 @@ int rchfsi_residual(rchfsi_ctx* h, const double* X, const double* Lambda, double
     const int64_t m = c.p.m;
     // a complex block needs only the first N embedded columns
     const int N = c.cplx ? c.Nc : c.p.block;
+    if (c.op_kind == RCHFSI_OP_FE_CELL && !c.cplx && c.p.rr_mode == RCHFSI_RR_FP64_EMULATED) {
+      const size_t blk = (size_t)m * N;
+      const double* Xd = rows_block(c, X, c.w.X.p);
+      const std::vector<double> lam = lam_any(c, Lambda);
+      RC_CUDA(cudaMemcpyAsync(c.w.evals.p, lam.data(), N * sizeof(double), cudaMemcpyHostToDevice, c.s));
+      // (X is read before W is written, so they may overlap)
+      double* Wd = is_device_pointer(W) ? W : c.w.W.p;
+      fe_residual_rows_tc(c.s, *c.fe, Xd, c.w.evals.p, N, c.num_sms, c.w.stage_in.ensure(blk),
+                          c.w.stage_out.ensure(blk), c.w.ozws, Wd, c.w.rabs.p);
+      if (W && Wd != W) from_device(c, Wd, W, blk);
+      from_device(c, c.w.rabs.p, rnorm, N);
+      RC_CUDA(cudaStreamSynchronize(c.s));
+      return RCHFSI_OK;
+    }
     load_any(c, X, c.w.X.p);
     const std::vector<double> lam = lam_any(c, Lambda);
     RC_CUDA(cudaMemcpyAsync(c.w.evals.p, lam.data(), N * sizeof(double), cudaMemcpyHostToDevice, c.s));
@@ -1050,7 +1064,7 @@ int rchfsi_residual(rchfsi_ctx* h, const double* X, const double* Lambda, double
     resid_form_f64(c.s, m, N, c.w.AX.p, c.w.BX.p, c.w.evals.p, c.w.W.p);
     store_any(c, c.w.W.p, W);
     if (rnorm) {
-      resid_rel_norms(c.s, m, N, c.w.W.p, c.w.X.p, c.w.rabs.p, c.w.xnrm.p);
+      resid_rel_norms(c.s, m, N, c.w.W.p, nullptr, c.w.rabs.p, nullptr);
       from_device(c, c.w.rabs.p, rnorm, N);
     }
     RC_CUDA(cudaStreamSynchronize(c.s));

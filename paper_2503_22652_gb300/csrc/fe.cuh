@@ -56,6 +56,11 @@ void fe_apply_f64_rows(cudaStream_t s, const FeOp& op, bool useB, const double* 
 void fe_apply_f64_cols_tc(cudaStream_t s, const FeOp& op, const double* X, double* AX, double* BX, int n,
                           int num_sms, double* accA, double* accB);
 
+// W = A X - B X diag(lam) and the 2-norms of its columns for row-major X and W (real operators): the
+// accumulators become W directly, without A X, B X and their layout changes.  part: partial sums (grown as needed).
+void fe_residual_rows_tc(cudaStream_t s, const FeOp& op, const double* X, const double* lam, int n, int num_sms,
+                         double* accA, double* accB, DevBuf<double>& part, double* W, double* norms);
+
 // Filter product for FE operators on row-major m x n blocks, accumulated into Rx (the
 // product-free recurrence terms are applied to Rx beforehand):
 //   dmode 0: Rx += a * A Ry,  1: Rx += a * A D^-1 Ry (Algorithm 3),  2: Rx += a * D^-1 A Ry (Algorithm 2)

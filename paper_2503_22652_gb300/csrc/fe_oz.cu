@@ -161,10 +161,11 @@ __global__ void rowexp_kernel(int64_t n_cells, int nc, const int* __restrict__ d
 // Value of accumulator entry (row i, column j): V 2^(rowexp(dof) + cexp(j) + H - 62), with
 // dof = i mod mrow (the two halves of a complex embedding share the dof's scale; m <= 2 mrow).  An exponent
 // above the FP64 range marks a non-finite input in that row of a cell matrix or column of X.
+template <bool INT = false>
 __device__ __forceinline__ double fixed_value(long long V, int er, int ec, int H) {
   if (er > 1024 || ec > 1024) return __longlong_as_double(0x7ff8000000000000LL);
   if (V == 0) return 0.0;
-  return fixed_to_f64(V, er + ec + H - 62);
+  return INT ? fixed_to_f64_int(V, er + ec + H - 62) : fixed_to_f64(V, er + ec + H - 62);
 }
 
 // Fixed-point accumulator (row-major m x n) -> FP64 column-major Ycol (leading dimension m), through
@@ -228,6 +229,119 @@ __global__ void __launch_bounds__(256) xslice_cols_kernel(int64_t m, int n, int 
 #pragma unroll
     for (int t = 0; t < S; ++t) dst[(int64_t)t * (pstride / 2)] = bf16_pair(t0[t], t1[t]);
   }
+}
+
+// Column exponents of a row-major m x n block (cexp preset below every exponent): 32 columns per block and a
+// chunk of rows per blockIdx.y, coalesced along the rows, four rows in flight per thread.
+__global__ void __launch_bounds__(256) colexp_rows_kernel(int64_t m, int n, const double* __restrict__ X, int* cexp) {
+  __shared__ int red[8][32];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, j = blockIdx.x * 32 + tx;
+  const int64_t step = 8 * (int64_t)gridDim.y;
+  int e = -100000;
+  if (j < n)
+    for (int64_t i = 8 * (int64_t)blockIdx.y + ty; i < m; i += 4 * step) {
+      double v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = i + u * step < m ? X[(i + u * step) * n + j] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) e = max(e, exp_of(v[u]));
+    }
+  red[ty][tx] = e;
+  __syncthreads();
+  if (ty == 0 && j < n) {
+#pragma unroll
+    for (int y = 1; y < 8; ++y) e = max(e, red[y][tx]);
+    atomicMax(cexp + j, e);
+  }
+}
+
+// The slice planes of a row-major m x n block: elementwise, two columns per thread.
+__global__ void __launch_bounds__(256) xslice_rows_kernel(int64_t m, int n, int np, const double* __restrict__ X,
+                                                          const int* __restrict__ cexp,
+                                                          __nv_bfloat16* __restrict__ planes) {
+  const int64_t pstride = m * (int64_t)np;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int j = blockIdx.y * 64 + 2 * tx;
+  const int e0 = (j < n) ? max(cexp[j], -100000) : 0, e1 = (j + 1 < n) ? max(cexp[j + 1], -100000) : 0;
+  for (int64_t i0 = (int64_t)blockIdx.x * 32; i0 < m; i0 += (int64_t)gridDim.x * 32) {
+    double x0[4], x1[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t i = i0 + 8 * u + ty;
+      x0[u] = i < m && j < n ? X[i * n + j] : 0.0;
+      x1[u] = i < m && j + 1 < n ? X[i * n + j + 1] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t i = i0 + 8 * u + ty;
+      if (i >= m) break;
+      float t0[S], t1[S];
+      digits7(fixed56(x0[u], e0 == -100000 ? 0 : e0), t0);
+      digits7(fixed56(x1[u], e1 == -100000 ? 0 : e1), t1);
+      uint32_t* dst = reinterpret_cast<uint32_t*>(planes + i * np + j);
+#pragma unroll
+      for (int t = 0; t < S; ++t) dst[(int64_t)t * (pstride / 2)] = bf16_pair(t0[t], t1[t]);
+    }
+  }
+}
+
+// W = A X - B X diag(lam) from the two fixed-point accumulators, row-major m x n, and the sums of squares of
+// its columns over this block's rows (part[blockIdx.y][j]).  32 columns per block, chunks of rows per
+// blockIdx.y.  The accumulators are converted with integer arithmetic: the FP64 pipe, which the conversions
+// would share with the two FP64 products per element, is what bounds the pass otherwise.
+__global__ void __launch_bounds__(256) fixed_residual_kernel(int64_t m, int n, const long long* __restrict__ VA,
+                                                             const long long* __restrict__ VB,
+                                                             const int* __restrict__ rowA, const int* __restrict__ rowB,
+                                                             const int* __restrict__ cexp, int HA, int HB,
+                                                             const double* __restrict__ lam, double* __restrict__ W,
+                                                             double* __restrict__ part) {
+  __shared__ double red[8][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, j = blockIdx.x * 32 + tx;
+  const int64_t step = 8 * (int64_t)gridDim.y;
+  double sum = 0.0;
+  if (j < n) {
+    const double l = lam[j];
+    const int ec = max(cexp[j], -100000);
+    for (int64_t i = 8 * (int64_t)blockIdx.y + ty; i < m; i += 4 * step) {
+      long long a[4], b[4];
+      int ra[4], rb[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t r = i + u * step;
+        const bool in = r < m;
+        a[u] = in ? VA[r * n + j] : 0;
+        b[u] = in ? VB[r * n + j] : 0;
+        ra[u] = in ? rowA[r] : 0;
+        rb[u] = in ? rowB[r] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t r = i + u * step;
+        if (r >= m) break;
+        const double w = fma(-l, fixed_value<true>(b[u], rb[u], ec, HB), fixed_value<true>(a[u], ra[u], ec, HA));
+        W[r * n + j] = w;
+        sum = fma(w, w, sum);
+      }
+    }
+  }
+  red[ty][tx] = sum;
+  __syncthreads();
+  if (ty == 0 && j < n) {
+#pragma unroll
+    for (int y = 1; y < 8; ++y) sum += red[y][tx];
+    part[(int64_t)blockIdx.y * n + j] = sum;
+  }
+}
+
+// norms[j] = sqrt of the sum of the parts of column j: one warp per column.
+__global__ void __launch_bounds__(256) part_norms_kernel(int n, int parts, const double* __restrict__ part,
+                                                         double* __restrict__ norms) {
+  const int j = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x & 31;
+  if (j >= n) return;
+  double s = 0.0;
+  for (int q = lane; q < parts; q += 32) s += part[(int64_t)q * n + j];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) norms[j] = sqrt(s);
 }
 
 struct FeOzArgs {
@@ -726,6 +840,44 @@ void fe_apply_f64_cols_tc(cudaStream_t s, const FeOp& op, const double* X, doubl
     fixed_to_cols_kernel<<<dim3(cdiv(m, 32), cdiv(n, 32)), 256, 0, s>>>(m, n, mrow, V, rowexp, cexp, H, out);
     RC_LAUNCH();
   }
+}
+
+void fe_residual_rows_tc(cudaStream_t s, const FeOp& op, const double* X, const double* lam, int n, int num_sms,
+                         double* accA, double* accB, DevBuf<double>& part, double* W, double* norms) {
+  RC_CHECK(op.nc <= kNCP && !op.cplx, RCHFSI_ERR_INVALID_ARG, "row-major residual: real operators with n_c <= 128");
+  const int64_t m = op.m;
+  if (n <= 0 || m <= 0) return;
+  int* cexp = op.ozcexp.ensure(n);
+  const int np = (int)cdiv(n, kBN) * kBN;
+  const int64_t total = m * (int64_t)np;
+  __nv_bfloat16* planes = op.ozplanes.ensure((size_t)S * total);
+  // rows in chunks, for about eight blocks per SM over the column tiles
+  const unsigned ct = cdiv(n, 32);
+  const unsigned chunks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(cdiv(m, 64), (int64_t)num_sms * 8 / ct + 1));
+  {
+    prof::Scope ps(s, RCHFSI_KERNEL_RR_AUX, 0.0, 16.0 * m * n + 14.0 * (double)total);
+    RC_CUDA(cudaMemsetAsync(cexp, 0x80, sizeof(int) * n, s));
+    colexp_rows_kernel<<<dim3(ct, chunks), 256, 0, s>>>(m, n, X, cexp);
+    RC_LAUNCH();
+    const unsigned xb = (unsigned)std::min<int64_t>(cdiv(m, 32), (int64_t)num_sms * 16);
+    xslice_rows_kernel<<<dim3(xb, (unsigned)(np / 64)), 256, 0, s>>>(m, n, np, X, cexp, planes);
+    RC_LAUNCH();
+  }
+  long long* V[2] = {reinterpret_cast<long long*>(accA), reinterpret_cast<long long*>(accB)};
+  const int* row[2];
+  int H[2];
+  for (int which = 0; which < 2; ++which) {
+    RC_CUDA(cudaMemsetAsync(V[which], 0, sizeof(long long) * m * n, s));
+    row[which] = ensure_rowexp(s, op, which == 1);
+    H[which] = headroom(op, which == 1);
+    launch_oz(s, num_sms, op, which == 1, planes, total, np, row[which], H[which], V[which], n, false);
+  }
+  prof::Scope ps(s, RCHFSI_KERNEL_RR_AUX, 4.0 * m * n, 24.0 * m * n);
+  double* pt = part.ensure((size_t)chunks * n);
+  fixed_residual_kernel<<<dim3(ct, chunks), 256, 0, s>>>(m, n, V[0], V[1], row[0], row[1], cexp, H[0], H[1], lam, W, pt);
+  RC_LAUNCH();
+  part_norms_kernel<<<cdiv(n, 8), 256, 0, s>>>(n, (int)chunks, pt, norms);
+  RC_LAUNCH();
 }
 
 }  // namespace rchfsi

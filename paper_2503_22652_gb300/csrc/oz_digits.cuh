@@ -90,4 +90,19 @@ __device__ __forceinline__ double fixed_to_f64(long long v, int e) {
   return __longlong_as_double(__double_as_longlong(d) + ((long long)e << 52));
 }
 
+// The same in integer arithmetic, for passes that need the FP64 pipe for something else.
+__device__ __forceinline__ double fixed_to_f64_int(long long v, int e) {
+  if (v == 0) return 0.0;
+  const unsigned long long sgn = v < 0 ? (1ull << 63) : 0ull;
+  unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)a);
+  a <<= lz;                          // leading one at bit 63
+  unsigned long long mant = a >> 11;  // 53 significant bits
+  const unsigned long long rem = a & 0x7ffull;
+  if (rem > 0x400ull || (rem == 0x400ull && (mant & 1ull))) ++mant;
+  const int be = 1086 - lz + e;  // v 2^e = 1.f 2^(63 - lz + e); a carry of the rounding runs into the exponent
+  if (be <= 0 || be >= 2046) return ldexp((double)v, e);  // out of the normal range: rare
+  return __longlong_as_double((long long)(sgn | (((unsigned long long)be << 52) + (mant - (1ull << 52)))));
+}
+
 }  // namespace rchfsi

@@ -81,3 +81,25 @@ def test_output_may_overlap_inputs_fe(N, prec, tol):
     for ref, got in _overlaps(s, X, L, W, args):
         for y in (ref, got):
             assert np.linalg.norm(y - exact) <= tol * np.linalg.norm(exact - base)
+
+
+@pytest.mark.parametrize("N", [1, 31, 65, 130])
+def test_fe_residual_rows(N):
+    from oracle import fe as ofe
+    q = wl.fe_problem(3)
+    A = ofe.assemble(q["cell_dofs"], q["A_cells"], q["m"])
+    B = ofe.assemble(q["cell_dofs"], q["B_cell"], q["m"])
+    rng = np.random.default_rng(N)
+    X = rng.standard_normal((q["m"], N)) * np.logspace(-5, 5, N)[None, :]
+    X[:, N // 2] = 0.0
+    L = np.sort(rng.uniform(-20.0, 30.0, N))
+    s = Solver(q["m"], nev=1, block=N, rr_mode="emulated")
+    s.set_fe(q["cell_dofs"], q["A_cells"], q["B_cell"], q["Dinv"])
+    W, r = s.residual(X, L)
+    ref = A @ X - (B @ X) * L[None, :]
+    scale = np.abs(A).sum(1).max() * np.linalg.norm(X, axis=0) + 1e-300
+    assert (np.linalg.norm(W - ref, axis=0) / scale).max() <= 1e-14
+    assert np.allclose(r, np.linalg.norm(ref, axis=0), rtol=1e-12, atol=1e-12 * scale.max() * 1e-3)
+    X[3, 0] = np.inf
+    W, r = s.residual(X, L)
+    assert np.isnan(r[0]) and (N == 1 or np.isfinite(r[1:]).all())
