@@ -1001,13 +1001,14 @@ int rchfsi_filter(rchfsi_ctx* h, const double* X, const double* Lambda, const do
     need_op(h);
     RC_CHECK(Yp, RCHFSI_ERR_INVALID_ARG, "Yp is NULL");
     rchfsi_ctx& c = *h;
-    const std::vector<double> lam = lam_any(c, Lambda);
     if (filter_takes_rows(c)) {
+      RC_CHECK(Lambda, RCHFSI_ERR_INVALID_ARG, "NULL vector argument");
       RC_CHECK(W, RCHFSI_ERR_INVALID_ARG, "NULL block argument");
-      filter_rows(c, X, lam.data(), W, lmin, lT, lmax, degree, Yp);
+      filter_rows(c, X, Lambda, W, lmin, lT, lmax, degree, Yp);
       RC_CUDA(cudaStreamSynchronize(c.s));
       return RCHFSI_OK;
     }
+    const std::vector<double> lam = lam_any(c, Lambda);
     load_any(c, X, c.w.X.p);
     load_any(c, W, c.w.W.p);
     filter_any(c, c.w.X.p, lam.data(), c.w.W.p, lmin, lT, lmax, degree, c.w.Y.p, false, false);

@@ -525,24 +525,16 @@ bool filter_takes_rows(const rchfsi_ctx& c) {
   return !c.cplx && c.p.precision != RCHFSI_FP64 && !(c.op_kind == RCHFSI_OP_DENSE && c.dense.has_dinv_dense);
 }
 
-void filter_internal(rchfsi_ctx& c, const double* X, const double* lam_host, const double* W, double lmin, double lT,
+void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const double* W, double lmin, double lT,
                      double lmax, int p, double* Y, bool chfsi, bool rows) {
   check_bounds(lmin, lT, lmax, p);
   const int N = c.p.block;
   double e, cc, s1;
   std::vector<Coef> co;
   filter_scalars(lmin, lT, lmax, p, e, cc, s1, co);
-  std::vector<double> tab;
-  if (!chfsi) {
-    lambda_table(lam_host, N, e, cc, s1, co, tab);
-  } else {
-    tab.assign((size_t)(p + 1) * N, 0.0);
-  }
   // The degree loop of a dense TF32 / BF16 filter runs as one launch where the operator has at most a
   // quarter as many row tiles as the GPU has SMs (see tc_loop_plan) and its workspace fits the budget.
   TcLoopPlan loop;
-  LoopTables ls;
-  size_t coef_at = 0, cnt_at = 0;
   const int loop_steps = p - 1 + (chfsi ? 1 : 0);
   if (c.op_kind == RCHFSI_OP_DENSE && (c.p.precision == RCHFSI_TF32 || c.p.precision == RCHFSI_BF16) &&
       loop_steps > 0) {
@@ -553,11 +545,56 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam_host, con
     if (loop.ok && c.p.hbm_budget_bytes && c.w.split.n < loop.ws_floats &&
         device_bytes(c) - c.w.split.bytes() + loop.ws_floats * sizeof(float) > c.p.hbm_budget_bytes)
       loop.ok = false;
+    if (loop.ok) c.w.split.ensure(loop.ws_floats);
+  }
+  // one buffer: the Lambda table, and for the loop the coefficients and Lambda rows 1 .. p - 1 in FP32 and the
+  // counters on 128-byte lines
+  const size_t coef_at = (size_t)(p + 1) * N;
+  const size_t floats = loop.ok ? 3 * (size_t)loop_steps + (chfsi ? 0 : (size_t)loop_steps * N) : 0;
+  const size_t cnt_at = (coef_at + (floats + 1) / 2 + 15) / 16 * 16;
+  const size_t total = loop.ok ? cnt_at + loop.counters / 2 : coef_at;
+  double* dtab = c.w.lamtab.ensure(total);
+  LoopTables ls;
+  if (loop.ok) {
+    ls.coef = reinterpret_cast<const float*>(dtab + coef_at);
+    ls.lam = ls.coef + 3 * (size_t)loop_steps;
+    ls.counters = reinterpret_cast<int*>(dtab + cnt_at);
+  }
+  std::vector<double> tab;
+  if (!chfsi && p - 1 <= kTableSteps && is_device_pointer(lam)) {
+    // Lambda is on the device: so is its recurrence, and the call does not wait for a copy to the host and back
+    FilterTables t;
+    t.steps = p - 1;
+    t.N = N;
+    t.s1e = s1 / e;
+    t.cc = cc;
+    for (int k = 0; k < p - 1; ++k) {
+      t.a[k] = co[k].a;
+      t.b[k] = co[k].b;
+      t.c[k] = co[k].c;
+    }
+    t.lam = lam;
+    t.tab = dtab;
+    t.coef = const_cast<float*>(ls.coef);
+    t.lamf = const_cast<float*>(ls.lam);
+    t.counters = ls.counters;
+    t.ncounters = loop.ok ? (int)loop.counters : 0;
+    filter_tables(c.s, t);
+  } else {
+    if (chfsi) {
+      tab.assign(total, 0.0);
+    } else {
+      std::vector<double> host;
+      if (is_device_pointer(lam)) {
+        host.resize(N);
+        RC_CUDA(cudaMemcpyAsync(host.data(), lam, N * sizeof(double), cudaMemcpyDeviceToHost, c.s));
+        RC_CUDA(cudaStreamSynchronize(c.s));
+        lam = host.data();
+      }
+      lambda_table(lam, N, e, cc, s1, co, tab);
+      tab.resize(total, 0.0);
+    }
     if (loop.ok) {
-      coef_at = tab.size();
-      const size_t floats = 3 * (size_t)loop_steps + (chfsi ? 0 : (size_t)loop_steps * N);
-      cnt_at = (coef_at + (floats + 1) / 2 + 15) / 16 * 16;  // counters on 128-byte lines
-      tab.resize(cnt_at + loop.counters / 2, 0.0);
       float* f = reinterpret_cast<float*>(tab.data() + coef_at);
       int o = 0;
       if (chfsi) {
@@ -572,18 +609,12 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam_host, con
       }
       if (!chfsi)
         for (size_t t = 0; t < (size_t)loop_steps * N; ++t) f[o + t] = (float)tab[(size_t)N + t];
-      c.w.split.ensure(loop.ws_floats);
     }
+    RC_CUDA(cudaMemcpyAsync(dtab, tab.data(), total * sizeof(double), cudaMemcpyHostToDevice, c.s));
   }
-  double* dtab = c.w.lamtab.ensure(tab.size());
-  if (loop.ok) {
-    ls.coef = reinterpret_cast<const float*>(dtab + coef_at);
-    ls.lam = ls.coef + 3 * (size_t)loop_steps;
-    ls.counters = reinterpret_cast<int*>(dtab + cnt_at);
-  }
-  RC_CUDA(cudaMemcpyAsync(dtab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, c.s));
   // zero "lambda" vector used by reconstructions that only upcast
-  RC_CUDA(cudaMemsetAsync(c.w.nrm.p, 0, sizeof(double) * N, c.s));
+  if (chfsi || (c.op_kind == RCHFSI_OP_DENSE && c.dense.has_dinv_dense))
+    RC_CUDA(cudaMemsetAsync(c.w.nrm.p, 0, sizeof(double) * N, c.s));
   if (c.op_kind == RCHFSI_OP_DENSE)
     filter_dense(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi, loop, ls, rows);
   else

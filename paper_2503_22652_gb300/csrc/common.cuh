@@ -155,6 +155,19 @@ void rows_to_cols_recon(cudaStream_t s, int64_t m, int64_t n, const float* R, do
 void rows_f32x2(cudaStream_t s, int64_t m, int64_t n, const double* W, double s1, double s2, float* o1, float* o2);
 void rows_recon(cudaStream_t s, int64_t m, int64_t n, const float* R, double rs, const double* dinv, const double* X,
                 const double* lam, double* Y);
+// The tables of one filter from Lambda on the device: rows C_0 .. C_p of the Lambda recurrence (tab, (steps + 2) x N)
+// and, when given, its rows 1 .. steps in FP32 (lamf), the step coefficients in FP32 (coef) and zeroed counters.
+constexpr int kTableSteps = 96;
+struct FilterTables {
+  int steps, N, ncounters;
+  double s1e, cc, a[kTableSteps], b[kTableSteps], c[kTableSteps];
+  const double* lam;
+  double* tab;
+  float* coef;
+  float* lamf;
+  int* counters;
+};
+void filter_tables(cudaStream_t s, const FilterTables& t);
 // Dense filter with row-major callers' blocks: o1 = s1 W and o2 = W (may be null) column-major of pitch ld; and
 // Y = dinv .* R + X diag(lam), R column-major of pitch ldr, X and Y row-major (Y may be X).
 void rows_to_cols_lowp_f32(cudaStream_t s, int64_t m, int64_t n, const double* W, double s1, float* o1, float* o2,

@@ -51,6 +51,32 @@ __device__ __forceinline__ double f64_of(float x) {
                                           (((unsigned long long)(b & 0x7fffffffu) << 29) + (896ULL << 52))));
 }
 
+// One column per lane, one warp per block: a chain of 3 FP64 instructions (64 clocks each) per step.
+__global__ void __launch_bounds__(32) filter_tables_kernel(const __grid_constant__ FilterTables t) {
+  const int j = blockIdx.x * 32 + threadIdx.x;
+  if (j < t.N) {
+    const double lm = t.lam[j] - t.cc;
+    double lx = 1.0, ly = t.s1e * lm;
+    t.tab[j] = 1.0;
+    t.tab[(int64_t)t.N + j] = ly;
+    for (int k = 0; k < t.steps; ++k) {
+      if (t.lamf) t.lamf[(int64_t)k * t.N + j] = f32_rn(ly);
+      const double nx = fma(t.a[k] * lm, ly, t.c[k] * lx);
+      lx = ly;
+      ly = nx;
+      t.tab[(int64_t)(k + 2) * t.N + j] = ly;
+    }
+  }
+  const int stride = gridDim.x * 32;
+  if (t.coef)
+    for (int k = j; k < t.steps; k += stride) {
+      t.coef[3 * k] = f32_rn(t.a[k]);
+      t.coef[3 * k + 1] = f32_rn(t.b[k]);
+      t.coef[3 * k + 2] = f32_rn(t.c[k]);
+    }
+  for (int i = j; i < t.ncounters; i += stride) t.counters[i] = 0;
+}
+
 // o1(i, j) = (float)(W(i, j) s1), o2(i, j) = (float)(W(i, j) s2): W column-major (leading dimension
 // m), o1 and o2 row-major m x n.  32 x 32 shared-memory tiles, rows on blockIdx.x.
 __global__ void __launch_bounds__(256) cols_to_rows_f32x2_kernel(int64_t m, int64_t n, const double* __restrict__ W,
@@ -471,6 +497,11 @@ void cols_to_rows_recon_f32(cudaStream_t s, int64_t m, int64_t n, const float* R
 void cols_to_rows_recon_bf16(cudaStream_t s, int64_t m, int64_t n, const __nv_bfloat16* R, int64_t ldr,
                              const double* dinv, const double* X, const double* lam, double* Y) {
   cols_to_rows_recon<__nv_bfloat16>(s, m, n, R, ldr, dinv, X, lam, Y);
+}
+
+void filter_tables(cudaStream_t s, const FilterTables& t) {
+  filter_tables_kernel<<<cdiv(t.N, 32), 32, 0, s>>>(t);
+  RC_LAUNCH();
 }
 
 static bool pairs_ok(int64_t n, const void* a, const void* b) {

@@ -98,7 +98,8 @@ const double* dinv_diag(const rchfsi_ctx& c);
 // Algorithm 3 / Algorithm 2 on column-major inputs; Y is column-major FP64.  rows: all three are row-major
 // (only where filter_takes_rows says so; Y may be X, or an array that does not overlap X).
 bool filter_takes_rows(const rchfsi_ctx& c);
-void filter_internal(rchfsi_ctx& c, const double* X, const double* lam_host, const double* W, double lmin,
+// lam: N values, on the host or the device.
+void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const double* W, double lmin,
                      double lT, double lmax, int p, double* Y, bool chfsi, bool rows = false);
 
 // Rayleigh-Ritz on column-major Y (scaled in place): X and evals (device) are outputs, and with `products`
