@@ -1,11 +1,13 @@
 // FP64-accurate products from BF16 tensor-core slices (see oz_gemm.cuh for the scheme).
 //
 // oz_gemm_kernel: persistent CTAs (one per SM) walking (128 x 64 output tile, K range) items.
-// Warp 0 (one lane) streams, per 32-wide K chunk, the 7 A and the 7 B slices of the tile (8 KB and
-// 4 KB each, 64-byte swizzle) into one 84 KB stage with TMA, two stages, one barrier per stage;
+// Warp 0 (one lane) streams, per 64-wide K chunk, the 7 A and the 7 B slices of the tile (16 KB and
+// 8 KB each, whole 128-byte rows, 128-byte swizzle) with TMA, every slice into a slot of its own ring;
 // warp 1 (the whole warp, one elected lane issuing) runs, for each A slice s, the products with B
-// slices t <= 6 - s (2 x tcgen05.mma kind::f16, K = 16) into the TMEM accumulator of level s + t,
-// GROUP chunks (128 K terms) per exact accumulation group.  TMEM holds 8 level blocks of 64 columns,
+// slices t <= 6 - s (4 x tcgen05.mma kind::f16, K = 16) into the TMEM accumulator of level s + t,
+// GROUP chunks (128 K terms) per exact accumulation group.  Pass s is the last to read A slice s and
+// B slice 6 - s, so each pass ends with one commit that frees both and the next chunk's slices arrive
+// while this one is multiplied.  TMEM holds 8 level blocks of 64 columns,
 // 7 for the group and one spare, rotated so that the next group's first writes go to blocks in the
 // order they are freed; warps 2-17 (four per TMEM lane quarter, 16 columns each) fold level L of a
 // group as soon as the group's pass L is done: tcgen05.ld, exact scaling by 2^-8L and TwoSum into
@@ -13,6 +15,12 @@
 // exponent arithmetic, is stored in FP64 (or, with split-K, written as a partial and summed by a
 // second kernel) while the next item's MMAs run.  The host splits K only as far as the items fill the
 // CTAs.
+// Bound: issue of the 128 x 64 x 16 MMAs by one warp beside 16 busy epilogue warps.  A pass runs its A tile (16 K
+// values) against all its B slices before the next, with the tile kept in the collector: 35 clocks per MMA alone
+// instead of 48 (shared-memory reads of A).  Measured per MMA in the kernel: 86 clocks with stages of whole 32-wide
+// chunks, 87 with a ring and an arrival barrier per slice, 68 with the arrivals merged into five per chunk (a wait
+// that finds its data there still costs about 130 clocks).  262144 x 600 x 600: 6.79 -> 5.50 ms, the Gram matrix of
+// 600 columns of 262144 4.03 -> 3.25 ms.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -31,15 +39,17 @@ constexpr int BM = 128;
 constexpr int KC = 64;            // K tile of the slicing kernel (K is padded to a multiple of it)
 // Chunks accumulated in TMEM before a drain: 2 x 64 = 128 K terms per exact FP32 sum (each term a
 // product of two integer slices, |t_s t_r| <= 2^16, so every partial sum stays below 2^23).
-constexpr int KCH = 32;           // K chunk of the products: one 64-byte row of BF16 per slice
-constexpr int GROUP = 4;          // chunks per exact accumulation group (4 x 32 = 128 K terms)
-constexpr int NSTAGE = 2;
+constexpr int KCH = 64;           // K chunk of the products: one 128-byte row of BF16 per slice
+constexpr int GROUP = 2;          // chunks per exact accumulation group (2 x 64 = 128 K terms)
+constexpr int kARing = 8;         // A slices in flight (a power of two)
+constexpr int kBRing = 8;         // B slices 6 .. 1 in flight (a power of two); slice 0 alternates between two slots
+constexpr int kPassRing = 16;     // barriers of finished passes: more than the passes the producer runs ahead
 constexpr int BN = 64;            // output tile columns
 constexpr int kThreads = 576;     // 18 warps: TMA producer, MMA issuer, 16 epilogue warps
 constexpr int kEpiThreads = 512;
-constexpr uint32_t kASlice = BM * 64;        // 8 KB per A slice of a chunk
-constexpr uint32_t kBSlice = BN * 64;        // 4 KB per B slice of a chunk
-constexpr uint32_t kStage = S * (kASlice + kBSlice);  // all 14 slices of one chunk: 84 KB
+constexpr uint32_t kASlice = BM * 128;       // 16 KB per A slice of a chunk
+constexpr uint32_t kBSlice = BN * 128;       // 8 KB per B slice of a chunk
+constexpr uint32_t kSmemBytes = kARing * kASlice + (kBRing + 2) * kBSlice;  // 208 KB
 constexpr uint32_t kTmemCols = 512;          // 8 level blocks x 64 columns
 
 // ---------------------------------------------------------------- slicing
@@ -224,19 +234,6 @@ __device__ __forceinline__ uint32_t perm_next(uint32_t perm) {
 }
 constexpr uint32_t kPerm0 = 0x76543210u;
 
-// Shared-memory descriptor of a K-major tile with 64-byte rows and 64-byte swizzle (the layout the
-// TMA's 64-byte swizzle writes: 16-byte chunk c of row r at chunk c ^ ((r >> 1) & 3)), 8-row atoms
-// 512 bytes apart; layout type 4 of the descriptor (checked on the GPU against a plain product).
-__device__ __forceinline__ uint64_t sw64_desc(uint32_t smem_addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((smem_addr >> 4) & 0x3FFF);
-  d |= (uint64_t)(16 >> 4) << 16;
-  d |= (uint64_t)(512 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;
-  return d;
-}
-
 // Work item -> (row tile, column tile, K split).  Items run split-major, column tile fastest, so
 // CTAs working at the same time share the row tile's A slices and the split's K range in L2.  With
 // `upper`, row tile tm keeps only the column tiles tn >= tm BM / BN (those reaching i <= j).
@@ -268,19 +265,23 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   // lev[g & 1][L]: level L of accumulation group g has all its products (two sets, so that the next
   // group's levels never complete a phase that the epilogue is still waiting for)
-  __shared__ __align__(8) uint64_t sfull[NSTAGE], sempty[NSTAGE], lev[2][S], bfree[8], mdone;
+  // arrivals by chunk parity: A slices 0 | 1, 2 | 3, 4 | 5, 6 and all B slices (a wait of the issuer costs about
+  // 130 clocks, four MMAs, even when it finds its data there)
+  __shared__ __align__(8) uint64_t afull[2][4], bfull[2], pass_done[kPassRing], lev[2][S], bfree[8], mdone;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  // stage b: A slices at b * kStage + s * kASlice, B slices after them (K-major, 64-byte swizzle)
+  uint8_t* sB = smem + kARing * kASlice;   // ring of B slices 6 .. 1
+  uint8_t* sB0 = sB + kBRing * kBSlice;    // two slots of B slice 0
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < NSTAGE; ++i) {
-      tc::mbar_init(&sfull[i], 1);
-      tc::mbar_init(&sempty[i], 1);
+    for (int i = 0; i < 2; ++i) {
+      for (int g = 0; g < 4; ++g) tc::mbar_init(&afull[i][g], 1);
+      tc::mbar_init(&bfull[i], 1);
     }
+    for (int i = 0; i < kPassRing; ++i) tc::mbar_init(&pass_done[i], 1);
     for (int L = 0; L < S; ++L) {
       tc::mbar_init(&lev[0][L], 1);
       tc::mbar_init(&lev[1][L], 1);
@@ -313,32 +314,63 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      // ---------------- TMA producer: per K chunk, the 7 A and 7 B slices into one stage
-      int64_t cg = 0;  // chunks issued so far
+      // ---------------- TMA producer.  Counted over the whole launch: chunk cg, pass 7 cg + s (it reads A
+      // slice s), B ring entry 6 cg + (6 - t) for slice t >= 1.  Order of the loads = order of first use.
+      int64_t cg = 0;
+      int64_t seen = -1;  // passes up to this one are known to be done
+      int armed = 0;      // arrivals of chunk cg armed so far: A group 0, B, A groups 1 .. 3
       bool ok = true;
+      auto pass_is_done = [&](int64_t pass) -> bool {
+        if (pass <= seen) return true;
+        if (*vabort || !tc::mbar_wait(&pass_done[pass & (kPassRing - 1)], (uint32_t)(pass / kPassRing) & 1u)) return false;
+        seen = pass;
+        return true;
+      };
       for (int64_t it = blockIdx.x; it < p.items && ok; it += G) {
         const OzItem w = oz_item(p, it);
         const int nch = chunks_of(w.split), c_begin = w.split * p.chunks_per_split;
-        for (int ci = 0; ci < nch; ++ci, ++cg) {
-          const int k0 = (c_begin + ci) * KCH;
-          const int b = (int)(cg % NSTAGE);
-          if (*vabort || !tc::mbar_wait(&sempty[b], (uint32_t)((cg / NSTAGE) & 1) ^ 1u)) {
-            ok = false;
-            break;
+        for (int ci = 0; ci < nch; ++ci) {
+          const int k0 = (c_begin + ci) * KCH, z = (int)(cg & 1);
+          armed = 0;
+          auto load_a = [&](int s) {
+            const int64_t pass = S * cg + s;  // the slot's previous slice was read by pass - kARing
+            if (!pass_is_done(pass - kARing)) return false;
+            const int slot = (int)(pass & (kARing - 1)), g = (s + 1) / 2;
+            if (s == 0 || (s & 1)) {
+              tc::mbar_arrive_expect_tx(&afull[z][g], s == 0 ? kASlice : 2 * kASlice);
+              ++armed;
+            }
+            tc::tma_load_2d(smem + (size_t)slot * kASlice, &mapA, &afull[z][g], k0, s * p.MP + w.tm * BM);
+            return true;
+          };
+          ok = load_a(0) && pass_is_done(S * (cg - 2) + S - 1);
+          if (!ok) break;
+          tc::mbar_arrive_expect_tx(&bfull[z], S * kBSlice);
+          ++armed;
+          tc::tma_load_2d(sB0 + (size_t)z * kBSlice, &mapB, &bfull[z], k0, w.tn * BN);
+          for (int t = S - 1; t >= 1 && ok; --t) {
+            const int64_t q = (S - 1) * cg + (S - 1 - t), o = q - kBRing;  // o: the slot's previous entry
+            ok = o < 0 || pass_is_done(S * (o / (S - 1)) + o % (S - 1));
+            if (ok)
+              tc::tma_load_2d(sB + (size_t)(q & (kBRing - 1)) * kBSlice, &mapB, &bfull[z], k0, t * p.NP + w.tn * BN);
           }
-          uint8_t* st = smem + (size_t)b * kStage;
-          tc::mbar_arrive_expect_tx(&sfull[b], kStage);
-          for (int t = 0; t < S; ++t) {
-            tc::tma_load_2d(st + (size_t)t * kASlice, &mapA, &sfull[b], k0, t * p.MP + w.tm * BM);
-            tc::tma_load_2d(st + (size_t)S * kASlice + (size_t)t * kBSlice, &mapB, &sfull[b], k0, t * p.NP + w.tn * BN);
-          }
+          for (int s = 1; s < S && ok; ++s) ok = load_a(s);
+          if (!ok) break;
+          ++cg;
         }
       }
       if (!ok) {
         fail();
-        // wait (bounded) for copies that may still be landing in this CTA's shared memory
-        for (int64_t c = (cg > NSTAGE ? cg - NSTAGE : 0); c < cg; ++c)
-          tc::mbar_wait(&sfull[c % NSTAGE], (uint32_t)((c / NSTAGE) & 1));
+        // wait for copies that may still be landing in this CTA's shared memory: whole chunks by their barriers,
+        // the copies of the unfinished one (its arrivals may never complete) for a time far above a copy's
+        for (int64_t c = (cg > 2 ? cg - 2 : 0); c < cg; ++c) {
+          const int z = (int)(c & 1);
+          if (c == cg - 2 && armed) continue;  // (its barriers are in use by chunk cg, and its copies were all read)
+          for (int g = 0; g < 4; ++g) tc::mbar_wait(&afull[z][g], (uint32_t)(c >> 1) & 1u);
+          tc::mbar_wait(&bfull[z], (uint32_t)(c >> 1) & 1u);
+        }
+        const long long t0 = clock64();
+        while (clock64() - t0 < 4000000LL) {}
       }
     }
   } else if (warp == 1) {
@@ -349,52 +381,81 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t perm = kPerm0, use_par = 0;  // use_par bit b: parity of the uses of level block b so far
     int64_t cg = 0, gidx = 0;
     bool ok = true;
+    const uint64_t a_base = tc::sw128_desc(tc::smem_u32(smem)), b_base = tc::sw128_desc(tc::smem_u32(sB)),
+                   b0_base = tc::sw128_desc(tc::smem_u32(sB0));
     for (int64_t it = blockIdx.x; it < p.items && ok; it += G) {
       const OzItem wi = oz_item(p, it);
       const int nch = chunks_of(wi.split);
       for (int ci = 0; ci < nch && ok; ++ci, ++cg) {
-        const int b = (int)(cg % NSTAGE);
         const bool first = (ci % GROUP) == 0, last = (ci % GROUP) == GROUP - 1 || ci == nch - 1;
-        bool w = !*vabort && tc::mbar_wait(&sfull[b], (uint32_t)((cg / NSTAGE) & 1));
+        uint32_t dcol[S];  // TMEM columns of the levels
+        uint64_t bd[S];    // descriptors of the chunk's B slices
+#pragma unroll
+        for (int L = 0; L < S; ++L) dcol[L] = tmem + perm_block(perm, L) * (uint32_t)BN;
+        const uint32_t z = (uint32_t)cg & 1u, par = (uint32_t)(cg >> 1) & 1u;
+        bd[0] = tc::desc_add(b0_base, z * kBSlice);
+#pragma unroll
+        for (int t = 1; t < S; ++t)
+          bd[t] = tc::desc_add(b_base, ((uint32_t)((S - 1) * cg + (S - 1 - t)) & (kBRing - 1)) * kBSlice);
+        // a wait that runs out is looked at once per chunk: the products in between then run on whatever the
+        // slots hold, and the launch fails
+        bool w = !*vabort;
+        w &= tc::mbar_wait(&bfull[z], par);
+        w &= tc::mbar_wait(&afull[z][0], par);
+        auto wait_blocks = [&](int t) {  // the epilogue releases blocks in the order 6, 5, .., 1 of the next group
+          const uint32_t blk = perm_block(perm, t);
+          w &= tc::mbar_wait(&bfree[blk], ((use_par >> blk) & 1u) ^ 1u);
+        };
+        if (first) wait_blocks(5);
+        tc::tc_fence_after();
+        // one A tile (16 K values) against B slices t0, t0 + 1, .., kept in the collector between them
+        auto run = [&](int s, int n, auto slice) {
+          const uint64_t a0 = tc::desc_add(a_base, ((uint32_t)(S * cg + s) & (kARing - 1)) * kASlice);
+#pragma unroll
+          for (int kk = 0; kk < KCH / 16; ++kk)
+#pragma unroll
+            for (int u = 0; u < n; ++u) {
+              const int t = slice(u);
+              tc::mma_f16_run(leader, u, n, dcol[s + t], tc::desc_add(a0, kk * 32), tc::desc_add(bd[t], kk * 32), idesc,
+                              first && s == 0 && kk == 0 ? 0u : 1u);
+            }
+        };
+        auto pass_end = [&](int s) {
+          __syncwarp();
+          if (leader) {
+            tc::mma_commit(&pass_done[(S * cg + s) & (kPassRing - 1)]);  // A slice s and B slice 6 - s are free
+            if (last) tc::mma_commit(&lev[gidx & 1][s]);                 // level s of the group has all its products
+          }
+          __syncwarp();
+        };
+        // pass 0 in two runs, the first into the blocks that are released early (0: the spare, 6, 5)
+        run(0, 3, [](int u) { return u == 0 ? 0 : S - u; });
+        if (first) {
+          wait_blocks(1);
+          use_par ^= 0xffu & ~(1u << perm_block(perm, 7));  // the seven blocks of this group
+        }
+        w &= tc::mbar_wait(&afull[z][1], par);
+        tc::tc_fence_after();
+        run(0, 4, [](int u) { return 4 - u; });
+        pass_end(0);
+        run(1, 6, [](int u) { return u; });
+        pass_end(1);
+        w &= tc::mbar_wait(&afull[z][2], par);
+        tc::tc_fence_after();
+        run(2, 5, [](int u) { return u; });
+        pass_end(2);
+        run(3, 4, [](int u) { return u; });
+        pass_end(3);
+        w &= tc::mbar_wait(&afull[z][3], par);
+        tc::tc_fence_after();
+        run(4, 3, [](int u) { return u; });
+        pass_end(4);
+        run(5, 2, [](int u) { return u; });
+        pass_end(5);
+        run(6, 1, [](int u) { return u; });
+        pass_end(6);
         ok = __all_sync(0xffffffffu, w);
         if (!ok) break;
-        const uint32_t st = tc::smem_u32(smem + (size_t)b * kStage);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const uint64_t a0 = sw64_desc(st + (uint32_t)s * kASlice);
-#pragma unroll
-          for (int u = 0; u < S - s; ++u) {
-            // the group's first pass makes the first write of each level, into a block the
-            // epilogue has released, in the order they are released (spare first, then 6, .., 1)
-            const bool fresh = first && s == 0;
-            const int t = fresh ? (u == 0 ? 0 : S - u) : u;
-            const uint32_t blk = perm_block(perm, s + t);
-            if (fresh) {
-              w = !*vabort && tc::mbar_wait(&bfree[blk], ((use_par >> blk) & 1u) ^ 1u);
-              ok = __all_sync(0xffffffffu, w);
-              if (!ok) break;
-              use_par ^= 1u << blk;
-              tc::tc_fence_after();
-            }
-            const uint32_t d = tmem + blk * (uint32_t)BN;
-            const uint64_t b0 = sw64_desc(st + (uint32_t)S * kASlice + (uint32_t)t * kBSlice);
-#pragma unroll
-            for (int kk = 0; kk < KCH / 16; ++kk)
-              if (leader)
-                tc::mma_f16(d, tc::desc_add(a0, kk * 32), tc::desc_add(b0, kk * 32), idesc,
-                            (fresh && kk == 0) ? 0u : 1u);
-          }
-          if (!ok) break;
-          if (last) {
-            __syncwarp();
-            if (leader) tc::mma_commit(&lev[gidx & 1][s]);  // level s of the group has all its products
-            __syncwarp();
-          }
-        }
-        if (!ok) break;
-        __syncwarp();
-        if (leader) tc::mma_commit(&sempty[b]);
-        __syncwarp();
         if (last) {
           perm = perm_next(perm);
           ++gidx;
@@ -506,7 +567,7 @@ CUtensorMap slice_map(const OzOperand& op, int box_rows) {
   cuuint32_t box[2] = {(cuuint32_t)KCH, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)op.sl.p, dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   RC_CHECK(r == CUDA_SUCCESS, RCHFSI_ERR_CUDA, "cuTensorMapEncodeTiled failed for a slice tensor");
   return m;
@@ -587,10 +648,10 @@ void oz_slice(cudaStream_t s, int64_t R, int64_t K, const double* X, int64_t rs,
 namespace {
 
 // Split-K count: the smallest with which the (tile, split) items fill whole rounds of one item per
-// persistent CTA to >= 90% (else the best found), each split keeping >= 4 chunks so that its
+// persistent CTA to >= 90% (else the best found), each split keeping >= 2 chunks so that its
 // drains and final store stay amortised.
 int choose_split(int tiles, int nchunks, int num_sms, double* eff_out) {
-  const int max_split = std::max(1, std::min(64, nchunks / 4));
+  const int max_split = std::max(1, std::min(64, nchunks / 2));
   double best = -1.0;
   int nsplit = 1;
   for (int ns = 1; ns <= max_split; ++ns) {
@@ -642,7 +703,7 @@ void oz_gemm(cudaStream_t s, int num_sms, const OzOperand& A, const OzOperand& B
   nsplit = (nchunks + per - 1) / per;
   const CUtensorMap ma = slice_map(A, BM);
   const CUtensorMap mb = slice_map(B, BN);
-  constexpr size_t smem = (size_t)NSTAGE * kStage + 1024;
+  constexpr size_t smem = (size_t)kSmemBytes + 1024;
   set_smem_limit(reinterpret_cast<const void*>(oz_gemm_kernel), (int)smem);
   OzArgs p;
   p.M = (int)M;

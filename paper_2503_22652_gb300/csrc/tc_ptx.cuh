@@ -112,6 +112,39 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64
       : "memory");
 }
 
+// The same with the A operand kept in the tensor core's collector buffer: kFill reads it from shared memory and
+// keeps it, kUse and kLastUse take it from there.  For runs of MMAs that multiply one A tile (16 K values) with
+// several B tiles.
+enum Collector { kDiscard = 0, kFill = 1, kUse = 2, kLastUse = 3 };
+template <int COL>
+__device__ __forceinline__ void mma_f16_col(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                            uint32_t accumulate) {
+#define RC_MMA_F16(SUFFIX)                                                    \
+  asm volatile(                                                               \
+      "{\n"                                                                   \
+      ".reg .pred p;\n"                                                       \
+      "setp.ne.b32 p, %4, 0;\n"                                               \
+      "tcgen05.mma.cta_group::1.kind::f16" SUFFIX " [%0], %1, %2, %3, p;\n"   \
+      "}\n" ::"r"(d_tmem),                                                    \
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)                   \
+      : "memory")
+  if (COL == kFill) RC_MMA_F16(".collector::a::fill");
+  else if (COL == kUse) RC_MMA_F16(".collector::a::use");
+  else if (COL == kLastUse) RC_MMA_F16(".collector::a::lastuse");
+  else RC_MMA_F16("");
+#undef RC_MMA_F16
+}
+
+// MMA u of a run of n that share the A tile (u and n known at compile time), issued by the leader.
+__device__ __forceinline__ void mma_f16_run(bool leader, int u, int n, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
+                                            uint32_t accumulate) {
+  if (!leader) return;
+  if (n == 1) mma_f16(d, a, b, idesc, accumulate);
+  else if (u == 0) mma_f16_col<kFill>(d, a, b, idesc, accumulate);
+  else if (u == n - 1) mma_f16_col<kLastUse>(d, a, b, idesc, accumulate);
+  else mma_f16_col<kUse>(d, a, b, idesc, accumulate);
+}
+
 // Arrive on `bar` when all previously issued tcgen05.mma of this thread have completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
