@@ -1672,55 +1672,156 @@ __global__ void __launch_bounds__(32) inviter_kernel(int n, const double* __rest
 
 size_t inviter_smem(int n) { return (8 * (size_t)n + 1) * sizeof(double); }
 
-// V = Q Z = H_0 H_1 ... H_{n-3} Z, one warp per column (in place on V), the column held in registers
-// (rows lane + 32 t, t < R) and the next Householder vector prefetched while the current one is
-// applied.  For n <= 32 R.
-template <int R>
-__global__ void __launch_bounds__(64) backtransform_reg_kernel(int n, const double* __restrict__ H,
-                                                               const double* __restrict__ tau, double* V) {
-  const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (col >= n) return;
-  double* zc = V + (size_t)col * n;
-  double z[R], hc[R], hn[R];
+// Four warp sums at once: lane l receives the sum of v[l & 3], one conversion for all four.
+__device__ __forceinline__ double warp_sum4_fx(const double (&v)[4], int lane) {
+  long long t = 0;
+  uint32_t top = 0;
 #pragma unroll
-  for (int t = 0; t < R; ++t) {
-    const int i = lane + 32 * t;
-    z[t] = i < n ? zc[i] : 0.0;
+  for (int a = 0; a < 4; ++a) {
+    const uint32_t hi = (uint32_t)__double2hiint(v[a]), lo = (uint32_t)__double2loint(v[a]);
+    const uint32_t e0 = (hi >> 20) & 0x7ffu, ex = max(e0, 1u);
+    const uint32_t tp = __reduce_max_sync(0xffffffffu, ex), sh = min(tp - ex, 63u);
+    const uint32_t mh = (hi & 0xfffffu) | (e0 ? 0x100000u : 0u);
+    const unsigned long long mant = ((((unsigned long long)mh << 32) | lo) << 9) >> sh;
+    const long long f = (int32_t)hi < 0 ? -(long long)mant : (long long)mant;
+    const uint32_t sl = __reduce_add_sync(0xffffffffu, (uint32_t)f & 0x3ffffffu);
+    const uint32_t sm = __reduce_add_sync(0xffffffffu, (uint32_t)(f >> 26) & 0x3ffffffu);
+    const int sg = __reduce_add_sync(0xffffffffu, (int)(f >> 52));
+    if ((lane & 3) == a) {
+      t = ((long long)sg << 47) + ((long long)sm << 21) + (long long)(sl >> 5);
+      top = tp;
+    }
   }
-  int k = n - 3;
-  if (k < 0) return;
+  const double d = __ll2double_rn(t);
+  const int he = __double2hiint(d), ef = ((he >> 20) & 0x7ff) + (int)top - 1079;
+  if (top == 0x7ffu) return __longlong_as_double(0x7ff8000000000000LL);  // a non-finite addend
+  return t != 0 && ef > 0 ? __hiloint2double(he + (((int)top - 1079) << 20), __double2loint(d)) : 0.0;
+}
+
+// The reflectors of the back-transform in groups of four, k0 = n - 3 - 4 g first: with p_a = v_a . z for the
+// untouched z, the four steps are z -= sum_a s_a v_a, s = T p (T lower triangular, T_aa = tau_a,
+// T_ab = -tau_a sum_{b <= c < a} (v_a . v_c) T_cb).  One warp per group writes T (16 doubles).
+__global__ void __launch_bounds__(32) reflector_groups_kernel(int n, const double* __restrict__ H,
+                                                              const double* __restrict__ tau, double* __restrict__ T) {
+  const int lane = threadIdx.x, k0 = n - 3 - 4 * (int)blockIdx.x;
+  double g[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // (1,0) (2,0) (2,1) (3,0) (3,1) (3,2)
+  for (int i = max(k0 - 2, 0) + lane; i < n; i += 32) {
+    double v[4];
 #pragma unroll
-  for (int t = 0; t < R; ++t) {
-    const int i = lane + 32 * t;
-    hc[t] = (i > k && i < n) ? H[(size_t)k * n + i] : 0.0;
+    for (int a = 0; a < 4; ++a) v[a] = (k0 - a >= 0 && i > k0 - a) ? H[(size_t)(k0 - a) * n + i] : 0.0;
+    g[0] = fma(v[1], v[0], g[0]);
+    g[1] = fma(v[2], v[0], g[1]);
+    g[2] = fma(v[2], v[1], g[2]);
+    g[3] = fma(v[3], v[0], g[3]);
+    g[4] = fma(v[3], v[1], g[4]);
+    g[5] = fma(v[3], v[2], g[5]);
   }
-  for (; k >= 0; --k) {
-    if (k > 0) {
 #pragma unroll
-      for (int t = 0; t < R; ++t) {
-        const int i = lane + 32 * t;
-        hn[t] = (i > k - 1 && i < n) ? H[(size_t)(k - 1) * n + i] : 0.0;
+  for (int q = 0; q < 6; ++q) g[q] = warp_sum_fx(g[q]);
+  if (lane == 0) {
+    double t[4][4] = {}, ta[4];
+    for (int a = 0; a < 4; ++a) ta[a] = k0 - a >= 0 ? tau[k0 - a] : 0.0;
+    const double ga[4][4] = {{0, 0, 0, 0}, {g[0], 0, 0, 0}, {g[1], g[2], 0, 0}, {g[3], g[4], g[5], 0}};
+    for (int a = 0; a < 4; ++a) {
+      t[a][a] = ta[a];
+      for (int b = 0; b < a; ++b) {
+        double x = 0.0;
+        for (int c = b; c < a; ++c) x = fma(ga[a][c], t[c][b], x);
+        t[a][b] = -ta[a] * x;
       }
     }
-    const double tk = tau[k];
-    // (rows up to k are not touched: their chunks are skipped, an FP64 instruction costs the same
-    // with zeros; likewise the chunks past n of a wider instantiation)
-    double s = 0.0;
+    for (int a = 0; a < 4; ++a)
+      for (int b = 0; b < 4; ++b) T[16 * (size_t)blockIdx.x + 4 * a + b] = t[a][b];
+  }
+}
+
+// V = Q Z = H_0 H_1 ... H_{n-3} Z (in place on V), S warps per column, the column in registers (rows
+// lane + 32 t, t = r S + part, r < RR), four reflectors per round (see above).  Bound: FP64 instructions, 64
+// clocks each per sub-partition.  One warp per column used two of the four sub-partitions of 120 SMs at
+// n = 240, and paid a warp sum (about 700 clocks with its waits) per reflector: 240 us there, 26 us at n = 60,
+// 2.41 ms at n = 600.  S is the largest with which n S warps fit on the 608 sub-partitions.
+template <int RR, int S>
+__global__ void __launch_bounds__(128) backtransform_reg_kernel(int n, const double* __restrict__ H,
+                                                                const double* __restrict__ T, double* V) {
+  constexpr bool kKeep = RR <= 5;  // the reflectors' chunks stay in registers between the two uses
+  __shared__ double part_sum[2][4][4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cb = warp / S, part = warp % S;
+  const int col = blockIdx.x * (4 / S) + cb;
+  if (col >= n) return;
+  double* zc = V + (size_t)col * n;
+  double z[RR], h[kKeep ? 4 : 1][kKeep ? RR : 1], hn[kKeep ? 4 : 1][kKeep ? RR : 1];
 #pragma unroll
-    for (int t = 0; t < R; ++t)
-      if (32 * t + 31 > k && 32 * t < n) s = fma(hc[t], z[t], s);
-    s = warp_sum_fx(s) * tk;
+  for (int r = 0; r < RR; ++r) {
+    const int i = lane + 32 * (r * S + part);
+    z[r] = i < n ? zc[i] : 0.0;
+  }
+  auto at = [&](int k, int r) {
+    const int i = lane + 32 * (r * S + part);
+    return (k >= 0 && i > k && i < n) ? __ldg(H + (size_t)k * n + i) : 0.0;
+  };
+  const int groups = (n - 2 + 3) / 4;
+  if (kKeep && groups > 0) {
 #pragma unroll
-    for (int t = 0; t < R; ++t) {
-      if (32 * t + 31 > k && 32 * t < n) z[t] = fma(-s, hc[t], z[t]);
-      hc[t] = hn[t];
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int r = 0; r < RR; ++r) hn[a][r] = at(n - 3 - a, r);
+  }
+  for (int g = 0; g < groups; ++g) {
+    const int k0 = n - 3 - 4 * g;
+    const double2* tp = reinterpret_cast<const double2*>(T + 16 * (size_t)g + 4 * (lane & 3));  // row of T
+    const double2 t01 = __ldg(tp), t23 = __ldg(tp + 1);
+    double p[4] = {0.0, 0.0, 0.0, 0.0};
+    // (rows up to k are not touched: chunks without any other are skipped, an FP64 instruction costs the
+    // same with zeros; likewise the chunks past n)
+    if (kKeep) {
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int r = 0; r < RR; ++r) {
+          h[a][r] = hn[a][r];
+          hn[a][r] = at(k0 - 4 - a, r);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < RR; ++r) {
+      const int t = r * S + part;
+      if (32 * t + 31 > k0 - 3 && 32 * t < n) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) p[a] = fma(kKeep ? h[a][r] : at(k0 - a, r), z[r], p[a]);
+      }
+    }
+    double mine = warp_sum4_fx(p, lane);  // of reflector lane & 3
+    if (S > 1) {
+      double* ps = &part_sum[g & 1][0][0];
+      if (lane < 4) ps[4 * warp + lane] = mine;
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + cb), "r"(32 * S) : "memory");
+      mine = ps[4 * cb * S + (lane & 3)];
+#pragma unroll
+      for (int q = 1; q < S; ++q) mine += ps[4 * (cb * S + q) + (lane & 3)];
+    }
+    // s = T p: lane a & 3 holds row a
+    double sa = 0.0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const double pb = __shfl_sync(0xffffffffu, mine, b);
+      sa = fma(b == 0 ? t01.x : b == 1 ? t01.y : b == 2 ? t23.x : t23.y, pb, sa);
+    }
+    double s[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) s[a] = -__shfl_sync(0xffffffffu, sa, a);
+#pragma unroll
+    for (int r = 0; r < RR; ++r) {
+      const int t = r * S + part;
+      if (32 * t + 31 > k0 - 3 && 32 * t < n) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) z[r] = fma(s[a], kKeep ? h[a][r] : at(k0 - a, r), z[r]);
+      }
     }
   }
 #pragma unroll
-  for (int t = 0; t < R; ++t) {
-    const int i = lane + 32 * t;
-    if (i < n) zc[i] = z[t];
+  for (int r = 0; r < RR; ++r) {
+    const int i = lane + 32 * (r * S + part);
+    if (i < n) zc[i] = z[r];
   }
 }
 
@@ -1903,9 +2004,9 @@ bool launch_tridiag_xch(cudaStream_t s, int n, int num_sms, const double* M, dou
   return true;
 }
 
-template <int R>
-void launch_backtransform(cudaStream_t s, int n, const double* H, const double* tau, double* V) {
-  backtransform_reg_kernel<R><<<cdiv(n, 2), 64, 0, s>>>(n, H, tau, V);
+template <int RR, int S>
+void launch_backtransform(cudaStream_t s, int n, const double* H, const double* T, double* V) {
+  backtransform_reg_kernel<RR, S><<<cdiv(n, 4 / S), 128, 0, s>>>(n, H, T, V);
   RC_LAUNCH();
 }
 
@@ -1941,9 +2042,11 @@ int cholesky_inverse_f64(cudaStream_t s, int n, double* A, double* L, double* Li
 bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, DevBuf<double>& ws, int* d_flag,
                  int num_sms, const OzScratch* oz) {
   if (n < 1 || n > 3072) return false;
-  // workspace: H, S, V2 (n^2 each), d, e, tau, p (n each), xch (n + 8), tnorm, exchange packets
-  const size_t nn = (size_t)n * n;
-  double* H = ws.ensure(3 * nn + 6 * (size_t)n + 16 + tridiag_xch_ws(n));
+  // workspace: T (16 per group of four reflectors), H, S, V2 (n^2 each), d, e, tau, p (n each), xch (n + 8), tnorm,
+  // exchange packets
+  const size_t nn = (size_t)n * n, tn = ((size_t)(n + 3) / 4 * 16 + 31) / 32 * 32;
+  double* T = ws.ensure(tn + 3 * nn + 6 * (size_t)n + 16 + tridiag_xch_ws(n));
+  double* H = T + tn;
   double* S = H + nn;
   double* V2 = S + nn;
   double* d = V2 + nn;
@@ -2013,16 +2116,21 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
   gemm_f64(s, n, n, n, V2, n, false, S, n, true, z);
   }
   // 5. V = Q Z
-  const int R = (n + 31) / 32;
-  if (R <= 2) launch_backtransform<2>(s, n, H, tau, V);
-  else if (R <= 4) launch_backtransform<4>(s, n, H, tau, V);
-  else if (R <= 8) launch_backtransform<8>(s, n, H, tau, V);
-  else if (R <= 16) launch_backtransform<16>(s, n, H, tau, V);
-  else if (R <= 32) launch_backtransform<32>(s, n, H, tau, V);
-  else {
+  if (n > 1024) {
     backtransform_kernel<<<cdiv(n, 2), 64, 0, s>>>(n, H, tau, V);
     RC_LAUNCH();
+    return true;
   }
+  if (n > 2) {
+    reflector_groups_kernel<<<(n - 2 + 3) / 4, 32, 0, s>>>(n, H, tau, T);
+    RC_LAUNCH();
+  }
+  if (n <= 64) launch_backtransform<1, 2>(s, n, H, T, V);
+  else if (n <= 128) launch_backtransform<1, 4>(s, n, H, T, V);
+  else if (n <= 152) launch_backtransform<2, 4>(s, n, H, T, V);
+  else if (n <= 320) launch_backtransform<5, 2>(s, n, H, T, V);
+  else if (n <= 640) launch_backtransform<20, 1>(s, n, H, T, V);
+  else launch_backtransform<32, 1>(s, n, H, T, V);
   return true;
 }
 
