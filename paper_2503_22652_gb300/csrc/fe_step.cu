@@ -472,6 +472,358 @@ __global__ void __launch_bounds__(kThreads, 1) fe_step_kernel(const __grid_const
   }
 }
 
+// ---------------------------------------------------------------- the transposed step
+// The same step with the block's columns as the rows of the MMA: D^T (128 columns x 128 nodes) = T^T + V_c^T
+// (A_c D_c^-1)^T.  V_c^T is the A operand and lives in TMEM (lane = column), so a converter thread reads its
+// column of the staged rows (a warp reads 128 consecutive bytes per row) and writes it with tcgen05.st: no
+// rewriting of the stage into a K-major image, no barrier among the converters, and the stage is free as soon
+// as it has been read.  The cell image is the B operand as it stands (K-major).  In the epilogue a warp holds
+// 32 consecutive columns of one node, so every red is a whole 128-byte line.
+//   warp 0      cell images in four 32-wide K blocks, each refilled as soon as the last tile's MMAs on it are done
+//   warp 1      MMA issuer (M = 128 columns, N = 128 nodes)
+//   warps 2-9   convert: TMEM quarter w % 4 = 32 columns, half of the nodes each
+//   warps 10-17 epilogue: the same quarters, half of the nodes each
+//   warps 18-21 gather: half tiles of 64 columns into a ring of stages
+// At 16^3 cells x 600 columns the step above took 857 us, and 610 us without any of its gathers and reds: its
+// chain of conversion, barrier and rewriting was the bound, not memory (0.41 ms at the copy rate).  This one takes
+// 533 us there; below about 64 columns, where half of its 128 lanes are idle, the other is faster (6^3 x 48: 11.0
+// against 13 us), so both stand and fe_step_tune picks by time.
+constexpr int kTThreads = 704;
+constexpr int kTGather = 128;
+constexpr int kTStages = 3;
+constexpr uint32_t kTV = kNCP * 256;                    // 128 rows x 64 FP32
+constexpr uint32_t kTStage = kTV + (kWRows + 1) * 256;  // the owned rows of W and a row of zeros
+constexpr uint32_t kABlock = kABytes / 4;               // 32 K values of the cell image
+constexpr int kTab = 4;                                 // cells whose tables are held
+
+struct CellTab {
+  int dof[kNCP];
+  int orow[kWRows];   // dofs of the owned rows, in compact order
+  uint8_t pos[kNCP];  // row of W in the stage: compact position of an owned node, else the row of zeros
+};
+constexpr size_t kTSmem = kABytes + kTStages * ((size_t)kTStage + 64 * 4) + kTab * sizeof(CellTab) + 1024;
+
+// (predicated inside: a branch around each add made an add wait for the address of the one before, 130 clocks)
+__device__ __forceinline__ void red_add_f32(float* p, float a, bool on) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p red.global.add.f32 [%0], %1;\n}" ::"l"(p), "f"(a),
+               "r"((uint32_t)on)
+               : "memory");
+}
+
+// D[tmem] += A[tmem] * B[smem]^T, TF32.
+__device__ __forceinline__ void mma_tf32_ts(uint32_t d, uint32_t a, uint64_t b_desc, uint32_t idesc) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, 1, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+      "r"(a), "l"(b_desc), "r"(idesc)
+      : "memory");
+}
+
+__global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_constant__ StepBatch p) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t afull[4], aempty[4], bfull[kTStages], bempty[kTStages], ifull[2], accfull[2],
+      accempty[2], tfree[kTab], mma_done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sA = smem;
+  uint8_t* sB = smem + kABytes;
+  float* sL = reinterpret_cast<float*>(sB + (size_t)kTStages * kTStage);  // Lambda of each stage's columns
+  CellTab* tabs = reinterpret_cast<CellTab*>(sL + kTStages * 64);
+  for (int i = threadIdx.x; i < kTStages * 64; i += kTThreads)  // the rows of zeros
+    reinterpret_cast<float*>(sB + (size_t)(i / 64) * kTStage + kTV + kWRows * 256)[i % 64] = 0.f;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 4; ++i) {
+      tc::mbar_init(&afull[i], 1);
+      tc::mbar_init(&aempty[i], 1);
+    }
+    for (int i = 0; i < kTStages; ++i) {
+      tc::mbar_init(&bfull[i], kTGather + 1);  // every gathering thread's copies, and the cell's table
+      tc::mbar_init(&bempty[i], 128);          // the converters of the stage's 64 columns
+    }
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(&ifull[i], 256);
+      tc::mbar_init(&accfull[i], 1);
+      tc::mbar_init(&accempty[i], 256);
+    }
+    for (int i = 0; i < kTab; ++i) tc::mbar_init(&tfree[i], 8);
+    tc::mbar_init(&mma_done, 1);
+    tc::fence_barrier_init();
+    abort_flag = 0;
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(&tmem_slot, 512);
+    tc::tmem_relinquish();
+    tc::tc_fence_before();
+  }
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = tmem_slot;  // D of tile parity x at 128 x, the V operand at 256 + 128 x
+  volatile int* vabort = &abort_flag;
+  auto fail = [&]() {
+    *vabort = 1;
+    atomicExch(p.err, 1);
+  };
+  const int64_t G = gridDim.x;
+
+  if (warp == 0) {
+    // ---------------- cell images
+    if (lane == 0) {
+      int64_t cl = 0;
+      int issued = 0;
+      for (int64_t g = blockIdx.x; g < p.total_cells && !*vabort; g += G, ++cl) {
+        const StepPartDev& P = p.part[part_of(p, g)];
+        const uint8_t* src = P.img + (g - P.cell_off) * (int64_t)kABytes;
+        for (issued = 0; issued < 4; ++issued) {
+          if (*vabort || !tc::mbar_wait(&aempty[issued], (uint32_t)(cl & 1) ^ 1u)) {
+            fail();
+            break;
+          }
+          tc::mbar_arrive_expect_tx(&afull[issued], kABlock);
+          bulk_g2s(sA + (size_t)issued * kABlock, src + (size_t)issued * kABlock, kABlock, &afull[issued]);
+        }
+      }
+      if (*vabort) {  // copies already issued land before the shared memory is released (bounded)
+        // the last cell begun is cl - 1: blocks from `issued` on still hold the one before
+        for (int b = 0; b < 4; ++b) {
+          const int64_t c = b < issued ? cl - 1 : cl - 2;
+          if (c >= 0) tc::mbar_wait(&afull[b], (uint32_t)(c & 1));
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: accumulates onto the owner terms the converters stored
+    const bool leader = tc::elect_one();
+    constexpr uint32_t idesc = tc::instr_desc(2u, 128, kNCP);  // TF32, B K-major
+    const uint64_t b0 = tc::sw128_desc(tc::smem_u32(sA));
+    uint32_t j = 0, cl = 0;
+    bool stop = false;
+    for (int64_t g = blockIdx.x; g < p.total_cells && !stop; g += G, ++cl) {
+      const StepPartDev& P = p.part[part_of(p, g)];
+      const int ntiles = P.ntiles;
+      for (int t = 0; t < ntiles && !stop; ++t, ++j) {
+        const uint32_t xb = (uint32_t)(j & 1);
+        bool ok = !*vabort && tc::mbar_wait(&ifull[xb], (uint32_t)((j >> 1) & 1));
+        const uint32_t d = tmem + xb * 128u, a = tmem + 256u + xb * 128u;
+#pragma unroll
+        for (int kb = 0; kb < 4; ++kb) {
+          if (ok && t == 0) ok = tc::mbar_wait(&afull[kb], (uint32_t)(cl & 1));
+          if (kb == 0 || t == 0) {
+            if (!__all_sync(0xffffffffu, ok)) {
+              if (leader) fail();
+              stop = true;
+              break;
+            }
+            tc::tc_fence_after();
+          }
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            if (leader) mma_tf32_ts(d, a + (uint32_t)(kb * 32 + kk * 8), tc::desc_add(b0, kb * kABlock + kk * 32), idesc);
+          __syncwarp();
+          if (leader && t == ntiles - 1) tc::mma_commit(&aempty[kb]);
+          __syncwarp();
+        }
+        if (leader && !stop) tc::mma_commit(&accfull[xb]);
+        __syncwarp();
+      }
+    }
+    // every MMA issued has completed before TMEM is released
+    if (leader) {
+      tc::mma_commit(&mma_done);
+      tc::mbar_wait(&mma_done, 0u);
+    }
+    __syncwarp();
+  } else if (warp < 10) {
+    // ---------------- convert: this thread's column c of the tile, nodes k0 .. k0 + 63
+    const int q = warp & 3, k0 = 64 * ((warp - 2) >> 2), hp = q >> 1;
+    const int cs = (q & 1) * 32 + lane;  // column within the half tile
+    // (j: tiles so far, 32 bits and its low ones only; s0, ph0: stage and phase of the tile's first half)
+    uint32_t j = 0, cl = 0, ph0 = 0;
+    int s0 = 0;
+    bool stop = false;
+    for (int64_t g = blockIdx.x; g < p.total_cells && !stop; g += G, ++cl) {
+      const StepPartDev& P = p.part[part_of(p, g)];
+      const CellTab& tab = tabs[cl % kTab];
+      const int n = P.n, ntiles = P.ntiles;
+      float al = P.alpha, be = P.beta, om = P.omega;
+      if (P.coef) {
+        al = (float)__ldg(P.coef);
+        be = (float)__ldg(P.coef + 1);
+        om = (float)__ldg(P.coef + 2);
+      }
+      al *= P.sign;
+      const float rbe = be / al, rom = om / al;  // owner terms divided by alpha
+      for (int t = 0; t < ntiles; ++t, ++j) {
+        const int nh = n - 128 * t > 64 ? 2 : 1;  // half tiles
+        const uint32_t xb = (uint32_t)(j & 1);
+        bool ok = !*vabort && tc::mbar_wait(&accempty[xb], (uint32_t)((j >> 1) & 1) ^ 1u);
+        const bool wrap = s0 + hp >= kTStages;
+        const int s = wrap ? s0 + hp - kTStages : s0 + hp;
+        if (ok && hp < nh) ok = tc::mbar_wait(&bfull[s], ph0 ^ (wrap ? 1u : 0u));
+        if (!ok) fail();
+        if (!__all_sync(0xffffffffu, ok)) {
+          stop = true;
+          break;
+        }
+        tc::tc_fence_after();
+        if (hp < nh) {
+          const float* V = reinterpret_cast<const float*>(sB + (size_t)s * kTStage) + cs;
+          const uint8_t* W = reinterpret_cast<const uint8_t*>(V) + kTV;
+          const float rl = rom * sL[s * 64 + cs];
+          const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16) + xb * 128u + (uint32_t)k0;
+#pragma unroll
+          for (int kb = 0; kb < 64; kb += 16) {
+            float x[16], d[16];
+            const uint4 pk = *reinterpret_cast<const uint4*>(tab.pos + k0 + kb);
+            const uint32_t pw[4] = {pk.x, pk.y, pk.z, pk.w};
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              x[u] = V[(k0 + kb + u) * 64];
+              // byte u of the positions, times the 256 bytes of a row
+              d[u] = *reinterpret_cast<const float*>(W + __byte_perm(pw[u >> 2], 0, 0x4404u | (uint32_t)((u & 3) << 4)));
+            }
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+              const bool own = ((pw[u >> 2] >> (8 * (u & 3))) & 0xffu) != (uint32_t)kWRows;
+              d[u] = fmaf(rl, d[u], own ? rbe * x[u] : 0.f);
+              x[u] = tf32_rna(x[u]);
+            }
+            tc::tmem_st16(lane_addr + (uint32_t)kb, d);
+            tc::tmem_st16(lane_addr + 256u + (uint32_t)kb, x);
+          }
+          tc::mbar_arrive(&bempty[s]);
+          tc::tmem_wait_st();
+          tc::tc_fence_before();
+        }
+        tc::mbar_arrive(&ifull[xb]);
+        s0 += nh;
+        if (s0 >= kTStages) {
+          s0 -= kTStages;
+          ph0 ^= 1u;
+        }
+      }
+    }
+  } else if (warp < 18) {
+    // ---------------- epilogue
+    const int q = warp & 3, k0 = 64 * ((warp - 10) >> 2);
+    uint32_t j = 0, cl = 0;
+    bool stop = false;
+    for (int64_t g = blockIdx.x; g < p.total_cells && !stop; g += G, ++cl) {
+      const StepPartDev& P = p.part[part_of(p, g)];
+      const CellTab& tab = tabs[cl % kTab];
+      const int nc = P.nc, n = P.n, ntiles = P.ntiles;
+      float al = P.coef ? (float)__ldg(P.coef) : P.alpha;
+      al *= P.sign;
+      for (int t = 0; t < ntiles; ++t, ++j) {
+        const uint32_t xb = (uint32_t)(j & 1);
+        const int col = 128 * t + q * 32 + lane;
+        // (ifull: the acquire that makes the cell's table visible here)
+        bool ok = !*vabort && tc::mbar_wait(&ifull[xb], (uint32_t)((j >> 1) & 1)) &&
+                  tc::mbar_wait(&accfull[xb], (uint32_t)((j >> 1) & 1));
+        if (!ok) fail();
+        if (!__all_sync(0xffffffffu, ok)) {
+          stop = true;
+          break;
+        }
+        tc::tc_fence_after();
+        if (128 * t + q * 32 < n) {
+          const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + xb * 128u + (uint32_t)k0;
+          float* U = P.U + col;
+#pragma unroll
+          for (int kb = 0; kb < 64; kb += 16) {
+            float v[16];
+            tc::tmem_ld16(taddr + (uint32_t)kb, v);
+            int dof[16];
+#pragma unroll
+            for (int u = 0; u < 16; u += 4) *reinterpret_cast<int4*>(dof + u) = *reinterpret_cast<const int4*>(tab.dof + k0 + kb + u);
+#pragma unroll
+            for (int u = 0; u < 16; ++u)
+              red_add_f32(U + (int64_t)dof[u] * n, al * v[u], col < n && k0 + kb + u < nc);
+          }
+        }
+        tc::tc_fence_before();
+        tc::mbar_arrive(&accempty[xb]);
+      }
+      __syncwarp();
+      if (lane == 0 && !stop) tc::mbar_arrive(&tfree[cl % kTab]);
+    }
+  } else {
+    // ---------------- gather: 16 lanes copy one 256-byte row segment
+    const int gt = threadIdx.x - 576;
+    const int ch = gt & 15, r0 = gt >> 4;
+    uint32_t cl = 0, ph = 1;  // ph: phase parity that frees stage s
+    int s = 0;
+    bool stop = false;
+    for (int64_t g = blockIdx.x; g < p.total_cells; g += G, ++cl) {
+      const StepPartDev& P = p.part[part_of(p, g)];
+      const int64_t cell = g - P.cell_off;
+      CellTab& tab = tabs[cl % kTab];
+      const int nc = P.nc, n = P.n;
+      // the cell's tables, once its predecessor in the same place is done with
+      bool ok = !stop && !*vabort && tc::mbar_wait(&tfree[cl % kTab], (uint32_t)((cl / kTab) & 1) ^ 1u);
+      int o = -1;
+      if (ok) {
+        const int d = __ldg(P.dofs + cell * nc + min(gt, nc - 1));  // padding rows repeat
+        if (P.owner && gt < nc) o = (int)__ldg(P.own_pos + cell * kNCP + gt);
+        tab.dof[gt] = d;
+        tab.pos[gt] = (uint8_t)(o >= 0 ? o : kWRows);
+        if (o >= 0) tab.orow[o] = d;
+      }
+      // barriers of the gather warps: owned rows of the cell, and whether any thread gave up
+      uint32_t nown, bad;
+      asm volatile("{\n.reg .pred q;\nsetp.ge.s32 q, %1, 0;\nbarrier.cta.red.popc.u32 %0, 2, 128, q;\n}"
+                   : "=r"(nown)
+                   : "r"(o)
+                   : "memory");
+      asm volatile("{\n.reg .pred q;\nsetp.ne.s32 q, %1, 0;\nbarrier.cta.red.popc.u32 %0, 2, 128, q;\n}"
+                   : "=r"(bad)
+                   : "r"((int)!ok)
+                   : "memory");
+      if (bad) {
+        fail();
+        break;
+      }
+      int rows[kNCP / 8];
+#pragma unroll
+      for (int i = 0; i < kNCP / 8; ++i) rows[i] = tab.dof[r0 + 8 * i];
+      for (int hs = 0; hs * 64 < n; ++hs) {
+        if (*vabort || !tc::mbar_wait(&bempty[s], ph)) {
+          fail();
+          stop = true;  // (the gather warps leave together, at the vote of the next cell)
+          break;
+        }
+        const int col = hs * 64 + 4 * ch;
+        const bool in = col < n;
+        const float* Vc = P.V + (in ? col : 0);
+        const float* Wc = P.W + (in ? col : 0);
+        uint8_t* dst = sB + (size_t)s * kTStage + r0 * 256 + ch * 16;
+#pragma unroll
+        for (int i = 0; i < kNCP / 8; ++i)  // (rows of padding nodes: zeros)
+          cp_async16(dst + i * 2048, Vc + (int64_t)rows[i] * n, in && r0 + 8 * i < nc);
+        for (int r = r0; r < (int)nown; r += 8)
+          cp_async16(dst + kTV + (r - r0) * 256, Wc + (int64_t)tab.orow[r] * n, in);
+        if (gt < 16) cp_async16(sL + s * 64 + 4 * gt, P.lam + (in ? col : 0), in);
+        cp_async_arrive_noinc(&bfull[s]);
+        if (gt == 0) tc::mbar_arrive(&bfull[s]);
+        if (++s == kTStages) {
+          s = 0;
+          ph ^= 1u;
+        }
+      }
+    }
+    // copies still in flight land before the shared memory is released
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, 512);
+  }
+}
+
 // Shared-memory plan of a tile width: cell-image buffers and stages (V rows, owned W rows) that fit.
 struct Plan {
   int nA, nslots;
@@ -546,8 +898,9 @@ int fe_step_parts(FeOp& op, const float* V, const float* W, float* U, const floa
 
 void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, int num_sms) {
   RC_CHECK(nparts >= 1 && nparts <= kMaxParts, RCHFSI_ERR_INVALID_ARG, "fused FE step: 1..64 parts per launch");
-  RC_CHECK(BN == 32 || BN == 64 || BN == 96, RCHFSI_ERR_INVALID_ARG, "fused FE step: column tile of 32, 64 or 96");
-  const Plan pl = make_plan(BN);
+  RC_CHECK(BN == 32 || BN == 64 || BN == 96 || BN == 128, RCHFSI_ERR_INVALID_ARG,
+           "fused FE step: column tile of 32, 64, 96 or 128");
+  const Plan pl = BN == 128 ? Plan{1, kTStages, kTSmem} : make_plan(BN);
   RC_CHECK(pl.nA > 0, RCHFSI_ERR_INVALID_ARG, "fused FE step: no shared-memory plan for this tile");
   StepBatch b{};
   b.nparts = nparts;
@@ -599,6 +952,11 @@ void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, 
   switch (BN) {
     case 32: launch<32>(s, b, pl, grid); break;
     case 64: launch<64>(s, b, pl, grid); break;
+    case 128:
+      set_smem_limit(reinterpret_cast<const void*>(fe_step_t_kernel), kSmemMax - 512);
+      fe_step_t_kernel<<<grid, kTThreads, kTSmem, s>>>(b);
+      RC_LAUNCH();
+      break;
     default: launch<96>(s, b, pl, grid); break;
   }
 }
@@ -613,6 +971,7 @@ int fe_step_tune(cudaStream_t s, int num_sms, FeOp& op, int n, const float* V, c
   std::vector<int> cand;
   for (int bn : {32, 64, 96})
     if (bn <= std::max(32, (n + 31) / 32 * 32) && make_plan(bn).nA > 0) cand.push_back(bn);
+  cand.push_back(128);
   DevBuf<float> scratch;
   float* out = scratch.ensure((size_t)op.m * n);
   cudaEvent_t e0, e1;
