@@ -1533,76 +1533,68 @@ __global__ void __launch_bounds__(32 * TE_WARPS) tri_eig_kernel(int n, const dou
 }
 
 // ------------------------------------------------------------------ tridiagonal eigenvectors
-// LU factorisation with partial pivoting of T - lam I (one thread).  Row i of U holds u0 (diagonal),
-// u1, u2 (first and second superdiagonals); mult/sw record the elimination of row i + 1.
-__device__ void tri_lu(int n, const double* d, const double* e, double lam, double small, double* u0, double* u1,
+// LU factorisation with partial pivoting of T - lam I, one matrix per lane: the pivoting is by selects, so that the
+// lanes of a warp factor the matrices of a cluster's members in the time of one.  Row i of U is 1 / u0 (u0inv, the
+// pivot clamped away from zero), u1, u2 (first and second superdiagonals); mult/sw record the elimination of
+// row i + 1.
+__device__ void tri_lu(int n, const double* d, const double* e, double lam, double small, double* u0inv, double* u1,
                        double* u2, double* mult, int* sw) {
-  for (int i = 0; i < n; ++i) {
-    u0[i] = d[i] - lam;
-    u1[i] = i + 1 < n ? e[i] : 0.0;
-    u2[i] = 0.0;
-  }
+  double p0 = d[0] - lam, p1 = e[0];  // the current row
+  auto inv = [&](double u) {
+    const double a = fabs(u) < small ? small : fabs(u);
+    return copysign(rcp_h3(a), u);
+  };
   for (int i = 0; i + 1 < n; ++i) {
     const double c = e[i];  // subdiagonal entry (i + 1, i)
-    if (fabs(u0[i]) >= fabs(c)) {
-      if (u0[i] == 0.0) u0[i] = small;
-      const double m = c / u0[i];
-      mult[i] = m;
-      sw[i] = 0;
-      u0[i + 1] -= m * u1[i];
-    } else {
-      // exchange rows i and i + 1, then eliminate
-      const double m = u0[i] / c;
-      mult[i] = m;
-      sw[i] = 1;
-      const double r0 = u1[i];   // old row i: (u0, u1, 0) at columns i, i+1, i+2
-      const double a1 = u0[i + 1], b1 = u1[i + 1];
-      u0[i] = c;
-      u1[i] = a1;
-      u2[i] = b1;
-      u0[i + 1] = r0 - m * a1;
-      u1[i + 1] = -m * b1;
-    }
+    const double a1 = d[i + 1] - lam, b1 = e[i + 1];
+    const bool swap = fabs(p0) < fabs(c);
+    const double piv = swap ? c : p0, r = inv(piv);
+    const double q1 = swap ? a1 : p1;
+    const double m = (swap ? p0 : c) * r;
+    u0inv[i] = r;
+    u1[i] = q1;
+    u2[i] = swap ? b1 : 0.0;
+    mult[i] = m;
+    sw[i] = swap ? 1 : 0;
+    p0 = fma(-m, q1, swap ? p1 : a1);
+    p1 = swap ? -m * b1 : b1;
   }
-  if (u0[n - 1] == 0.0) u0[n - 1] = small;
-  // keep the reciprocals of the pivots (clamped away from zero) so the solves need no divide
-  for (int i = 0; i < n; ++i) {
-    double u = u0[i];
-    if (fabs(u) < small) u = u >= 0.0 ? small : -small;
-    u0[i] = 1.0 / u;
-  }
+  u0inv[n - 1] = inv(p0);
+  u1[n - 1] = u2[n - 1] = 0.0;
 }
 
-// y <- (T - lam I)^-1 y with the factors of tri_lu (one thread; u0 holds the pivot reciprocals).
-__device__ void tri_solve(int n, const double* u0, const double* u1, const double* u2, const double* mult,
+// y <- (T - lam I)^-1 y with the factors of tri_lu (one system per lane).
+__device__ void tri_solve(int n, const double* u0inv, const double* u1, const double* u2, const double* mult,
                           const int* sw, double* y) {
+  double t = y[0];
   for (int i = 0; i + 1 < n; ++i) {
-    if (sw[i]) {
-      const double t = y[i];
-      y[i] = y[i + 1];
-      y[i + 1] = t - mult[i] * y[i];
-    } else {
-      y[i + 1] -= mult[i] * y[i];
-    }
+    const double v = y[i + 1], m = mult[i];
+    const bool s = sw[i] != 0;
+    y[i] = s ? v : t;
+    t = s ? fma(-m, v, t) : fma(-m, t, v);
   }
-  for (int i = n - 1; i >= 0; --i) {
-    double s = y[i];
-    if (i + 1 < n) s -= u1[i] * y[i + 1];
-    if (i + 2 < n) s -= u2[i] * y[i + 2];
-    y[i] = s * u0[i];
+  double y1 = t * u0inv[n - 1], y2 = 0.0;
+  y[n - 1] = y1;
+  for (int i = n - 2; i >= 0; --i) {
+    const double x = fma(-u1[i], y1, fma(-u2[i], y2, y[i])) * u0inv[i];
+    y[i] = x;
+    y2 = y1;
+    y1 = x;
   }
 }
 
 // One warp (one CTA) per cluster of eigenvalues, a cluster being a run of eigenvalues with
 // consecutive gaps <= 1e-9 ||T|| (numerically degenerate, e.g. the pairs of a complex problem's
-// real embedding): inverse iteration for each member in turn, with Gram-Schmidt (twice) against the
+// real embedding): inverse iteration, `batch` members at a time (a lane each: the factorisation and the solves
+// are chains of FP64 instructions, and a pair of n = 192 took 530 us one member after the other), with
+// Gram-Schmidt (twice) against the
 // members already done.  Eigenvectors of better separated eigenvalues come out orthogonal to
 // O(eps ||T|| / gap); the caller removes that residue with one Newton-Schulz step.  The LU factors
-// and the iterate live in shared memory (6 n doubles).  Z (n x n, column-major) receives the unit
+// and the iterates live in shared memory (5.5 n doubles per member).  Z (n x n, column-major) receives the unit
 // eigenvectors of T.  A cluster larger than maxc sets *flag (the caller then uses another solver).
 __global__ void __launch_bounds__(32) inviter_kernel(int n, const double* __restrict__ d, const double* __restrict__ e,
                                                      const double* __restrict__ lam, const double* __restrict__ tnorm_p,
-                                                     double* Z, int maxc, int clusters_only, int* flag) {
+                                                     double* Z, int maxc, int clusters_only, int batch, int* flag) {
   extern __shared__ double sm[];
   const int j = blockIdx.x;
   const int lane = threadIdx.x & 31;
@@ -1617,60 +1609,63 @@ __global__ void __launch_bounds__(32) inviter_kernel(int n, const double* __rest
     if (lane == 0) atomicExch(flag, 1);
     return;
   }
-  const double small = DBL_EPSILON * fmax(tnorm, DBL_MIN);
-  double* u0 = sm;
-  double* u1 = u0 + n;
-  double* u2 = u1 + n;
-  double* mult = u2 + n;
-  double* y = mult + n;
-  int* sw = reinterpret_cast<int*>(y + n);
-  double* dd = reinterpret_cast<double*>(sw) + (n + 1) / 2;  // copies of d and e (n each)
+  const double small = fmax(DBL_EPSILON * tnorm, 4.0 * DBL_MIN);  // (its reciprocal is a normal number)
+  double* dd = sm;        // copies of d and e (n each)
   double* ee = dd + n;
+  double* fac = ee + n;   // per member of the batch: 1 / u0, u1, u2, mult (n each)
+  double* ys = fac + (size_t)batch * 4 * n;  // iterates
+  int* sws = reinterpret_cast<int*>(ys + (size_t)batch * n);
   for (int m = lane; m < n; m += 32) {
     dd[m] = d[m];
     ee[m] = m + 1 < n ? e[m] : 0.0;
   }
   __syncwarp();
-  for (int i = j; i < k; ++i) {
-    if (lane == 0) tri_lu(n, dd, ee, lam[i], small, u0, u1, u2, mult, sw);
-    // deterministic start vector with no structure shared with T
-    double nr = 0.0;
-    for (int m = lane; m < n; m += 32) {
-      const double v = cos(0.7548776662 * m + 1.3247179572 * (i - j) + 0.5) + 0.1;
-      y[m] = v;
-      nr += v * v;
-    }
-    nr = warp_sum(nr);
-    for (int m = lane; m < n; m += 32) y[m] *= rsqrt(nr);
+  for (int i0 = j; i0 < k; i0 += batch) {
+    const int nb = min(batch, k - i0);
+    double* f = fac + (size_t)min(lane, nb - 1) * 4 * n;
+    double* y = ys + (size_t)min(lane, nb - 1) * n;
+    int* sw = sws + (size_t)min(lane, nb - 1) * n;
+    if (lane < nb) tri_lu(n, dd, ee, lam[i0 + lane], small, f, f + n, f + 2 * n, f + 3 * n, sw);
+    // deterministic start vectors with no structure shared with T
+    for (int b = 0; b < nb; ++b)
+      for (int m = lane; m < n; m += 32)
+        ys[(size_t)b * n + m] = cosf(0.75487767f * (float)m + 1.3247180f * (float)(i0 + b - j) + 0.5f) + 0.1f;
     __syncwarp();
     // the shift is accurate to a few ulps, so two solves already give the eigenvector to round-off
     for (int it = 0; it < 2; ++it) {
-      if (lane == 0) tri_solve(n, u0, u1, u2, mult, sw, y);
+      if (lane < nb) tri_solve(n, f, f + n, f + 2 * n, f + 3 * n, sw, y);
       __syncwarp();
-      for (int rep = 0; rep < 2; ++rep) {
-        for (int l = j; l < i; ++l) {
-          const double* zl = Z + (size_t)l * n;
-          double dt = 0.0;
-          for (int m = lane; m < n; m += 32) dt += zl[m] * y[m];
-          dt = warp_sum(dt);
-          for (int m = lane; m < n; m += 32) y[m] -= dt * zl[m];
+      for (int b = 0; b < nb; ++b) {
+        double* yb = ys + (size_t)b * n;
+        // (unit length first: the solve has blown the vector up)
+        for (int rep = 0; rep < 3; ++rep) {
+          double nr = 0.0;
+          for (int m = lane; m < n; m += 32) nr = fma(yb[m], yb[m], nr);
+          nr = warp_sum(nr);
+          const double sc = 1.0 / sqrt(nr);
+          for (int m = lane; m < n; m += 32) yb[m] *= sc;
           __syncwarp();
+          if (rep == 2) break;
+          for (int l = j; l < i0 + b; ++l) {
+            const double* zl = l < i0 ? Z + (size_t)l * n : ys + (size_t)(l - i0) * n;
+            double dt = 0.0;
+            for (int m = lane; m < n; m += 32) dt = fma(zl[m], yb[m], dt);
+            dt = warp_sum(dt);
+            for (int m = lane; m < n; m += 32) yb[m] = fma(-dt, zl[m], yb[m]);
+            __syncwarp();
+          }
         }
       }
-      nr = 0.0;
-      for (int m = lane; m < n; m += 32) nr += y[m] * y[m];
-      nr = warp_sum(nr);
-      const double sc = 1.0 / sqrt(nr);
-      for (int m = lane; m < n; m += 32) y[m] *= sc;
-      __syncwarp();
     }
-    double* zi = Z + (size_t)i * n;
-    for (int m = lane; m < n; m += 32) zi[m] = y[m];
+    for (int b = 0; b < nb; ++b) {
+      double* zi = Z + (size_t)(i0 + b) * n;
+      for (int m = lane; m < n; m += 32) zi[m] = ys[(size_t)b * n + m];
+    }
     __syncwarp();
   }
 }
 
-size_t inviter_smem(int n) { return (8 * (size_t)n + 1) * sizeof(double); }
+size_t inviter_smem(int n, int batch) { return (2 * (size_t)n + (size_t)batch * 5 * n + ((size_t)batch * n + 1) / 2) * sizeof(double); }
 
 // Four warp sums at once: lane l receives the sum of v[l & 3], one conversion for all four.
 __device__ __forceinline__ double warp_sum4_fx(const double (&v)[4], int lane) {
@@ -2081,7 +2076,10 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
   }
   RC_LAUNCH();
   set_smem_limit(reinterpret_cast<const void*>(inviter_kernel), (int)SMEM_CAP);
-  inviter_kernel<<<n, 32, inviter_smem(n), s>>>(n, d, e, evals, tnorm, V2, INV_MAX_CLUSTER, pairs ? 1 : 0, d_flag);
+  int batch = 4;
+  while (batch > 1 && inviter_smem(n, batch) > 48 * 1024) --batch;
+  inviter_kernel<<<n, 32, inviter_smem(n, batch), s>>>(n, d, e, evals, tnorm, V2, INV_MAX_CLUSTER, pairs ? 1 : 0, batch,
+                                                       d_flag);
   RC_LAUNCH();
   // 4. one Newton-Schulz step towards the orthogonal factor: Z <- Z (3 I - Z^T Z) / 2
   if (oz && n <= kSmallGemmMaxN) {
