@@ -28,7 +28,7 @@
 //              longer read, so each pass ends with two commits: "level s done" and "slice 6-s free".
 //              TMEM holds 8 level blocks of 64 columns: 7 for the item, one spare, rotated so that
 //              the next item's first writes go to blocks in the order the epilogue frees them;
-//   warps 2-3  gather (two dof rows each): 16-byte cp.async of the rows' 64 columns of each slice
+//   warps 2-3  gather: 16-byte cp.async, eight lanes per row, of the rows' 64 columns of each slice
 //              plane into the MN-major 128-byte-swizzled image X_c^(t), slice by slice as the
 //              previous item releases them (slice 0, freed last, alternates between two images);
 //   warps 4-19 epilogue (four per TMEM lane quarter, 16 columns each): folds level L into a
@@ -503,35 +503,51 @@ __global__ void __launch_bounds__(kThreads, 1) fe_oz_kernel(const __grid_constan
     for (int64_t j = 0; j < items && ok; ++j) {
 #pragma unroll
       for (int s = 0; s < S; ++s) {
-        bool w = !*vabort && tc::mbar_wait(&afull[q], qpar);
+        const bool w = !*vabort && tc::mbar_wait(&afull[q], qpar);
         ok = __all_sync(0xffffffffu, w);
         if (!ok) break;
         tc::tc_fence_after();
         const uint64_t a0 = tc::sw128_desc(tc::smem_u32(sA + (size_t)q * kASlice));
-#pragma unroll
-        for (int u = 0; u < S - s; ++u) {
-          // pass 0 takes the X slices in the order the gather refills them (0, 6, 5, .., 1) and
-          // makes the first write of each level, into a block the epilogue has released
-          const int t = (s == 0) ? (u == 0 ? 0 : S - u) : u;
-          const uint32_t blk = perm_block(perm, s + t);
-          if (s == 0) {
-            w = !*vabort && tc::mbar_wait(&xfull[x_block(t, j)], x_par(t, j));
-            if (w) w = tc::mbar_wait(&bfree[blk], ((use_par >> blk) & 1u) ^ 1u);
-            ok = __all_sync(0xffffffffu, w);
-            if (!ok) break;
-            use_par ^= 1u << blk;
-            tc::tc_fence_after();
-          }
-          const uint32_t d = tmem + blk * (uint32_t)kBN;
-          const uint64_t x0 = tc::desc_add(x_desc, (uint32_t)x_block(t, j) * kXSlice);
+        // a run of MMAs takes one A tile (16 K values) against X slices t0, t0 - 1, .. or 0, 1, ..; the tile
+        // stays in the collector, so shared memory is read for X only
+        auto run = [&](int n, auto slice) {
 #pragma unroll
           for (int kk = 0; kk < kNCP / 16; ++kk) {
             const int kel = kk * 16;
             const uint32_t aoff = (uint32_t)(kel >> 6) * kNCP * kRowBytes + (uint32_t)((kel & 63) * 2);
-            // MN-major X: 16 K rows (two 1024-byte atoms) per MMA
-            if (leader)
-              tc::mma_f16(d, tc::desc_add(a0, aoff), tc::desc_add(x0, (uint32_t)kk * 2048u), idesc,
-                          (s == 0 && kk == 0) ? 0u : 1u);
+#pragma unroll
+            for (int u = 0; u < n; ++u) {
+              const int t = slice(u);
+              // MN-major X: 16 K rows (two 1024-byte atoms) per MMA
+              tc::mma_f16_run(leader, u, n, tmem + perm_block(perm, s + t) * (uint32_t)kBN, tc::desc_add(a0, aoff),
+                              tc::desc_add(x_desc, (uint32_t)x_block(t, j) * kXSlice + (uint32_t)kk * 2048u), idesc,
+                              (s == 0 && kk == 0) ? 0u : 1u);
+            }
+          }
+        };
+        if (s > 0) {
+          run(S - s, [](int u) { return u; });
+        } else {
+          // pass 0 takes the X slices in the order the gather refills them (0, 6, 5, .., 1) and makes the first
+          // write of each level, into a block the epilogue has released; in three runs, so that it starts
+          // before all of them are there
+#pragma unroll
+          for (int r = 0; r < 3; ++r) {
+            const int u0 = r == 0 ? 0 : r == 1 ? 3 : 5, n = r == 0 ? 3 : 2;
+            bool w2 = true;
+#pragma unroll
+            for (int u = u0; u < u0 + n; ++u) {
+              const int t = u == 0 ? 0 : S - u;
+              const uint32_t blk = perm_block(perm, t);
+              w2 = w2 && tc::mbar_wait(&xfull[x_block(t, j)], x_par(t, j));
+              // blocks are released in the order of t: the run's last stands for all
+              if (u == u0 + n - 1) w2 = w2 && tc::mbar_wait(&bfree[blk], ((use_par >> blk) & 1u) ^ 1u);
+              use_par ^= 1u << blk;
+            }
+            ok = __all_sync(0xffffffffu, w2);
+            if (!ok) break;
+            tc::tc_fence_after();
+            run(n, [u0](int u) { return u0 + u == 0 ? 0 : S - (u0 + u); });
           }
         }
         if (!ok) break;
@@ -558,49 +574,58 @@ __global__ void __launch_bounds__(kThreads, 1) fe_oz_kernel(const __grid_constan
     __syncwarp();
     tc::mbar_wait(&mdone, 0);
   } else if (warp < 4) {
-    // ---------------- gather: thread k copies dofs k and k + 64, 64 columns of every slice plane
-    // (zeros for the padding rows >= n_c), slice 0 first (its block was freed two items ago), then
+    // ---------------- gather: eight lanes copy the 128 bytes of one row of a slice plane (a warp instruction
+    // touches four whole lines; with a lane per row it touched 32, and every line eight times), zeros for
+    // the padding rows >= n_c; slice 0 first (its block was freed two items ago), then
     // 6, 5, .., 1 as the previous item releases them.  A slice is signalled once its copies have
     // landed: wait for all but the newest group, make the writes visible to the tensor cores, arrive.
-    const int k = threadIdx.x - 64;  // 0 .. 63
-    const uint32_t xs = tc::smem_u32(sX);
+    const int gt = threadIdx.x - 64;  // 0 .. 63
+    const int c = gt & 7, r0 = gt >> 3;
+    const uint32_t xs = tc::smem_u32(sX) + mn_chunk_off(r0, c);  // rows r0 + 8 i: 1024 bytes apart
+    int dof[kNCP / 8];
     for (int64_t j = 0; j < items; ++j) {
-      const int64_t cell = blockIdx.x + (j / p.ntiles) * G;
       const int tile = (int)(j % p.ntiles);
-      const __nv_bfloat16* src0[2];
-      bool in[2];
+      if (tile == 0) {
+        const int64_t cell = blockIdx.x + (j / p.ntiles) * G;
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const int kr = k + 64 * r;
-        const int g = (kr < p.nc) ? __ldg(p.dofs + cell * p.nc + kr) : -1;
-        in[r] = g >= 0;
-        src0[r] = p.planes + (in[r] ? (int64_t)g * p.np + (int64_t)tile * kBN : 0);
+        for (int i = 0; i < kNCP / 8; ++i) {
+          const int kr = r0 + 8 * i;
+          dof[i] = (kr < p.nc) ? __ldg(p.dofs + cell * p.nc + kr) : -1;
+        }
       }
       bool ok = true;
       int prev = -1;
+      auto signal = [&]() {
+        fence_proxy_async();
+        tc::mbar_arrive(&xfull[prev]);
+        prev = -1;
+      };
       for (int u = 0; u < S; ++u) {
         const int t = (u == 0) ? 0 : S - u;
         const int b = x_block(t, j);
         // slice t >= 1 is free once pass 6 - t of the previous item is done; slice 0's block once
         // the item before that is done
-        const bool freed = t ? (j == 0 || tc::mbar_wait(&lev[(j - 1) & 1][S - 1 - t], (uint32_t)(((j - 1) >> 1) & 1)))
-                             : tc::mbar_wait(&xempty[b], x_par(0, j) ^ 1u);
-        if (*vabort || !freed) {
-          ok = false;
-          break;
+        uint64_t* bar = t ? &lev[(j - 1) & 1][S - 1 - t] : &xempty[b];
+        const uint32_t par = t ? (uint32_t)(((j - 1) >> 1) & 1) : x_par(0, j) ^ 1u;
+        if (!(t && j == 0) && !tc::mbar_try_wait(bar, par)) {
+          if (prev >= 0) {  // a wait: the copies issued so far are signalled first
+            cp_async_wait<0>();
+            signal();
+          }
+          if (*vabort || !tc::mbar_wait(bar, par)) {
+            ok = false;
+            break;
+          }
         }
         const uint32_t dst = xs + (uint32_t)b * kXSlice;
+        const __nv_bfloat16* src = p.planes + (int64_t)t * p.plane_stride + (int64_t)tile * kBN + 8 * c;
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const __nv_bfloat16* src = src0[r] + (int64_t)t * p.plane_stride;
-#pragma unroll
-          for (int c = 0; c < kBN / 8; ++c) cp_async16(dst + mn_chunk_off(k + 64 * r, c), src + 8 * c, in[r]);
-        }
+        for (int i = 0; i < kNCP / 8; ++i)
+          cp_async16(dst + i * 1024u, src + (int64_t)max(dof[i], 0) * p.np, dof[i] >= 0);
         cp_async_commit();
         if (prev >= 0) {
           cp_async_wait<1>();
-          fence_proxy_async();
-          tc::mbar_arrive(&xfull[prev]);
+          signal();
         }
         prev = b;
       }
@@ -609,8 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1) fe_oz_kernel(const __grid_constan
         fail();
         break;
       }
-      fence_proxy_async();
-      tc::mbar_arrive(&xfull[prev]);
+      signal();
     }
   } else {
     // ---------------- epilogue: fold level L as soon as pass L is done and release its block,
