@@ -263,10 +263,11 @@ static void dense_step_lowp(rchfsi_ctx& c, bool chfsi, int prec, const void* Ry,
 
 // Tables of the one-launch degree loop (tc_loop.cu), behind the Lambda table in the same upload: the
 // coefficients and Lambda values of each step in FP32 and the zeroed counters.
+// (also, but for the coefficients, of the FE degree loop of fe_step.cu)
 struct LoopTables {
   const float* coef = nullptr;
-  const float* lam = nullptr;
-  int* counters = nullptr;
+  const float* lam = nullptr;  // row 1 of the table, N values per row
+  int* counters = nullptr;     // null: no one-launch loop
 };
 
 static void filter_dense(rchfsi_ctx& c, const double* X, const double* W, int p, const double* lamtab, double e,
@@ -425,7 +426,8 @@ static void filter_dense(rchfsi_ctx& c, const double* X, const double* W, int p,
 
 // rows: X, W and Y are row-major, as callers hold them, instead of column-major (not with FP64).
 static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, const double* lamtab, double e,
-                      double cc, double s1, const std::vector<Coef>& co, double* Y, bool chfsi, bool rows) {
+                      double cc, double s1, const std::vector<Coef>& co, double* Y, bool chfsi, bool rows,
+                      const LoopTables& ls) {
   const int64_t m = c.p.m;
   const int N = c.p.block;
   const size_t blk = (size_t)m * N;
@@ -479,17 +481,29 @@ static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, co
     // S_1 = W and W, row-major FP32, in one pass over W
     enter(W, 1.0, RY, Wl);
     fill_zero(c.s, RX, blk * sizeof(float));  // S_0 = R_0 = 0
-    if (!co.empty()) {
+    if (!co.empty() && ls.counters) {
+      // all degree steps in one launch
+      std::vector<float> cf(3 * co.size());
+      for (int k = 2; k <= p; ++k) {
+        double q[3];
+        fused_coefs(co, sc, k, q);
+        for (int u = 0; u < 3; ++u) cf[3 * (k - 2) + u] = (float)q[u];
+      }
+      FeStepPart parts[4];
+      const int np = fe_step_parts(f, RY, Wl, RX, ls.lam, N, cf[0], cf[1], cf[2], nullptr, parts);
+      const FeStepLoop loop{(int)co.size(), cf.data(), RY, RX, ls.counters};
+      fe_step_batch(c.s, parts, np, 128, c.num_sms, &loop);
+      if (co.size() % 2) std::swap(RX, RY);
+    } else if (!co.empty()) {
       float* lamf = c.w.lamtab_f.ensure((size_t)(p + 1) * N);  // the Lambda table in FP32 for the kernel
       cast_f64_to_f32(c.s, (int64_t)(p + 1) * N, lamtab, lamf, 1.0, 0);
-      const int BN = fe_step_tune(c.s, c.num_sms, f, N, RY, Wl, lamf + N);
       for (int k = 2; k <= p; ++k) {
         double cf[3];
         fused_coefs(co, sc, k, cf);
         FeStepPart parts[4];
         const int np = fe_step_parts(f, RY, Wl, RX, lamf + (size_t)(k - 1) * N, N, (float)cf[0], (float)cf[1],
                                      (float)cf[2], nullptr, parts);
-        fe_step_batch(c.s, parts, np, BN, c.num_sms);
+        fe_step_batch(c.s, parts, np, 128, c.num_sms);
         std::swap(RX, RY);
       }
     }
@@ -547,17 +561,24 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
       loop.ok = false;
     if (loop.ok) c.w.split.ensure(loop.ws_floats);
   }
-  // one buffer: the Lambda table, and for the loop the coefficients and Lambda rows 1 .. p - 1 in FP32 and the
+  // the fused FE steps likewise, whatever the mesh
+  const bool fe_loop = c.op_kind == RCHFSI_OP_FE_CELL && !chfsi && p >= 2 && p - 1 <= kTableSteps &&
+                       fe_step_supported(*c.fe, N, c.p.precision);
+  // one buffer: the Lambda table, and for a loop the coefficients and Lambda rows 1 .. p - 1 in FP32 and the
   // counters on 128-byte lines
+  const bool tables = loop.ok || fe_loop;
   const size_t coef_at = (size_t)(p + 1) * N;
-  const size_t floats = loop.ok ? 3 * (size_t)loop_steps + (chfsi ? 0 : (size_t)loop_steps * N) : 0;
-  const size_t cnt_at = (coef_at + (floats + 1) / 2 + 15) / 16 * 16;
-  const size_t total = loop.ok ? cnt_at + loop.counters / 2 : coef_at;
+  const size_t ncoef = tables ? ((size_t)3 * loop_steps + 3) / 4 * 4 : 0;  // (the rows start on 16 bytes)
+  const size_t floats = tables ? ncoef + (chfsi ? 0 : (size_t)loop_steps * N) : 0;
+  const size_t lam_at = (coef_at + 1) / 2 * 2;
+  const size_t cnt_at = (lam_at + (floats + 1) / 2 + 15) / 16 * 16;
+  const size_t ncnt = loop.ok ? loop.counters : fe_loop ? 32 : 0;
+  const size_t total = tables ? cnt_at + ncnt / 2 : coef_at;
   double* dtab = c.w.lamtab.ensure(total);
   LoopTables ls;
-  if (loop.ok) {
-    ls.coef = reinterpret_cast<const float*>(dtab + coef_at);
-    ls.lam = ls.coef + 3 * (size_t)loop_steps;
+  if (tables) {
+    ls.coef = reinterpret_cast<const float*>(dtab + lam_at);
+    ls.lam = ls.coef + ncoef;
     ls.counters = reinterpret_cast<int*>(dtab + cnt_at);
   }
   std::vector<double> tab;
@@ -578,7 +599,7 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
     t.coef = const_cast<float*>(ls.coef);
     t.lamf = const_cast<float*>(ls.lam);
     t.counters = ls.counters;
-    t.ncounters = loop.ok ? (int)loop.counters : 0;
+    t.ncounters = (int)ncnt;
     filter_tables(c.s, t);
   } else {
     if (chfsi) {
@@ -594,8 +615,8 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
       lambda_table(lam, N, e, cc, s1, co, tab);
       tab.resize(total, 0.0);
     }
-    if (loop.ok) {
-      float* f = reinterpret_cast<float*>(tab.data() + coef_at);
+    if (tables) {
+      float* f = reinterpret_cast<float*>(tab.data() + lam_at);
       int o = 0;
       if (chfsi) {
         f[o++] = (float)(s1 / e);
@@ -608,7 +629,7 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
         f[o++] = (float)q.c;
       }
       if (!chfsi)
-        for (size_t t = 0; t < (size_t)loop_steps * N; ++t) f[o + t] = (float)tab[(size_t)N + t];
+        for (size_t t = 0; t < (size_t)loop_steps * N; ++t) f[ncoef + t] = (float)tab[(size_t)N + t];
     }
     RC_CUDA(cudaMemcpyAsync(dtab, tab.data(), total * sizeof(double), cudaMemcpyHostToDevice, c.s));
   }
@@ -618,7 +639,7 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
   if (c.op_kind == RCHFSI_OP_DENSE)
     filter_dense(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi, loop, ls, rows);
   else
-    filter_fe(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi, rows);
+    filter_fe(c, X, W, p, dtab, e, cc, s1, co, Y, chfsi, rows, ls);
   // the host table must outlive the async copy; then read the kernels' timeout flag
   int flag = 0;
   RC_CUDA(cudaMemcpyAsync(&flag, c.w.info.p + 2, sizeof(int), cudaMemcpyDeviceToHost, c.s));

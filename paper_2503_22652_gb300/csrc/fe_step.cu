@@ -97,6 +97,8 @@ struct StepPartDev {
   int64_t n_cells, cell_off;
   float alpha, beta, omega, sign;
   int nc, n, ntiles, owner;  // owner = 0: no owner terms in this part
+  const float* V2;  // V and U of the odd steps of a loop
+  float* U2;
 };
 
 struct StepBatch {
@@ -105,6 +107,11 @@ struct StepBatch {
   int nparts, nA, nslots;
   uint32_t tmem_cols;
   int* err;
+  // a loop of degree steps (fe_step_t_kernel only, nsteps > 1): alpha, beta, omega per step in `coefs` in place of the
+  // parts' own, lam advances by n per step, and the CTAs meet between steps at the counter *sync
+  int nsteps;
+  int* sync;
+  float coefs[3 * kTableSteps];
 };
 
 __device__ __forceinline__ int part_of(const StepBatch& p, int64_t g) {
@@ -519,6 +526,33 @@ __device__ __forceinline__ void mma_tf32_ts(uint32_t d, uint32_t a, uint64_t b_d
       : "memory");
 }
 
+// The CTA's cells, step by step.
+struct StepCell {
+  int64_t g;
+  int st;
+  __device__ __forceinline__ bool first() const { return g == (int64_t)blockIdx.x; }
+  __device__ __forceinline__ bool last(const StepBatch& p) const { return g + gridDim.x >= p.total_cells; }
+  __device__ __forceinline__ void next(const StepBatch& p) {
+    g += gridDim.x;
+    if (g >= p.total_cells) {
+      g = blockIdx.x;
+      ++st;
+    }
+  }
+};
+
+// *p >= want (acquire), with the limit of the other waits; false also once another CTA has failed.
+__device__ __forceinline__ bool wait_steps(const int* p, int want, const int* err) {
+  const long long t0 = clock64();
+  for (int spin = 0;; ++spin) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    if (v >= want) return true;
+    if (clock64() - t0 > tc::kWaitCycles) return false;
+    if ((spin & 255) == 255 && *(volatile const int*)err) return false;
+  }
+}
+
 __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_constant__ StepBatch p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t afull[4], aempty[4], bfull[kTStages], bempty[kTStages], ifull[2], accfull[2],
@@ -567,14 +601,14 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
     *vabort = 1;
     atomicExch(p.err, 1);
   };
-  const int64_t G = gridDim.x;
 
   if (warp == 0) {
     // ---------------- cell images
     if (lane == 0) {
       int64_t cl = 0;
       int issued = 0;
-      for (int64_t g = blockIdx.x; g < p.total_cells && !*vabort; g += G, ++cl) {
+      for (StepCell it{blockIdx.x, 0}; it.st < p.nsteps && !*vabort; it.next(p), ++cl) {
+        const int64_t g = it.g;
         const StepPartDev& P = p.part[part_of(p, g)];
         const uint8_t* src = P.img + (g - P.cell_off) * (int64_t)kABytes;
         for (issued = 0; issued < 4; ++issued) {
@@ -601,7 +635,8 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
     const uint64_t b0 = tc::sw128_desc(tc::smem_u32(sA));
     uint32_t j = 0, cl = 0;
     bool stop = false;
-    for (int64_t g = blockIdx.x; g < p.total_cells && !stop; g += G, ++cl) {
+    for (StepCell it{blockIdx.x, 0}; it.st < p.nsteps && !stop; it.next(p), ++cl) {
+      const int64_t g = it.g;
       const StepPartDev& P = p.part[part_of(p, g)];
       const int ntiles = P.ntiles;
       for (int t = 0; t < ntiles && !stop; ++t, ++j) {
@@ -644,12 +679,17 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
     uint32_t j = 0, cl = 0, ph0 = 0;
     int s0 = 0;
     bool stop = false;
-    for (int64_t g = blockIdx.x; g < p.total_cells && !stop; g += G, ++cl) {
+    for (StepCell it{blockIdx.x, 0}; it.st < p.nsteps && !stop; it.next(p), ++cl) {
+      const int64_t g = it.g;
       const StepPartDev& P = p.part[part_of(p, g)];
       const CellTab& tab = tabs[cl % kTab];
       const int n = P.n, ntiles = P.ntiles;
       float al = P.alpha, be = P.beta, om = P.omega;
-      if (P.coef) {
+      if (p.nsteps > 1) {
+        al = p.coefs[3 * it.st];
+        be = p.coefs[3 * it.st + 1];
+        om = p.coefs[3 * it.st + 2];
+      } else if (P.coef) {
         al = (float)__ldg(P.coef);
         be = (float)__ldg(P.coef + 1);
         om = (float)__ldg(P.coef + 2);
@@ -711,12 +751,14 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
     const int q = warp & 3, k0 = 64 * ((warp - 10) >> 2);
     uint32_t j = 0, cl = 0;
     bool stop = false;
-    for (int64_t g = blockIdx.x; g < p.total_cells && !stop; g += G, ++cl) {
+    for (StepCell it{blockIdx.x, 0}; it.st < p.nsteps && !stop; it.next(p), ++cl) {
+      const int64_t g = it.g;
       const StepPartDev& P = p.part[part_of(p, g)];
       const CellTab& tab = tabs[cl % kTab];
       const int nc = P.nc, n = P.n, ntiles = P.ntiles;
-      float al = P.coef ? (float)__ldg(P.coef) : P.alpha;
+      float al = p.nsteps > 1 ? p.coefs[3 * it.st] : P.coef ? (float)__ldg(P.coef) : P.alpha;
       al *= P.sign;
+      float* Ub = (it.st & 1) ? P.U2 : P.U;
       for (int t = 0; t < ntiles; ++t, ++j) {
         const uint32_t xb = (uint32_t)(j & 1);
         const int col = 128 * t + q * 32 + lane;
@@ -731,7 +773,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
         tc::tc_fence_after();
         if (128 * t + q * 32 < n) {
           const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + xb * 128u + (uint32_t)k0;
-          float* U = P.U + col;
+          float* U = Ub + col;
 #pragma unroll
           for (int kb = 0; kb < 64; kb += 16) {
             float v[16];
@@ -747,8 +789,13 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
         tc::tc_fence_before();
         tc::mbar_arrive(&accempty[xb]);
       }
+      const bool meet = it.last(p) && it.st + 1 < p.nsteps;
+      if (meet) __threadfence();  // this step's adds, before the other CTAs read the rows
       __syncwarp();
-      if (lane == 0 && !stop) tc::mbar_arrive(&tfree[cl % kTab]);
+      if (lane == 0 && !stop) {
+        tc::mbar_arrive(&tfree[cl % kTab]);
+        if (meet) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.sync) : "memory");
+      }
     }
   } else {
     // ---------------- gather: 16 lanes copy one 256-byte row segment
@@ -757,13 +804,17 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
     uint32_t cl = 0, ph = 1;  // ph: phase parity that frees stage s
     int s = 0;
     bool stop = false;
-    for (int64_t g = blockIdx.x; g < p.total_cells; g += G, ++cl) {
+    for (StepCell it{blockIdx.x, 0}; it.st < p.nsteps; it.next(p), ++cl) {
+      const int64_t g = it.g;
       const StepPartDev& P = p.part[part_of(p, g)];
       const int64_t cell = g - P.cell_off;
       CellTab& tab = tabs[cl % kTab];
       const int nc = P.nc, n = P.n;
       // the cell's tables, once its predecessor in the same place is done with
       bool ok = !stop && !*vabort && tc::mbar_wait(&tfree[cl % kTab], (uint32_t)((cl / kTab) & 1) ^ 1u);
+      // a step reads what the one before has added: once all its adds (eight epilogue warps per CTA) are in
+      if (ok && it.st > 0 && it.first() && gt == 0) ok = wait_steps(p.sync, it.st * 8 * (int)gridDim.x, p.err);
+      const float* Vb = (it.st & 1) ? P.V2 : P.V;
       int o = -1;
       if (ok) {
         const int d = __ldg(P.dofs + cell * nc + min(gt, nc - 1));  // padding rows repeat
@@ -797,7 +848,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
         }
         const int col = hs * 64 + 4 * ch;
         const bool in = col < n;
-        const float* Vc = P.V + (in ? col : 0);
+        const float* Vc = Vb + (in ? col : 0);
         const float* Wc = P.W + (in ? col : 0);
         uint8_t* dst = sB + (size_t)s * kTStage + r0 * 256 + ch * 16;
 #pragma unroll
@@ -805,7 +856,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
           cp_async16(dst + i * 2048, Vc + (int64_t)rows[i] * n, in && r0 + 8 * i < nc);
         for (int r = r0; r < (int)nown; r += 8)
           cp_async16(dst + kTV + (r - r0) * 256, Wc + (int64_t)tab.orow[r] * n, in);
-        if (gt < 16) cp_async16(sL + s * 64 + 4 * gt, P.lam + (in ? col : 0), in);
+        if (gt < 16) cp_async16(sL + s * 64 + 4 * gt, P.lam + (int64_t)it.st * n + (in ? col : 0), in);
         cp_async_arrive_noinc(&bfull[s]);
         if (gt == 0) tc::mbar_arrive(&bfull[s]);
         if (++s == kTStages) {
@@ -896,14 +947,22 @@ int fe_step_parts(FeOp& op, const float* V, const float* W, float* U, const floa
   return 4;
 }
 
-void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, int num_sms) {
+void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, int num_sms, const FeStepLoop* loop) {
   RC_CHECK(nparts >= 1 && nparts <= kMaxParts, RCHFSI_ERR_INVALID_ARG, "fused FE step: 1..64 parts per launch");
   RC_CHECK(BN == 32 || BN == 64 || BN == 96 || BN == 128, RCHFSI_ERR_INVALID_ARG,
            "fused FE step: column tile of 32, 64, 96 or 128");
   const Plan pl = BN == 128 ? Plan{1, kTStages, kTSmem} : make_plan(BN);
   RC_CHECK(pl.nA > 0, RCHFSI_ERR_INVALID_ARG, "fused FE step: no shared-memory plan for this tile");
+  const int nsteps = loop ? loop->steps : 1;
+  RC_CHECK(nsteps == 1 || (BN == 128 && nsteps >= 1 && nsteps <= kTableSteps && loop->sync), RCHFSI_ERR_INVALID_ARG,
+           "fused FE loop: tiles of 128 columns, at most kTableSteps steps and a counter");
   StepBatch b{};
   b.nparts = nparts;
+  b.nsteps = nsteps;
+  if (nsteps > 1) {
+    b.sync = loop->sync;
+    std::copy(loop->coefs, loop->coefs + 3 * nsteps, b.coefs);
+  }
   b.nA = pl.nA;
   b.nslots = pl.nslots;
   int64_t off = 0;
@@ -924,6 +983,10 @@ void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, 
     P.V = t.V;
     P.W = t.W;
     P.U = t.U;
+    if (nsteps > 1) {  // the two blocks change places
+      P.V2 = loop->U + (t.V - loop->V);
+      P.U2 = loop->V + (t.U - loop->U);
+    }
     P.lam = t.lam;
     P.coef = t.coef;
     P.n_cells = op.n_cells;
@@ -948,13 +1011,19 @@ void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, 
   while (cols < (uint32_t)(2 * BN)) cols <<= 1;
   b.tmem_cols = cols;
   const unsigned grid = (unsigned)std::min<int64_t>(b.total_cells, (int64_t)num_sms);
-  prof::Scope ps(s, RCHFSI_KERNEL_FE_CELL, flops, bytes);
+  prof::Scope ps(s, RCHFSI_KERNEL_FE_CELL, flops * nsteps, bytes * nsteps);
   switch (BN) {
     case 32: launch<32>(s, b, pl, grid); break;
     case 64: launch<64>(s, b, pl, grid); break;
     case 128:
       set_smem_limit(reinterpret_cast<const void*>(fe_step_t_kernel), kSmemMax - 512);
-      fe_step_t_kernel<<<grid, kTThreads, kTSmem, s>>>(b);
+      if (nsteps > 1) {
+        void* args[] = {(void*)&b};
+        RC_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fe_step_t_kernel), dim3(grid), dim3(kTThreads),
+                                            args, kTSmem, s));
+      } else {
+        fe_step_t_kernel<<<grid, kTThreads, kTSmem, s>>>(b);
+      }
       RC_LAUNCH();
       break;
     default: launch<96>(s, b, pl, grid); break;

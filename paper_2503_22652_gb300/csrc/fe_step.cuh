@@ -35,8 +35,20 @@ int fe_step_parts(FeOp& op, const float* V, const float* W, float* U, const floa
 // Pack the operator's scaled cell images (A_c D_c^-1, TF32) and owner masks ahead of a capture.
 void fe_step_prepare(cudaStream_t s, FeOp& op);
 
-// All parts (at most 64) in one persistent launch; BN = column tile (32, 64 or 96).
-void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, int num_sms);
+// Several degree steps of one filter in one launch (BN = 128): coefs holds alpha, beta, omega per step; the parts are
+// those of the first step, their V and U inside the blocks V and U, which change places after every step; lam
+// advances by the part's n per step; sync: a zeroed device counter.
+struct FeStepLoop {
+  int steps;
+  const float* coefs;
+  float* V;
+  float* U;
+  int* sync;
+};
+
+// All parts (at most 64) in one persistent launch; BN = column tile (32, 64, 96 or 128).
+void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, int num_sms,
+                   const FeStepLoop* loop = nullptr);
 
 // Column tile for this operator and width, chosen by timing the candidates once per shape on the
 // problem's own data (into a scratch output); cached.

@@ -83,6 +83,29 @@ def test_output_may_overlap_inputs_fe(N, prec, tol):
             assert np.linalg.norm(y - exact) <= tol * np.linalg.norm(exact - base)
 
 
+# one step, an even and an odd number of them; widths around the half tiles and tiles of the step; fewer cells than
+# SMs and more; tolerance of the reduced-precision FE filter parity test
+@pytest.mark.parametrize("n,N,p", [(2, 4, 2), (2, 64, 3), (3, 68, 4), (3, 128, 5), (2, 132, 3), (6, 48, 4)])
+def test_fe_degree_loop(n, N, p):
+    from oracle import fe as ofe, filters
+    q = wl.fe_problem(n)
+    A = ofe.assemble(q["cell_dofs"], q["A_cells"], q["m"])
+    B = ofe.assemble(q["cell_dofs"], q["B_cell"], q["m"])
+    d = q["Dinv"]
+    rng = np.random.default_rng(N)
+    X = rng.standard_normal((q["m"], N))
+    L = np.sort(rng.uniform(-20.0, 30.0, N))
+    W = A @ X - (B @ X) * L[None, :]
+    args = (-25.0, 40.0, 2500.0, p)
+    exact = filters.rchfsi_filter(lambda R: A @ (d[:, None] * R), lambda R: d[:, None] * R, X, L, W, *args)
+    base = X * lambda_p(L, *args)[None, :]
+    s = Solver(q["m"], nev=max(1, N // 2), block=N, precision="tf32")
+    s.set_fe(q["cell_dofs"], q["A_cells"], q["B_cell"], q["Dinv"])
+    for _ in range(2):
+        got = s.filter(X, L, W, *args)
+        assert np.linalg.norm(got - exact) <= 5e-3 * np.linalg.norm(exact - base)
+
+
 @pytest.mark.parametrize("N", [1, 31, 65, 130])
 def test_fe_residual_rows(N):
     from oracle import fe as ofe
