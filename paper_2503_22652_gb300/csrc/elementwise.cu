@@ -36,17 +36,20 @@ __global__ void transpose_kernel(int64_t rows, int64_t cols, const double* __res
 // A conversion from or to a double holds the FP64 pipe like a multiply (about two per clock per SM), which
 // bounded the passes that open and close the FE filter: 262144 x 600, 1105 and 1187 us against 0.37 and
 // 0.47 ms of HBM traffic.
+// (the conversions proper stay behind a call: inlined, they are executed for every value and selected away)
+__device__ __noinline__ float f32_cvt(double x) { return (float)x; }
+__device__ __noinline__ double f64_cvt(float x) { return (double)x; }
 __device__ __forceinline__ float f32_rn(double x) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const unsigned long long r = u + 0x0fffffffULL + ((u >> 29) & 1ULL);  // round to nearest even at bit 29
   const uint32_t e = (uint32_t)(r >> 52) & 0x7ffu;
-  if (e - 897u > 253u) return (float)x;  // zero, subnormal, overflow, non-finite
+  if (e - 897u > 253u) return f32_cvt(x);  // zero, subnormal, overflow, non-finite
   const uint32_t v = (uint32_t)((r & 0x7fffffffffffffffULL) >> 29) - (896u << 23);
   return __uint_as_float(v | ((uint32_t)(u >> 32) & 0x80000000u));
 }
 __device__ __forceinline__ double f64_of(float x) {
   const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
-  if (e - 1u > 253u) return (double)x;
+  if (e - 1u > 253u) return f64_cvt(x);
   return __longlong_as_double((long long)(((unsigned long long)(b & 0x80000000u) << 32) |
                                           (((unsigned long long)(b & 0x7fffffffu) << 29) + (896ULL << 52))));
 }
