@@ -387,15 +387,6 @@ __device__ __forceinline__ void red_add_u64(unsigned long long* p, unsigned long
   asm volatile("red.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-__device__ __forceinline__ void two_sum(float& hi, float& lo, float b) {
-  const float s = hi + b;
-  const float bb = s - hi;
-  const float e = (hi - (s - bb)) + (b - bb);
-  hi = s;
-  lo += e;
-}
-
-
 // Level buffers in TMEM: 8 blocks of 64 columns, 7 holding the levels of the current item and one
 // spare.  perm packs, per level L = 0..6, its block (4 bits each; bits 28-31: the spare).  The next
 // item puts level 0 in the spare and levels 6, 5, .., 1 in the blocks of levels 0, 1, .., 5, the
@@ -652,15 +643,15 @@ __global__ void __launch_bounds__(kThreads, 1) fe_oz_kernel(const __grid_constan
       int g = -1, qs = 0;
       if (i < p.nc) {
         g = __ldg(p.dofs + cell * p.nc + i);
-        // the contribution (hi + lo) 2^(ea + ex - 16) in units of the accumulator's last place
+        // the contribution sum_L D_L 2^-8L 2^(ea + ex - 16) in units of the accumulator's last place
         // 2^(rowexp + ex + H - 62): the column exponent ex cancels
         const int ea = __ldg(p.aexp + cell * p.e_stride + i);
         qs = ea == -100000 ? 0 : max(46 - p.H + ea - __ldg(p.rowexp + g), -200);
       }
-      float hi[16], lo[16];
+      // sum_L D_L 2^(48 - 8 L) = top 2^32 + low, exact: a conversion and one wide multiply-add per level and column
+      long long top[16], low[16];
       bool ok = true;
-      float scale = 1.f;
-#pragma unroll 1
+#pragma unroll
       for (int L = 0; L < S; ++L) {
         const bool w = !*vabort && tc::mbar_wait(&lv[L], par);
         ok = __all_sync(0xffffffffu, w);
@@ -671,17 +662,12 @@ __global__ void __launch_bounds__(kThreads, 1) fe_oz_kernel(const __grid_constan
         tc::tmem_ld16(lane_base + blk * (uint32_t)kBN, v);
         tc::tc_fence_before();
         tc::mbar_arrive(&bfree[blk]);
-        if (L == 0) {
 #pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            hi[u] = v[u];
-            lo[u] = 0.f;
-          }
-        } else {
-#pragma unroll
-          for (int u = 0; u < 16; ++u) two_sum(hi[u], lo[u], v[u] * scale);
+        for (int u = 0; u < 16; ++u) {
+          const int d = __float2int_rn(v[u]);
+          if (L < 3) top[u] = (L == 0 ? 0 : top[u]) + (long long)d * (1 << (16 - 8 * (L < 3 ? L : 2)));
+          else low[u] = (L == 3 ? 0 : low[u]) + (long long)d * (1 << (24 - 8 * (L < 3 ? 3 : L - 3)));
         }
-        scale *= 0.00390625f;  // 2^-8 per level
       }
       if (!ok) {
         fail();
@@ -692,11 +678,15 @@ __global__ void __launch_bounds__(kThreads, 1) fe_oz_kernel(const __grid_constan
         // integer adds: exact, so the sum does not depend on the order of the cells
         unsigned long long* out = reinterpret_cast<unsigned long long*>(p.Y + (int64_t)g * p.n);
         const int c0 = tile * kBN + hq * 16;
+        // (top 2^32 + low) 2^(qs - 48), each part rounded to the accumulator's last place; qs <= 38 and top is below
+        // 2^40, so the left shift stays below 2^62
+        const int lt = max(qs - 16, 0), st = min(max(16 - qs, 0), 63), sl = min(48 - qs, 63);
+        const long long rt = (1LL << st) >> 1, rl = (1LL << sl) >> 1;
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
           const int col = c0 + u;
           if (col < p.n) {
-            const long long v = f32_to_fixed(hi[u], qs) + f32_to_fixed(lo[u], qs);
+            const long long v = (((top[u] << lt) + rt) >> st) + ((low[u] + rl) >> sl);
             red_add_u64(out + col, (unsigned long long)(p.neg ? -v : v));
           }
         }

@@ -51,35 +51,6 @@ __device__ __forceinline__ uint32_t bf16_pair(float a, float b) {
   return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
 }
 
-// x (finite FP32, |x| in the normal range or 0) times 2^p as an FP64 value, by integer arithmetic.
-__device__ __forceinline__ double f32_scaled(float x, int p) {
-  const uint32_t b = __float_as_uint(x);
-  const uint32_t e8 = (b >> 23) & 0xff;
-  if (e8 == 0) return 0.0;
-  const long long e = (long long)e8 - 127 + 1023 + p;
-  if (e <= 0 || e >= 2047) return ldexp((double)x, p);  // out of the normal range: rare, exact path
-  const unsigned long long bits = ((unsigned long long)(b >> 31) << 63) | ((unsigned long long)e << 52) |
-                                  ((unsigned long long)(b & 0x7fffff) << 29);
-  return __longlong_as_double((long long)bits);
-}
-
-// round(x 2^q) as a signed 64-bit integer (nearest, ties away from zero), by integer arithmetic,
-// for finite x with |x| 2^q < 2^62 and q <= 38 + 150 - (biased exponent of x).  Zero and FP32
-// subnormals give 0.  Branch-free: the 24-bit significand is placed at bit 39 and shifted right
-// by 39 - (its scale), rounding on the bits shifted out.
-__device__ __forceinline__ long long f32_to_fixed(float x, int q) {
-  const uint32_t b = __float_as_uint(x);
-  const uint32_t e8 = (b >> 23) & 0xffu;
-  const int r0 = 189 - (int)e8 - q;  // 39 - (e8 - 150 + q): the right shift
-  // |x| 2^q < 1/2 (r0 > 63) rounds to 0, as does a zero or subnormal x
-  const uint32_t mant = (e8 != 0u && r0 <= 63) ? ((b & 0x7fffffu) | 0x800000u) : 0u;
-  const int r = min(max(r0, 1), 63);
-  unsigned long long u = (unsigned long long)mant << 39;
-  u = (u + (1ull << (r - 1))) >> r;
-  const long long v = (long long)u;
-  return (b >> 31) ? -v : v;
-}
-
 // v 2^e as an FP64 value, rounded to nearest even: one conversion on the FP64 pipe, the scaling by
 // exponent arithmetic.
 __device__ __forceinline__ double fixed_to_f64(long long v, int e) {

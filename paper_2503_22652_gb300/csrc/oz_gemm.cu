@@ -10,9 +10,8 @@
 // while this one is multiplied.  TMEM holds 8 level blocks of 64 columns,
 // 7 for the group and one spare, rotated so that the next group's first writes go to blocks in the
 // order they are freed; warps 2-17 (four per TMEM lane quarter, 16 columns each) fold level L of a
-// group as soon as the group's pass L is done: tcgen05.ld, exact scaling by 2^-8L and TwoSum into
-// per-output float-float accumulators.  The final value (hi + lo) 2^(e_i + f_j - 16), formed by
-// exponent arithmetic, is stored in FP64 (or, with split-K, written as a partial and summed by a
+// group as soon as the group's pass L is done: tcgen05.ld and one 64-bit multiply-add into exact integer
+// accumulators.  The final value, two conversions scaled by exponent arithmetic and one FP64 add, is stored (or, with split-K, written as a partial and summed by a
 // second kernel) while the next item's MMAs run.  The host splits K only as far as the items fill the
 // CTAs.
 // Bound: issue of the 128 x 64 x 16 MMAs by one warp beside 16 busy epilogue warps.  A pass runs its A tile (16 K
@@ -212,14 +211,6 @@ struct OzArgs {
   int upper;       // only tiles that reach the upper triangle (i <= j) are computed
   int* err;
 };
-
-__device__ __forceinline__ void two_sum(float& hi, float& lo, float b) {
-  const float s = hi + b;
-  const float bb = s - hi;
-  const float e = (hi - (s - bb)) + (b - bb);
-  hi = s;
-  lo += e;
-}
 
 // Level blocks in TMEM: 8 blocks of 64 columns, 7 holding the levels of the current accumulation
 // group and one spare.  perm packs, per level L = 0..6, its block (4 bits each; bits 28-31: the
@@ -470,9 +461,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::mbar_wait(&mdone, 0);
   } else {
     // ---------------- epilogue: 16 warps, lane quarter q, 16 columns each.  Level L of a group is
-    // folded (exact scaling by 2^-8L, TwoSum into per-output float-float accumulators) as soon as
+    // folded into the integer accumulators as soon as
     // the group's pass L is done, and its block released; the final value of an item is stored while
-    // the next item's MMAs run.
+    // the next item's MMAs run.  (Every instruction here delays the issuing warp: with a scaling and a TwoSum in
+    // FP32 per level, seven instructions per value, an MMA took 68 clocks.)
     const int q = warp & 3, hq = (warp - 2) >> 2;
     const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(hq * 16);
     uint32_t perm = kPerm0;
@@ -481,14 +473,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int64_t it = blockIdx.x; it < p.items && ok; it += G) {
       const OzItem wi = oz_item(p, it);
       const int ngroups = (chunks_of(wi.split) + GROUP - 1) / GROUP;
-      float hi[16], lo[16];
+      // sum_L D_L 2^(48 - 8 L) = top 2^32 + low over all groups, exact in 64-bit integers (D_L below 2^24, up to
+      // 2^11 groups): a conversion and one wide multiply-add per level and column
+      long long top[16], low[16];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) hi[u] = lo[u] = 0.f;
+      for (int u = 0; u < 16; ++u) top[u] = low[u] = 0;
       for (int g = 0; g < ngroups && ok; ++g, ++gidx) {
         uint64_t* lv = lev[gidx & 1];
         const uint32_t par = (uint32_t)((gidx >> 1) & 1);
-        float scale = 1.f;
-#pragma unroll 1
+#pragma unroll
         for (int L = 0; L < S; ++L) {
           const bool w = !*vabort && tc::mbar_wait(&lv[L], par);
           ok = __all_sync(0xffffffffu, w);
@@ -500,8 +493,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc::tc_fence_before();
           tc::mbar_arrive(&bfree[blk]);
 #pragma unroll
-          for (int u = 0; u < 16; ++u) two_sum(hi[u], lo[u], v[u] * scale);
-          scale *= 0.00390625f;  // 2^-8
+          for (int u = 0; u < 16; ++u) {
+            const int d = __float2int_rn(v[u]);
+            if (L < 3) top[u] += (long long)d * (1 << (16 - 8 * (L < 3 ? L : 2)));
+            else low[u] += (long long)d * (1 << (24 - 8 * (L < 3 ? 3 : L - 3)));
+          }
         }
         perm = perm_next(perm);
       }
@@ -516,9 +512,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int u = 0; u < 16; ++u) {
           const int64_t jcol = (int64_t)wi.tn * BN + hq * 16 + u;
           if (jcol < p.N) {
-            // (hi + lo) 2^(e_i + f_j - 16): exact conversions by exponent arithmetic and one FP64 add
-            const int pw = ei + p.eb[jcol] - 16;
-            const double v = f32_scaled(hi[u], pw) + f32_scaled(lo[u], pw);
+            // (top 2^32 + low) 2^(e_i + f_j - 64): `top` is exact in FP64, `low` 2^-32 of its scale
+            const int pw = ei + p.eb[jcol] - 64;
+            const double v = fixed_to_f64(top[u], pw + 32) + fixed_to_f64(low[u], pw);
             if (p.partial) p.C[((int64_t)wi.split * p.N + jcol) * p.M + i] = v;
             else p.C[jcol * p.ldc + i] = v;
           }
@@ -699,6 +695,7 @@ void oz_gemm(cudaStream_t s, int num_sms, const OzOperand& A, const OzOperand& B
   // persistent CTAs over (tile, K split) items: split K only as far as the items then fill the CTAs
   double eff = 0.0;
   int nsplit = choose_split(kept, nchunks, num_sms, &eff);
+  nsplit = std::max(nsplit, (nchunks + (1 << 14) - 1) >> 14);  // the epilogue's integers hold 2^22 K terms
   const int per = (nchunks + nsplit - 1) / nsplit;
   nsplit = (nchunks + per - 1) / per;
   const CUtensorMap ma = slice_map(A, BM);
