@@ -1078,13 +1078,14 @@ int rchfsi_rayleigh_ritz(rchfsi_ctx* h, const double* Y, double* X, double* eval
     need_op(h);
     rchfsi_ctx& c = *h;
     load_any(c, Y, c.w.Y.p);
-    const int rc = rayleigh_ritz(c, c.w.Y.p, c.w.X.p, false, c.w.evals.p);
+    bool in_rows = false;
+    const int rc = rayleigh_ritz(c, c.w.Y.p, c.w.X.p, false, c.w.evals.p, is_device_pointer(X) ? X : nullptr, &in_rows);
     if (rc != RCHFSI_OK) return rc;
     if (c.cplx && !c.rr_paired) {
       std::vector<double> ev = host_vec(c, c.w.evals.p, c.p.block);
       pair_complex(c, ev);
     }
-    store_any(c, c.w.X.p, X);
+    if (!in_rows) store_any(c, c.w.X.p, X);
     from_device(c, c.w.evals.p, evals, c.cplx ? c.Nc : c.p.block);
     RC_CUDA(cudaStreamSynchronize(c.s));
     return RCHFSI_OK;

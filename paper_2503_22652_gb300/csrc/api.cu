@@ -919,7 +919,7 @@ void filter_fe_batch(cudaStream_t s, int num_sms, std::vector<FeFilterJob>& jobs
            RCHFSI_ERR_CUDA, "syevd failed");
 }
 
-int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* evals) {
+int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* evals, double* Xrows, bool* in_rows) {
   const int64_t m = c.p.m;
   const int N = c.p.block;
   Work& w = c.w;
@@ -1145,7 +1145,11 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* ev
       // E^T as ncol logical rows (row j = column j of E, contiguous); blocks as m logical rows (dofs)
       oz_slice(c.s, ncol, N, Erot, N, 1, w.ozE);
       oz_slice(c.s, m, N, Y, 1, m, w.ozL);
-      oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, X, m, w.ozws, eflag);
+      const bool rows = Xrows && !want && !c.cplx;
+      if (in_rows) *in_rows = rows;
+      // (a call that returns X row-major: the same product with the operands exchanged, X^T column-major)
+      if (rows) oz_gemm(c.s, c.num_sms, w.ozE, w.ozL, Xrows, N, w.ozws, eflag);
+      else oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, X, m, w.ozws, eflag);
       if (want && !direct) {
         oz_slice(c.s, m, N, AY, 1, m, w.ozL);
         oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, AX, m, w.ozws, eflag);

@@ -201,6 +201,7 @@ struct OzArgs {
   int MP, NP;      // rows per slice in the A and B slice tensors
   int chunks_per_split, nchunks;
   int n_tiles;     // column tiles
+  int m_fast;      // > 0: that many row tiles, walked fastest (fewer than column tiles)
   int kept;        // output tiles computed (all, or those reaching the upper triangle)
   int64_t items;   // kept x splits
   const int* ea;
@@ -225,8 +226,8 @@ __device__ __forceinline__ uint32_t perm_next(uint32_t perm) {
 }
 constexpr uint32_t kPerm0 = 0x76543210u;
 
-// Work item -> (row tile, column tile, K split).  Items run split-major, column tile fastest, so
-// CTAs working at the same time share the row tile's A slices and the split's K range in L2.  With
+// Work item -> (row tile, column tile, K split).  Items run split-major, the side with fewer tiles fastest, so
+// CTAs working at the same time share the slices of the longer operand and the split's K range in L2.  With
 // `upper`, row tile tm keeps only the column tiles tn >= tm BM / BN (those reaching i <= j).
 struct OzItem {
   int tm, tn, split;
@@ -236,8 +237,13 @@ __device__ __forceinline__ OzItem oz_item(const OzArgs& p, int64_t it) {
   r.split = (int)(it / p.kept);
   int t = (int)(it - (int64_t)r.split * p.kept);
   if (!p.upper) {
-    r.tm = t / p.n_tiles;
-    r.tn = t - r.tm * p.n_tiles;
+    if (p.m_fast > 0) {
+      r.tn = t / p.m_fast;
+      r.tm = t - r.tn * p.m_fast;
+    } else {
+      r.tm = t / p.n_tiles;
+      r.tn = t - r.tm * p.n_tiles;
+    }
     return r;
   }
   int tm = 0;
@@ -710,6 +716,7 @@ void oz_gemm(cudaStream_t s, int num_sms, const OzOperand& A, const OzOperand& B
   p.chunks_per_split = per;
   p.nchunks = nchunks;
   p.n_tiles = n_tiles;
+  p.m_fast = m_tiles < n_tiles ? m_tiles : 0;
   p.kept = kept;
   p.items = (int64_t)kept * nsplit;
   p.ea = A.ex.p;

@@ -104,7 +104,9 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
 
 // Rayleigh-Ritz on column-major Y (scaled in place): X and evals (device) are outputs, and with `products`
 // also A X and B X in c.w.AX and c.w.BX (a solve's residuals; a single call has no use for them).
-int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* evals);
+// Xrows: an m x N row-major device array that may take X instead of the column-major one (*in_rows tells).
+int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* evals, double* Xrows = nullptr,
+                  bool* in_rows = nullptr);
 
 // Lanczos bounds (host results).
 void lanczos(rchfsi_ctx& c, const double* v0_dev, int k, double* lmax, double* normA);
