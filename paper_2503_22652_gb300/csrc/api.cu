@@ -933,6 +933,7 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* ev
   double* AY = w.AY.p;
   double* BY = w.BY.p;
   const bool emu = c.p.rr_mode == RCHFSI_RR_FP64_EMULATED;
+  const bool unit_B = emu && !c.cplx && !has_B(c);  // B = I: no products with B are formed
   int* eflag = w.info.p + 2;
   // A complex problem's block is Y = [Y1, J Y1] (J = multiplication by i) and A, B commute with J:
   // the operator products are formed on the first Nc columns and completed by J, which halves the
@@ -955,7 +956,7 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* ev
           if (d.ozB.R != m) oz_slice(c.s, m, m, d.B.p, m, 1, d.ozB);
           oz_gemm(c.s, c.num_sms, d.ozB, w.ozL, BY, m, w.ozws, eflag);
           jcomplete(BY);
-        } else {
+        } else if (!unit_B) {
           RC_CUDA(cudaMemcpyAsync(BY, Y, sizeof(double) * m * N, cudaMemcpyDeviceToDevice, c.s));
         }
       } else {
@@ -968,8 +969,9 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* ev
       // (real problems: both are symmetric, only the tiles reaching the upper triangle are formed)
       oz_slice(c.s, Na, m, AY, m, 1, w.ozR);
       oz_gemm(c.s, c.num_sms, w.ozL, w.ozR, w.GA.p, N, w.ozws, eflag, Na == N);
-      oz_slice(c.s, Na, m, BY, m, 1, w.ozR);
-      oz_gemm(c.s, c.num_sms, w.ozL, w.ozR, w.GB.p, N, w.ozws, eflag, Na == N);
+      // (B = I: B Y is Y, whose slices are there)
+      if (!unit_B) oz_slice(c.s, Na, m, BY, m, 1, w.ozR);
+      oz_gemm(c.s, c.num_sms, w.ozL, unit_B ? w.ozL : w.ozR, w.GB.p, N, w.ozws, eflag, Na == N);
     } else {
       apply_AB_f64(c, Y, AY, BY, Na);
       jcomplete(AY);
@@ -1153,8 +1155,12 @@ int rayleigh_ritz(rchfsi_ctx& c, double* Y, double* X, bool products, double* ev
       if (want && !direct) {
         oz_slice(c.s, m, N, AY, 1, m, w.ozL);
         oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, AX, m, w.ozws, eflag);
-        oz_slice(c.s, m, N, BY, 1, m, w.ozL);
-        oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, BX, m, w.ozws, eflag);
+        if (unit_B) {
+          RC_CUDA(cudaMemcpyAsync(BX, X, sizeof(double) * m * N, cudaMemcpyDeviceToDevice, c.s));
+        } else {
+          oz_slice(c.s, m, N, BY, 1, m, w.ozL);
+          oz_gemm(c.s, c.num_sms, w.ozL, w.ozE, BX, m, w.ozws, eflag);
+        }
       }
     } else {
       gemm_f64(c.s, m, ncol, N, Y, m, false, Erot, N, true, epi_store(X, m));

@@ -535,14 +535,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+// Sum of the split-K partials; `mirror`: of the upper triangle, written to both.
 __global__ void oz_sum_kernel(int64_t M, int64_t N, int nsplit, const double* __restrict__ part, double* C,
-                              int64_t ldc) {
+                              int64_t ldc, int mirror) {
   const int64_t total = M * N;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t j = e / M, i = e - j * M;
+    if (mirror && i > j) continue;
     double acc = 0.0;
     for (int s = 0; s < nsplit; ++s) acc += part[(int64_t)s * total + e];
     C[j * ldc + i] = acc;
+    if (mirror && i < j) C[i * ldc + j] = acc;
   }
 }
 
@@ -744,10 +747,10 @@ void oz_gemm(cudaStream_t s, int num_sms, const OzOperand& A, const OzOperand& B
   if (nsplit > 1) {
     const int64_t total = M * N;
     const unsigned blocks = (unsigned)std::min<int64_t>((total + 255) / 256, (int64_t)num_sms * 8);
-    oz_sum_kernel<<<blocks, 256, 0, s>>>(M, N, nsplit, p.C, C, ldc);
+    oz_sum_kernel<<<blocks, 256, 0, s>>>(M, N, nsplit, p.C, C, ldc, symmetric ? 1 : 0);
     RC_LAUNCH();
   }
-  if (symmetric) {
+  if (symmetric && nsplit == 1) {
     const unsigned blocks = (unsigned)std::min<int64_t>((M * N + 255) / 256, (int64_t)num_sms * 4);
     mirror_upper_kernel<<<blocks, 256, 0, s>>>((int)M, C, ldc);
     RC_LAUNCH();

@@ -2059,8 +2059,7 @@ bool sym_eig_f64(cudaStream_t s, int n, double* M, double* V, double* evals, Dev
     RC_CUDA(cudaStreamSynchronize(s));
     return true;
   }
-  RC_CUDA(cudaMemsetAsync(e, 0, sizeof(double) * n, s));
-  RC_CUDA(cudaMemsetAsync(tau, 0, sizeof(double) * n, s));
+  RC_CUDA(cudaMemsetAsync(e, 0, sizeof(double) * 2 * n, s));  // and tau behind it
   // 1. Q^T M Q = T
   if (!launch_tridiag_xch(s, n, num_sms, M, H, d, e, tau, pkts, d_flag) &&
       !launch_resident(s, tridiag_smem_kernel<true>, tridiag_smem_kernel<false>, n, num_sms, n, (const double*)M, H,
