@@ -511,10 +511,24 @@ struct CellTab {
 constexpr size_t kTSmem = kABytes + kTStages * ((size_t)kTStage + 64 * 4) + kTab * sizeof(CellTab) + 1024;
 
 // (predicated inside: a branch around each add made an add wait for the address of the one before, 130 clocks)
-__device__ __forceinline__ void red_add_f32(float* p, float a, bool on) {
-  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p red.global.add.f32 [%0], %1;\n}" ::"l"(p), "f"(a),
-               "r"((uint32_t)on)
+__device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, float d, bool on) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %5, 0;\n@p red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n}" ::"l"(p),
+               "f"(a), "f"(b), "f"(c), "f"(d), "r"((uint32_t)on)
                : "memory");
+}
+
+// v[i] of lane 4 q + j (i, j < 4) goes to v[j] of lane 4 q + i.
+__device__ __forceinline__ void quad_transpose(float* v, int lane) {
+  const bool b0 = lane & 1, b1 = lane & 2;
+  const float s0 = __shfl_xor_sync(0xffffffffu, b0 ? v[0] : v[1], 1);
+  const float s1 = __shfl_xor_sync(0xffffffffu, b0 ? v[2] : v[3], 1);
+  const float x0 = b0 ? s0 : v[0], x1 = b0 ? v[1] : s0, x2 = b0 ? s1 : v[2], x3 = b0 ? v[3] : s1;
+  const float t0 = __shfl_xor_sync(0xffffffffu, b1 ? x0 : x2, 2);
+  const float t1 = __shfl_xor_sync(0xffffffffu, b1 ? x1 : x3, 2);
+  v[0] = b1 ? t0 : x0;
+  v[1] = b1 ? t1 : x1;
+  v[2] = b1 ? x2 : t0;
+  v[3] = b1 ? x3 : t1;
 }
 
 // D[tmem] += A[tmem] * B[smem]^T, TF32.
@@ -761,7 +775,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
       float* Ub = (it.st & 1) ? P.U2 : P.U;
       for (int t = 0; t < ntiles; ++t, ++j) {
         const uint32_t xb = (uint32_t)(j & 1);
-        const int col = 128 * t + q * 32 + lane;
+        const int col4 = 128 * t + q * 32 + (lane & ~3);
         // (ifull: the acquire that makes the cell's table visible here)
         bool ok = !*vabort && tc::mbar_wait(&ifull[xb], (uint32_t)((j >> 1) & 1)) &&
                   tc::mbar_wait(&accfull[xb], (uint32_t)((j >> 1) & 1));
@@ -773,17 +787,19 @@ __global__ void __launch_bounds__(kTThreads, 1) fe_step_t_kernel(const __grid_co
         tc::tc_fence_after();
         if (128 * t + q * 32 < n) {
           const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + xb * 128u + (uint32_t)k0;
-          float* U = Ub + col;
+          float* U = Ub + col4;
 #pragma unroll
           for (int kb = 0; kb < 64; kb += 16) {
             float v[16];
             tc::tmem_ld16(taddr + (uint32_t)kb, v);
-            int dof[16];
+            // four lanes exchange four nodes, so that each holds four columns of one: a quarter of the adds
 #pragma unroll
-            for (int u = 0; u < 16; u += 4) *reinterpret_cast<int4*>(dof + u) = *reinterpret_cast<const int4*>(tab.dof + k0 + kb + u);
-#pragma unroll
-            for (int u = 0; u < 16; ++u)
-              red_add_f32(U + (int64_t)dof[u] * n, al * v[u], col < n && k0 + kb + u < nc);
+            for (int g4 = 0; g4 < 16; g4 += 4) {
+              quad_transpose(v + g4, lane);
+              const int i = k0 + kb + g4 + (lane & 3);
+              red_add_v4(U + (int64_t)tab.dof[i] * n, al * v[g4], al * v[g4 + 1], al * v[g4 + 2], al * v[g4 + 3],
+                         col4 < n && i < nc);
+            }
           }
         }
         tc::tc_fence_before();
