@@ -653,10 +653,10 @@ void oz_slice(cudaStream_t s, int64_t R, int64_t K, const double* X, int64_t rs,
 namespace {
 
 // Split-K count: the smallest with which the (tile, split) items fill whole rounds of one item per
-// persistent CTA to >= 90% (else the best found), each split keeping >= 2 chunks so that its
-// drains and final store stay amortised.
+// persistent CTA to >= 90% (else the best found); a few output tiles (N x N products) go down to one
+// chunk per split, since a chunk is 3.3 us of MMAs in a CTA.
 int choose_split(int tiles, int nchunks, int num_sms, double* eff_out) {
-  const int max_split = std::max(1, std::min(64, nchunks / 2));
+  const int max_split = std::max(1, std::min(64, nchunks));
   double best = -1.0;
   int nsplit = 1;
   for (int ns = 1; ns <= max_split; ++ns) {
