@@ -596,10 +596,10 @@ def run_kpoints(args, rank, world, local_rank):
 
 
 def filter_step_roofline(prof, prob, pk, steps_per_solve):
-    """Roofline of one degree step of the filter (the hot path of Algorithm 3) on the FE workload:
-    the fused tensor-core kernel does the whole step (gather of D^-1 R_Y, cell products, recurrence
-    terms and scatter into R_X), so its launches are the steps.  Algorithmic bytes per step:
-    4 block streams (R_Y gathered, R_X read and written, W read) of m N FP32 values plus the cell
+    """Roofline of the degree steps of the filter (the hot path of Algorithm 3) on the FE workload:
+    the fused tensor-core kernel does whole steps (gather of D^-1 R_Y, cell products, recurrence
+    terms and scatter into R_X), and one launch does all steps of a filter call.  Algorithmic bytes per
+    step: 4 block streams (R_Y gathered, R_X read and written, W read) of m N FP32 values plus the cell
     matrices in the operand precision, C n_c^2 s."""
     r = prof.get("fe_cell")
     if not r or not r["launches"] or r["ms"] <= 0:
@@ -608,16 +608,19 @@ def filter_step_roofline(prof, prob, pk, steps_per_solve):
     per_ms = r["ms"] / r["launches"]
     per_bytes = r["bytes"] / r["launches"]
     ach = per_bytes / (per_ms * 1e-3) / 1e9
-    # DRAM traffic of the kernel from the ncu capture of profiles/fe_step_kernel_fe12_n600.md (12^3 cells,
-    # 1.227 GB per launch), scaled by the units processed (cells x columns) to this launch
-    units = prob["fe"]["cell_dofs"].shape[0] * prob["block"]
-    traffic = 1.227e9 * units / (1728 * 600)
+    dofs = prob["fe"]["cell_dofs"]
+    one = 16.0 * prob["m"] * prob["block"] + 4.0 * dofs.shape[0] * dofs.shape[1] ** 2
+    steps = max(1, round(per_bytes / one))
+    # DRAM traffic of the kernel from the ncu capture of profiles/fe_step_t_kernel_fe10_n600.md (10^3 cells,
+    # two steps): 1.013 of the algorithmic bytes
+    traffic = 1.013 * per_bytes
     return {"bound": "hbm", "achieved": round(ach, 1), "peak": hbm, "unit": "GB/s", "frac": round(ach / hbm, 4),
-            "traffic": traffic, "traffic_source": "ncu dram__bytes_read+write of fe_step_kernel at 12^3 cells x 600 "
-                                                  "columns, scaled by cells x columns",
+            "traffic": traffic, "traffic_source": "ncu dram__bytes_read+write of fe_step_t_kernel at 10^3 cells x 600 "
+                                                  "columns, scaled by the algorithmic bytes",
             "peak_source": "measured HBM copy, MEASURED_PEAKS.json (of measured)",
-            "kernel": "fe_step_kernel (one launch = one degree step of Algorithm 3)",
-            "algorithmic_bytes_per_step": per_bytes, "per_launch_ms": round(per_ms, 4),
+            "kernel": "fe_step_t_kernel (one launch = all degree steps of Algorithm 3)",
+            "algorithmic_bytes_per_step": per_bytes / steps, "steps_per_launch": steps,
+            "per_launch_ms": round(per_ms, 4),
             "launches_per_solve": r["launches"], "tflops": round(r["flops"] / (r["ms"] * 1e-3) / 1e12, 2)}
 
 

@@ -493,8 +493,9 @@ __global__ void __launch_bounds__(kThreads, 1) fe_step_kernel(const __grid_const
 //   warps 18-21 gather: half tiles of 64 columns into a ring of stages
 // At 16^3 cells x 600 columns the step above took 857 us, and 610 us without any of its gathers and reds: its
 // chain of conversion, barrier and rewriting was the bound, not memory (0.41 ms at the copy rate).  This one takes
-// 533 us there; below about 64 columns, where half of its 128 lanes are idle, the other is faster (6^3 x 48: 11.0
-// against 13 us), so both stand and fe_step_tune picks by time.
+// 498 us there; below about 64 columns, where half of its 128 lanes are idle, a launch of the other is faster (6^3 x 48: 11.0
+// against 13 us; 10.3 us a step when one launch does them all), so both stand and fe_step_tune picks by time
+// for the graphs of the batched filters.
 constexpr int kTThreads = 704;
 constexpr int kTGather = 128;
 constexpr int kTStages = 3;

@@ -370,7 +370,7 @@ Kernel pick(int elems) {
 
 // One CTA per (row tile, K split), all resident: at least four splits, so that a share of up to 64 columns fits
 // the epilogue's registers, and N in one tile.  Against the per-step launches (whole filter calls, degree 20 to
-// 30): m = 1000, N = 60 330 -> 195 us; m = 1537, N = 99 BF16 470 -> 285 us; m = 4000, N = 240 1117 -> 760 us.
+// 30): m = 1000, N = 60 330 -> 180 us; m = 1537, N = 99 BF16 470 -> 263 us; m = 4000, N = 240 1117 -> 810 us.
 TcLoopPlan tc_loop_plan(int num_sms, int64_t M, int64_t N, bool bf16) {
   TcLoopPlan p;
   p.M = M;
