@@ -665,8 +665,12 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_smem_kernel(int n, const 
 // Exchange: CL = true, one thread-block cluster: q by st.async, a by one bulk copy per CTA, both
 // completing bytes on the receiver's mbarrier.  CL = false, a cooperative grid: 16-byte packets
 // {low word, tag, high word, tag} through L2 (xg: 4 n packets, zeroed), polled by the thread that
-// needs the entry; the tag is the step.  Both buffers alternate by step: a CTA sends step k + 2 only
-// after it has received step k + 1 from everyone, and those sent it after they had read step k.
+// needs the entry; the tag is the step.  Both buffers alternate by step.  A CTA takes part in step k only
+// while it owns a column c >= k + 2, that is, while it has something to send for step k + 1; then it is
+// done (the last P steps, one CTA after another), receives nothing more and writes nothing more, and the
+// owner of column n - 1, which stays to the end, writes the outputs of the steps whose pivot column's
+// owner has left.  So the two buffers are enough: step k + 2 is sent only after step k + 1 has arrived
+// from every CTA that took part in step k, and each of them sent it after it had read step k.
 // Every wait is bounded: on a timeout *err is set to 2 and all CTAs leave.
 // Warps 0-7: rows and columns; warp 8: the scalars.  Outputs as tridiag_smem_kernel, with H(:, k) = u
 // and tau = eta (the same reflector).
@@ -721,6 +725,9 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
   const int P = gridDim.x, r = blockIdx.x;  // (a cluster launch is one cluster)
   const int ld = (n + 1) & ~1;
   const int nqm = (n + P - 1) / P, nq = (n - r + P - 1) / P;  // owned columns c = r + q P
+  // the last column that CTA `rank` owns (negative: none); it takes part in steps k <= last - 2
+  auto last_col = [&](int rank) { return rank < n ? rank + (n - 1 - rank) / P * P : -1; };
+  const int steps = max(0, min(n - 2, last_col(r) - 1));
   double* sm = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(sm_raw) + 15) & ~uintptr_t(15));
   double* cols = sm;                       // nqm x ld
   double* xa = cols + (size_t)nqm * ld;    // CL: two buffers of a, two of q
@@ -751,22 +758,25 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
     tc::mbar_arrive_expect_tx(&qbar[k & 1], (uint32_t)(8 * (n - k - 1) + 8 * (ld - ((k + 1) & ~1))));
   };
   if (CL && tid == 0)
-    for (int k = 0; k < 2 && k + 2 < n; ++k) expect(k);
+    for (int k = 0; k < 2 && k < steps; ++k) expect(k);
 
   // this lane's view of CTA `lane` of the cluster
   uint32_t rq = 0, ra = 0, rb = 0;
+  int last = -1;  // the last column of that CTA
   if (CL && lane < P) {
+    last = last_col(lane);
     rq = mapa_u32(tc::smem_u32(xq), (uint32_t)lane);
     ra = mapa_u32(tc::smem_u32(xa), (uint32_t)lane);
     rb = mapa_u32(tc::smem_u32(qbar), (uint32_t)lane);
   }
 
   // rank-2 update of step k on the owned columns c >= k + 2 (UPD), the products with x' and, with
-  // `send`, what step k + 1 needs
+  // `send`, what step k + 1 needs, to the CTAs that take part in it
   auto pass = [&](int k, bool upd, bool send) {
     const int s0 = k + 2, rr = n - s0;  // rows s0 .. n - 1
     const int qa = s0 - r > 0 ? (s0 - r + P - 1) / P : 0;
     const int b = (k + 1) & 1;
+    const bool to = CL && last >= k + 3;
     // (columns go to the warps in an order that loads sub-partition 0, which also runs the scalars, last)
     for (int q = qa + (((warp + 3) & 3) | (warp & 4)); q < nq; q += 16) {
       const int q2 = q + 8;
@@ -825,7 +835,7 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
           const int i0 = s0 & ~1;
-          if (lane < P)
+          if (to)
             bulk_s2s(ra + (uint32_t)((b * ld + i0) * 8), tc::smem_u32(cols + (size_t)q * ld + i0),
                      (uint32_t)((ld - i0) * 8), rb + 8u * b);
         } else {
@@ -837,7 +847,7 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
       const double d1 = warp_sum_fx(a1);
       const double d2 = two ? warp_sum_fx(a2) : 0.0;
       if (CL) {
-        if (lane < P) {
+        if (to) {
           st_async_f64(rq + (uint32_t)((b * ld + c) * 8), d1, rb + 8u * b);
           if (two) st_async_f64(rq + (uint32_t)((b * ld + c2) * 8), d2, rb + 8u * b);
         }
@@ -887,8 +897,9 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
     if (r == 0 && tid == 0) d[0] = X[0];
     if (warp == 8) scalars(0);
     else pass(-1, false, true);
-    for (int k = 0; k + 2 < n; ++k) {
+    for (int k = 0; k < steps; ++k) {
       const int b = k & 1;
+      const bool writes = r == (k + P < n ? k % P : (n - 1) % P);  // the outputs of this step
       if (warp < 8) {
         const bool any = [&] {  // (warp-uniform) does this warp hold a row of the trailing block
           bool a = false;
@@ -902,7 +913,7 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
         for (int j = 0; j < TX_ROWS; ++j) qv[j] = av[j] = 0.0;
         if (CL) {
           ok = tc::mbar_wait(&qbar[b], (uint32_t)((k >> 1) & 1));
-          if (tid == 0 && ok && k + 4 < n) expect(k + 2);
+          if (tid == 0 && ok && k + 2 < steps) expect(k + 2);
           if (any) {
             q0 = xq[b * ld + k + 1];
             a0 = xa[b * ld + k + 1];
@@ -992,7 +1003,7 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
                 W[i] = w;
                 X[i] = x;
                 xr[j] = x;
-                if (k % P == r) {
+                if (writes) {
                   H[(size_t)k * n + i] = u[j];
                   if (i == k + 1) {
                     d[k + 1] = x;  // a_0 - 2 u_0 w_0: the next diagonal entry
@@ -1011,11 +1022,10 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
         if (tid == 0) atomicExch(err, 2);
         break;
       }
-      const bool more = k + 3 < n;
       if (warp == 8) {
-        if (more) scalars(k + 1);
+        if (k + 1 < steps) scalars(k + 1);
       } else {
-        pass(k, true, more);
+        pass(k, true, k + 3 < n);
       }
     }
     __syncthreads();
