@@ -679,8 +679,9 @@ __global__ void __launch_bounds__(kThreads, 1) fe_oz_kernel(const __grid_constan
         unsigned long long* out = reinterpret_cast<unsigned long long*>(p.Y + (int64_t)g * p.n);
         const int c0 = tile * kBN + hq * 16;
         // (top 2^32 + low) 2^(qs - 48), each part rounded to the accumulator's last place; qs <= 38 and top is below
-        // 2^40, so the left shift stays below 2^62
-        const int lt = max(qs - 16, 0), st = min(max(16 - qs, 0), 63), sl = min(48 - qs, 63);
+        // 2^40, so the left shift stays below 2^62.  (Right shifts end at 62, where the half unit is still a positive
+        // number: top and low are below 2^61, so a shift of 62 or more gives 0)
+        const int lt = max(qs - 16, 0), st = min(max(16 - qs, 0), 62), sl = min(48 - qs, 62);
         const long long rt = (1LL << st) >> 1, rl = (1LL << sl) >> 1;
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
