@@ -81,7 +81,14 @@ __device__ __forceinline__ double warp_sum(double v) {
 // into 26-bit limbs and added with redux.sync.  The result is within 1/8 unit in the last place of
 // the largest addend plus one rounding, closer than a tree of FP64 adds, and costs one FP64
 // instruction (a conversion) instead of five.  Non-finite addends take the FP64 tree (NaN and Inf
-// propagate); a result below the normal range is 0.
+// propagate); a result below the normal range is 0, one above it infinite.
+__device__ __forceinline__ double fx_scaled(long long t, uint32_t top) {  // t 2^(top - 1075 - 9 + 5)
+  const double d = __ll2double_rn(t);
+  const int he = __double2hiint(d), ef = ((he >> 20) & 0x7ff) + (int)top - 1079;
+  if (t == 0 || ef <= 0) return 0.0;
+  if (ef >= 0x7ff) return __hiloint2double((he & (int)0x80000000) | 0x7ff00000, 0);
+  return __hiloint2double(he + (((int)top - 1079) << 20), __double2loint(d));
+}
 __device__ __forceinline__ double warp_sum_fx(double v) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
   const uint32_t e0 = (hi >> 20) & 0x7ffu;
@@ -97,10 +104,7 @@ __device__ __forceinline__ double warp_sum_fx(double v) {
   const int h = (int)(f >> 52);
   const uint32_t sl = __reduce_add_sync(0xffffffffu, l), sm = __reduce_add_sync(0xffffffffu, m);
   const int sg = __reduce_add_sync(0xffffffffu, h);
-  const long long t = ((long long)sg << 47) + ((long long)sm << 21) + (long long)(sl >> 5);
-  const double d = __ll2double_rn(t);  // scaled by 2^(top - 1075 - 9 + 5) below
-  const int he = __double2hiint(d), ef = ((he >> 20) & 0x7ff) + (int)top - 1079;
-  return t != 0 && ef > 0 ? __hiloint2double(he + (((int)top - 1079) << 20), __double2loint(d)) : 0.0;
+  return fx_scaled(((long long)sg << 47) + ((long long)sm << 21) + (long long)(sl >> 5), top);
 }
 
 // 1 / sqrt(a) for a normal a > 0: FP32 seed y (22 bits), then one step of the third-order Householder
@@ -871,8 +875,8 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
       beta = -copysign(nx, alpha);
       u0 = copysign(g, alpha);  // alpha - beta
       eta = ri * rcp_h3(g);
-    } else if (s2 > 0.0) {
-      beta = eta = u0 = __longlong_as_double(0x7ff8000000000000LL);  // overflow of ||x||^2
+    } else if (s2 != 0.0) {
+      beta = eta = u0 = __longlong_as_double(0x7ff8000000000000LL);  // overflow of ||x||^2, or a NaN in x
     }
     const double ue = u0 * eta;
     if (lane == 0) {
@@ -1697,10 +1701,8 @@ __device__ __forceinline__ double warp_sum4_fx(const double (&v)[4], int lane) {
       top = tp;
     }
   }
-  const double d = __ll2double_rn(t);
-  const int he = __double2hiint(d), ef = ((he >> 20) & 0x7ff) + (int)top - 1079;
   if (top == 0x7ffu) return __longlong_as_double(0x7ff8000000000000LL);  // a non-finite addend
-  return t != 0 && ef > 0 ? __hiloint2double(he + (((int)top - 1079) << 20), __double2loint(d)) : 0.0;
+  return fx_scaled(t, top);
 }
 
 // The reflectors of the back-transform in groups of four, k0 = n - 3 - 4 g first: with p_a = v_a . z for the
