@@ -107,6 +107,8 @@ __device__ __forceinline__ double warp_sum_fx(double v) {
   return fx_scaled(((long long)sg << 47) + ((long long)sm << 21) + (long long)(sl >> 5), top);
 }
 
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
 // 1 / sqrt(a) for a normal a > 0: FP32 seed y (22 bits), then one step of the third-order Householder
 // iteration y (1 + e / 2 + 3 e^2 / 8), e = 1 - a y^2 (error e^3): 5 FP64 instructions.
 __device__ __forceinline__ double rsqrt_h3(double a) {
@@ -666,6 +668,8 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_smem_kernel(int n, const 
 // a (from the owner of column k + 1): every CTA then forms t, w and the next pivot column
 // x' = a - u w_0 - w u_0 for itself, all from the same bits, so nobody waits for an owner again.  One
 // pass over the owned columns applies the rank-2 update and forms the next products.
+// eta^2 and the products with it are formed on their own, which holds for ||x|| in 2^-240 .. 2^240.  Outside, u and
+// t are multiplied by the power of two nearest to 1 / ||x|| (and eta by its inverse square), which leaves u w^T as it is.
 // Exchange: CL = true, one thread-block cluster: q by st.async, a by one bulk copy per CTA, both
 // completing bytes on the receiver's mbarrier.  CL = false, a cooperative grid: 16-byte packets
 // {low word, tag, high word, tag} through L2 (xg: 4 n packets, zeroed), polled by the thread that
@@ -677,7 +681,7 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_smem_kernel(int n, const 
 // from every CTA that took part in step k, and each of them sent it after it had read step k.
 // Every wait is bounded: on a timeout *err is set to 2 and all CTAs leave.
 // Warps 0-7: rows and columns; warp 8: the scalars.  Outputs as tridiag_smem_kernel, with H(:, k) = u
-// and tau = eta (the same reflector).
+// and tau = eta (the same reflector, whatever the power of two).
 constexpr int TX_THREADS = 288;
 constexpr int TX_ROWS = 4;  // rows per thread: n <= 1024
 
@@ -724,7 +728,8 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
                                                                  int* err) {
   extern __shared__ double sm_raw[];
   __shared__ __align__(8) uint64_t qbar[2], sbar;
-  __shared__ double red[8], scal[6];  // scal: beta, eta, -eta^2 / 2, u_0, u_0 eta, -u_0 eta^2
+  // scal: beta, eta, -eta^2 / 2, u_0, u_0 eta, -u_0 eta^2 (of the scaled u), the power of two, beta unscaled
+  __shared__ double red[8], scal[8];
   __shared__ int abort_flag[2];
   const int P = gridDim.x, r = blockIdx.x;  // (a cluster launch is one cluster)
   const int ld = (n + 1) & ~1;
@@ -866,10 +871,18 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
     double s2 = 0.0;
     for (int i = k + 2 + lane; i < n; i += 32) s2 = fma(X[i], X[i], s2);
     s2 = warp_sum_fx(s2);
-    const double alpha = X[k + 1];
-    double beta = alpha, eta = 0.0, u0 = 0.0;
-    const double nx2 = fma(alpha, alpha, s2);
+    double alpha = X[k + 1];
+    double beta = alpha, eta = 0.0, u0 = 0.0, sig = 1.0, isig = 1.0;
+    double nx2 = fma(alpha, alpha, s2);
     if (s2 > 0.0 && nx2 < DBL_MAX) {
+      const int ex = exp_field(nx2) - 1023;
+      if (abs(ex) > 480) {
+        const int h = ex >> 1;
+        sig = __hiloint2double((1023 - h) << 20, 0);
+        isig = __hiloint2double((1023 + h) << 20, 0);
+        nx2 = nx2 * sig * sig;
+        alpha *= sig;
+      }
       // eta = 1 / (||x||^2 + |alpha| ||x||) = (1 / ||x||) / (||x|| + |alpha|)
       const double ri = rsqrt_h3(nx2), nx = nx2 * ri, g = nx + fabs(alpha);
       beta = -copysign(nx, alpha);
@@ -886,6 +899,8 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
       scal[3] = u0;
       scal[4] = ue;
       scal[5] = -(ue * eta);
+      scal[6] = sig;
+      scal[7] = beta * isig;
     }
     __syncwarp();
     if (lane == 0) tc::mbar_arrive(&sbar);
@@ -965,6 +980,15 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
         ok = tc::mbar_wait(&sbar, (uint32_t)(k & 1)) && ok;
         if (!ok) abort_flag[b] = 1;
         const double beta = scal[0], eta = scal[1], mh = scal[2], u0 = scal[3], ue = scal[4], f0 = scal[5];
+        const double sig = scal[6];
+        if (__double2hiint(sig) != 0x3ff00000) {  // not 1
+#pragma unroll
+          for (int j = 0; j < TX_ROWS; ++j) {
+            xr[j] *= sig;
+            qv[j] *= sig;
+          }
+          q0 *= sig;
+        }
         double u[TX_ROWS], z[TX_ROWS], y[TX_ROWS], g = 0.0, e0 = 0.0;
         if (any) {
 #pragma unroll
@@ -1011,7 +1035,7 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
                   H[(size_t)k * n + i] = u[j];
                   if (i == k + 1) {
                     d[k + 1] = x;  // a_0 - 2 u_0 w_0: the next diagonal entry
-                    e[k] = beta;
+                    e[k] = scal[7];
                     tau[k] = eta;
                   }
                   if (k + 3 == n && i == n - 1) e[n - 2] = x;
@@ -1251,7 +1275,6 @@ __device__ __forceinline__ double scale2(double x, int k) {
   const int nf = ef + k;
   return ef != 0 && nf > 0 ? __hiloint2double(hi + (k << 20), __double2loint(x)) : 0.0;
 }
-__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
 // FP32 Sturm count of T / ||T|| at x.
 __device__ __forceinline__ int sturm_count_f32(int n, const float* d, const float* e2, float x) {

@@ -32,3 +32,36 @@ def test_overflowing_sum_of_squares_is_not_a_result(N):
     except RChFSIError:
         return
     assert not np.isfinite(ev).all()
+
+
+# tolerances of the other projected-eigenproblem tests: 50 N eps ||M|| for values, 200 N eps for orthonormality
+@pytest.mark.parametrize("N", [12, 60, 130, 340])
+@pytest.mark.parametrize("power", [-480, -400, -300, -250, 250, 300, 400, 480])
+def test_scaled_matrices(N, power):
+    """Scaling A by a power of two scales the eigenvalues."""
+    A = _full(N, 2)
+    ref = np.linalg.eigvalsh(A)
+    s = Solver(N, nev=1, block=N)
+    s.set_dense(2.0 ** power * A)
+    X, ev = s.rayleigh_ritz(np.eye(N))
+    eps = np.finfo(float).eps
+    assert np.abs(ev * 2.0 ** -power - ref).max() <= 50 * N * eps * np.abs(ref).max()
+    assert np.abs(X.T @ X - np.eye(N)).max() <= 200 * N * eps
+
+
+@pytest.mark.parametrize("N", [12, 60, 340])
+@pytest.mark.parametrize("power", [-200, -260, -400, -505])
+def test_columns_of_tiny_entries(N, power):
+    """Off-diagonal entries far below the diagonal: in one half of the matrix, then in all of it."""
+    eps = np.finfo(float).eps
+    for h in (N // 2, 0):
+        A = _full(N, 3)
+        A[h:, :] *= 2.0 ** power
+        A[:h, h:] *= 2.0 ** power
+        A[np.arange(h, N), np.arange(h, N)] = np.linspace(1.0, 2.0, N - h)
+        ref = np.linalg.eigvalsh(A)
+        s = Solver(N, nev=1, block=N, rr_mode="fp64")
+        s.set_dense(A)
+        X, ev = s.rayleigh_ritz(np.eye(N))
+        assert np.abs(ev - ref).max() <= 50 * N * eps * np.abs(ref).max()
+        assert np.abs(X.T @ X - np.eye(N)).max() <= 200 * N * eps
