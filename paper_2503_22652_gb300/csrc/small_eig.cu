@@ -298,8 +298,9 @@ __global__ void __launch_bounds__(256) chol_inv_smem_kernel(int n, const double*
 // units of 128 outputs (two threads each) so that a few tiles still spread over the SMs.
 // The factor of a tile (tile_factor): LDL^T by columns with the same row operations applied to the
 // identity, one thread per (row, column mod 8), one CTA barrier per column; the chain of a column is
-// its FMA, the reciprocal of the pivot (an FP32 seed and 3 FP64 instructions) and one product.  The
-// square roots are taken at the end, for all 32 pivots in one go.
+// its FMA, the reciprocal of the pivot (an FP32 seed and 3 FP64 instructions; a division for pivots at
+// the ends of the FP64 range) and one product.  The square roots are taken at the end, for all 32 pivots
+// in one go.
 // info: 0, or j + 1 for the first column j whose pivot is not positive (L and L^-1 are then not
 // written in full).
 // Measured (cold, one call; before: a barrier per phase, the diagonal tile on one CTA, L^-1 after the
@@ -332,7 +333,9 @@ __device__ __forceinline__ void tile_factor(TileSmem& T, const double* M, int n,
       if (w == jw) {
         const double d = __shfl_sync(0xffffffffu, a[jq], j);
         const bool good = d > 0.0 && d < DBL_MAX;
-        const double m = a[jq] * rcp_h3(good ? d : 1.0);
+        const double p = good ? d : 1.0;
+        // (rcp_h3 wants d and 1 / d normal)
+        const double m = (unsigned)(exp_field(p) - 3) <= 2040u ? a[jq] * rcp_h3(p) : a[jq] / p;
         T.col[buf][i] = a[jq];
         T.mul[buf][i] = m;
         T.L[i][j] = a[jq];
@@ -360,7 +363,7 @@ __device__ __forceinline__ void tile_factor(TileSmem& T, const double* M, int n,
     }
   }
   __syncthreads();
-  if (w == 0) T.rs[i] = rsqrt_h3(T.piv[i]);
+  if (w == 0) T.rs[i] = exp_field(T.piv[i]) != 0 ? rsqrt_h3(T.piv[i]) : rsqrt(T.piv[i]);
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < 4; ++q) {

@@ -65,3 +65,19 @@ def test_columns_of_tiny_entries(N, power):
         X, ev = s.rayleigh_ritz(np.eye(N))
         assert np.abs(ev - ref).max() <= 50 * N * eps * np.abs(ref).max()
         assert np.abs(X.T @ X - np.eye(N)).max() <= 200 * N * eps
+
+
+@pytest.mark.parametrize("mode", ["emulated", "fp64"])
+@pytest.mark.parametrize("power", [-1040, -1030, -1022, 1021, 1022])
+def test_gram_matrices_at_the_ends_of_the_range(power, mode):
+    """A and B scaled alike: the eigenvalues stay.  Tolerance: 50 N units of the scaled matrices' last place."""
+    N = 40
+    r = np.random.default_rng(1)
+    A, B = r.uniform(-1.0, 1.0, (N, N)), r.uniform(-0.0125, 0.0125, (N, N))
+    A, B = A + A.T, np.eye(N) + B + B.T
+    L = np.linalg.inv(np.linalg.cholesky(B))
+    ref = np.linalg.eigvalsh(L @ A @ L.T)
+    s = Solver(N, nev=1, block=N, rr_mode=mode)
+    s.set_dense(np.ldexp(A, power), B=np.ldexp(B, power))
+    _, ev = s.rayleigh_ritz(np.eye(N))
+    assert np.abs(ev - ref).max() <= 50 * N * max(np.finfo(float).eps, 2.0 ** (-1074 - power)) * np.abs(ref).max()
