@@ -535,6 +535,20 @@ static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, co
   c.last_applies = (int64_t)co.size() + (chfsi ? 1 : 0);
 }
 
+// The device footprint (as check_budget counts it) of a dense TF32 / BF16 filter call that takes the one-launch
+// loop: what is there, and what the call will have added, the operator copy, R_X, R_Y and W, the tables and the
+// loop's workspace.
+static size_t loop_footprint(const rchfsi_ctx& c, const TcLoopPlan& loop, bool bf, bool chfsi, size_t table_doubles) {
+  const DenseOp& d = c.dense;
+  const size_t mp = padded(c.p.m), es = bf ? 2 : 4;
+  auto grow = [](size_t have, size_t need) { return need > have ? need - have : 0; };
+  const size_t op = bf ? (chfsi ? d.DA16 : d.AD16).bytes() : (chfsi ? d.DAtf : d.ADtf).bytes();
+  return device_bytes(c) + grow(op, (size_t)c.p.m * mp * es) +
+         3 * grow(bf ? c.w.R16a.bytes() : c.w.R32a.bytes(), mp * c.p.block * es) +
+         grow(c.w.lamtab.bytes(), table_doubles * sizeof(double)) +
+         grow(c.w.split.bytes(), loop.ws_floats * sizeof(float));
+}
+
 bool filter_takes_rows(const rchfsi_ctx& c) {
   return !c.cplx && c.p.precision != RCHFSI_FP64 && !(c.op_kind == RCHFSI_OP_DENSE && c.dense.has_dinv_dense);
 }
@@ -556,23 +570,28 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
     if (c.w.loop.M != c.p.m || c.w.loop.N != N || c.w.loop.bf16 != bf)
       c.w.loop = tc_loop_plan(c.num_sms, c.p.m, N, bf);
     loop = c.w.loop;
-    if (loop.ok && c.p.hbm_budget_bytes && c.w.split.n < loop.ws_floats &&
-        device_bytes(c) - c.w.split.bytes() + loop.ws_floats * sizeof(float) > c.p.hbm_budget_bytes)
-      loop.ok = false;
-    if (loop.ok) c.w.split.ensure(loop.ws_floats);
   }
   // the fused FE steps likewise, whatever the mesh
   const bool fe_loop = c.op_kind == RCHFSI_OP_FE_CELL && !chfsi && p >= 2 && p - 1 <= kTableSteps &&
                        fe_step_supported(*c.fe, N, c.p.precision);
   // one buffer: the Lambda table, and for a loop the coefficients and Lambda rows 1 .. p - 1 in FP32 and the
   // counters on 128-byte lines
-  const bool tables = loop.ok || fe_loop;
+  bool tables = loop.ok || fe_loop;
   const size_t coef_at = (size_t)(p + 1) * N;
-  const size_t ncoef = tables ? ((size_t)3 * loop_steps + 3) / 4 * 4 : 0;  // (the rows start on 16 bytes)
-  const size_t floats = tables ? ncoef + (chfsi ? 0 : (size_t)loop_steps * N) : 0;
+  const size_t ncoef = ((size_t)3 * loop_steps + 3) / 4 * 4;  // (the rows start on 16 bytes)
+  const size_t floats = ncoef + (chfsi ? 0 : (size_t)loop_steps * N);
   const size_t lam_at = (coef_at + 1) / 2 * 2;
   const size_t cnt_at = (lam_at + (floats + 1) / 2 + 15) / 16 * 16;
   const size_t ncnt = loop.ok ? loop.counters : fe_loop ? 32 : 0;
+  if (loop.ok) {
+    if (c.p.hbm_budget_bytes &&
+        loop_footprint(c, loop, c.p.precision == RCHFSI_BF16, chfsi, cnt_at + ncnt / 2) > c.p.hbm_budget_bytes) {
+      if (c.w.split.n >= loop.ws_floats) c.w.split.release();  // (the steps need less)
+      loop.ok = tables = false;
+    } else {
+      c.w.split.ensure(loop.ws_floats);
+    }
+  }
   const size_t total = tables ? cnt_at + ncnt / 2 : coef_at;
   double* dtab = c.w.lamtab.ensure(total);
   LoopTables ls;
@@ -599,7 +618,7 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
     t.coef = const_cast<float*>(ls.coef);
     t.lamf = const_cast<float*>(ls.lam);
     t.counters = ls.counters;
-    t.ncounters = (int)ncnt;
+    t.ncounters = tables ? (int)ncnt : 0;
     filter_tables(c.s, t);
   } else {
     if (chfsi) {
