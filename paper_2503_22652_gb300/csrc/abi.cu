@@ -210,8 +210,8 @@ void store_any(rchfsi_ctx& c, const double* src_col, double* dst, const std::vec
 // complex eigenvectors.  Each complex eigenpair appears as two real ones with equal eigenvalues,
 // spanning {x, i x}; for an isolated pair the first member is taken.  A cluster of more than two
 // equal eigenvalues (a complex eigenvalue of multiplicity > 1) is orthonormalised in the complex
-// B inner product (Gram-Schmidt on the device, using B X), dropping members that depend on the ones
-// already kept.  X, AX and BX (column-major, 2m rows; AX may be null) receive the same column
+// B inner product (Gram-Schmidt on the device, using B X), leaving out members that depend on the ones
+// kept.  X, AX and BX (column-major, 2m rows; AX may be null) receive the same column
 // operations, so they stay consistent.
 std::vector<int> select_complex(rchfsi_ctx& c, const std::vector<double>& ev, double* X, double* AX, double* BX) {
   const int n2 = (int)ev.size();
@@ -229,23 +229,32 @@ std::vector<int> select_complex(rchfsi_ctx& c, const std::vector<double>& ev, do
       out.push_back(k);
     } else {
       std::vector<int> kept;
-      for (int j = k; j < e && (int)kept.size() < size / 2; ++j) {
-        for (int l : kept) {
+      std::vector<char> used(size, 0);
+      // Of the members' squared norms past the kept ones' span, the mean over the cluster is the share of the pairs
+      // still to be found: in a large cluster the last ones may all be short.  So members left out are
+      // looked at again with a lower limit (and orthogonalised twice) until every pair has its vector.
+      for (double limit = 0.25; limit > 1e-6 && (int)kept.size() < size / 2; limit *= 0.25) {
+        for (int j = k; j < e && (int)kept.size() < size / 2; ++j) {
+          if (used[j - k]) continue;
           double h[2];
-          cplx_dot(c.s, c.mc, X, BX, l, j, d);
+          for (int rep = 0; rep < (limit < 0.25 ? 2 : 1); ++rep)
+            for (int l : kept) {
+              cplx_dot(c.s, c.mc, X, BX, l, j, d);
+              RC_CUDA(cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, c.s));
+              RC_CUDA(cudaStreamSynchronize(c.s));
+              cplx_axpy(c.s, c.mc, X, AX, BX, l, j, h[0], h[1], 1.0);
+            }
+          cplx_dot(c.s, c.mc, X, BX, j, j, d);
           RC_CUDA(cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, c.s));
           RC_CUDA(cudaStreamSynchronize(c.s));
-          cplx_axpy(c.s, c.mc, X, AX, BX, l, j, h[0], h[1], 1.0);
-        }
-        double h[2];
-        cplx_dot(c.s, c.mc, X, BX, j, j, d);
-        RC_CUDA(cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, c.s));
-        RC_CUDA(cudaStreamSynchronize(c.s));
-        if (h[0] > 0.25) {
-          cplx_axpy(c.s, c.mc, X, AX, BX, j, j, 0.0, 0.0, 1.0 / std::sqrt(h[0]));
-          kept.push_back(j);
+          if (h[0] > limit) {
+            cplx_axpy(c.s, c.mc, X, AX, BX, j, j, 0.0, 0.0, 1.0 / std::sqrt(h[0]));
+            kept.push_back(j);
+            used[j - k] = 1;
+          }
         }
       }
+      std::sort(kept.begin(), kept.end());
       for (int j : kept)
         if ((int)out.size() < c.Nc) out.push_back(j);
     }
