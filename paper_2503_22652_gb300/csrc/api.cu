@@ -497,13 +497,14 @@ static void filter_fe(rchfsi_ctx& c, const double* X, const double* W, int p, co
     } else if (!co.empty()) {
       float* lamf = c.w.lamtab_f.ensure((size_t)(p + 1) * N);  // the Lambda table in FP32 for the kernel
       cast_f64_to_f32(c.s, (int64_t)(p + 1) * N, lamtab, lamf, 1.0, 0);
+      const int tile = fe_step_tile(f, N, c.num_sms, p - 1 <= kTableSteps);
       for (int k = 2; k <= p; ++k) {
         double cf[3];
         fused_coefs(co, sc, k, cf);
         FeStepPart parts[4];
         const int np = fe_step_parts(f, RY, Wl, RX, lamf + (size_t)(k - 1) * N, N, (float)cf[0], (float)cf[1],
                                      (float)cf[2], nullptr, parts);
-        fe_step_batch(c.s, parts, np, 128, c.num_sms);
+        fe_step_batch(c.s, parts, np, tile, c.num_sms);
         std::swap(RX, RY);
       }
     }
@@ -571,9 +572,9 @@ void filter_internal(rchfsi_ctx& c, const double* X, const double* lam, const do
       c.w.loop = tc_loop_plan(c.num_sms, c.p.m, N, bf);
     loop = c.w.loop;
   }
-  // the fused FE steps likewise, whatever the mesh
+  // the fused FE steps likewise, where their tile is the wide one
   const bool fe_loop = c.op_kind == RCHFSI_OP_FE_CELL && !chfsi && p >= 2 && p - 1 <= kTableSteps &&
-                       fe_step_supported(*c.fe, N, c.p.precision);
+                       fe_step_supported(*c.fe, N, c.p.precision) && fe_step_tile(*c.fe, N, c.num_sms, true) == 128;
   // one buffer: the Lambda table, and for a loop the coefficients and Lambda rows 1 .. p - 1 in FP32 and the
   // counters on 128-byte lines
   bool tables = loop.ok || fe_loop;

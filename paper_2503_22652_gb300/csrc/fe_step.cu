@@ -494,8 +494,8 @@ __global__ void __launch_bounds__(kThreads, 1) fe_step_kernel(const __grid_const
 // At 16^3 cells x 600 columns the step above took 857 us, and 610 us without any of its gathers and reds: its
 // chain of conversion, barrier and rewriting was the bound, not memory (0.41 ms at the copy rate).  This one takes
 // 498 us there; below about 64 columns, where half of its 128 lanes are idle, a launch of the other is faster (6^3 x 48: 11.0
-// against 13 us; 10.3 us a step when one launch does them all), so both stand and fe_step_tune picks by time
-// for the graphs of the batched filters.
+// against 13 us; 10.3 us a step when one launch does them all), so both stand: fe_step_tile picks for a single
+// filter, fe_step_tune by time for the graphs of the batched filters.
 constexpr int kTThreads = 704;
 constexpr int kTGather = 128;
 constexpr int kTStages = 3;
@@ -939,6 +939,18 @@ std::map<std::tuple<int, int64_t, int, int>, int> g_tune;
 bool fe_step_supported(const FeOp& op, int n, int precision) {
   return precision == RCHFSI_TF32 && n % 4 == 0 && n >= 4 && op.nc <= kNCP && op.own_pos.p != nullptr &&
          op.own_max <= kWRows;
+}
+
+// Up to 32 columns fill a quarter of the 128 lanes of the transposed step, whose time per cell does not depend on the
+// width below 64; the other form's tile of 32 columns takes less, and loses a launch per step.  So it is taken where
+// there are at least four cell products per SM, or where the steps do not fit one launch anyway.  Whole calls in
+// us, 128 in one launch / 32 per step, degree 20: 16 columns 6^3 cells 302 / 325, 7^3 365 / 363, 8^3 442 / 410,
+// 9^3 538 / 459, 10^3 689 / 583, 14^3 1592 / 1354; 32 columns 8^3 443 / 452, 9^3 537 / 500, 10^3 700 / 630, 14^3
+// 1603 / 1440; 36 columns (two tiles) 8^3 440 / 570, 14^3 1607 / 1966; complex 32 columns 4^3 365 / 362, 6^3 669 / 637,
+// 8^3 1325 / 1158.  Degree 110, one launch per step either way, 32 columns: 6^3 1514 / 1297, 10^3 3555 / 2885.
+int fe_step_tile(const FeOp& op, int n, int num_sms, bool loop) {
+  const int64_t items = op.n_cells * (op.cplx ? 4 : 1);
+  return n <= 32 && (!loop || items >= 4 * (int64_t)num_sms) ? 32 : 128;
 }
 
 void fe_step_prepare(cudaStream_t s, FeOp& op) {

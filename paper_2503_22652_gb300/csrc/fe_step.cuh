@@ -50,7 +50,11 @@ struct FeStepLoop {
 void fe_step_batch(cudaStream_t s, const FeStepPart* parts, int nparts, int BN, int num_sms,
                    const FeStepLoop* loop = nullptr);
 
-// Column tile for this operator and width, chosen by timing the candidates once per shape on the
+// Column tile of a single filter of n columns: 128, in one launch where `loop` says that its steps fit one, or 32,
+// one launch per step.
+int fe_step_tile(const FeOp& op, int n, int num_sms, bool loop);
+
+// Column tile for this operator and width in a batch, chosen by timing the candidates once per shape on the
 // problem's own data (into a scratch output); cached.
 int fe_step_tune(cudaStream_t s, int num_sms, FeOp& op, int n, const float* V, const float* W, const float* lam);
 
