@@ -85,9 +85,9 @@ __device__ __forceinline__ double warp_sum(double v) {
 __device__ __forceinline__ double fx_scaled(long long t, uint32_t top) {  // t 2^(top - 1075 - 9 + 5)
   const double d = __ll2double_rn(t);
   const int he = __double2hiint(d), ef = ((he >> 20) & 0x7ff) + (int)top - 1079;
-  if (t == 0 || ef <= 0) return 0.0;
-  if (ef >= 0x7ff) return __hiloint2double((he & (int)0x80000000) | 0x7ff00000, 0);
-  return __hiloint2double(he + (((int)top - 1079) << 20), __double2loint(d));
+  const bool over = ef >= 0x7ff, in = t != 0 && ef > 0;  // (selects: a branch here is on every sum's path)
+  const int hi = over ? (he & (int)0x80000000) | 0x7ff00000 : he + (((int)top - 1079) << 20);
+  return __hiloint2double(in ? hi : 0, in && !over ? __double2loint(d) : 0);
 }
 __device__ __forceinline__ double warp_sum_fx(double v) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
@@ -313,6 +313,9 @@ struct TileSmem {
   int bad;
 };
 
+// (behind a call: inlined, its code would stand in every unrolled column)
+__device__ __noinline__ double div_f64(double a, double b) { return a / b; }
+
 // Factor tile (K, K) of M (column-major n x n, lower triangle) into T.L and T.D; T.bad = 0, or j + 1
 // for the first pivot j that is not positive and finite.  256 threads.
 __device__ __forceinline__ void tile_factor(TileSmem& T, const double* M, int n, int K) {
@@ -335,7 +338,7 @@ __device__ __forceinline__ void tile_factor(TileSmem& T, const double* M, int n,
         const bool good = d > 0.0 && d < DBL_MAX;
         const double p = good ? d : 1.0;
         // (rcp_h3 wants d and 1 / d normal)
-        const double m = (unsigned)(exp_field(p) - 3) <= 2040u ? a[jq] * rcp_h3(p) : a[jq] / p;
+        const double m = (unsigned)(exp_field(p) - 3) <= 2040u ? a[jq] * rcp_h3(p) : div_f64(a[jq], p);
         T.col[buf][i] = a[jq];
         T.mul[buf][i] = m;
         T.L[i][j] = a[jq];
@@ -875,14 +878,14 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
     for (int i = k + 2 + lane; i < n; i += 32) s2 = fma(X[i], X[i], s2);
     s2 = warp_sum_fx(s2);
     double alpha = X[k + 1];
-    double beta = alpha, eta = 0.0, u0 = 0.0, sig = 1.0, isig = 1.0;
+    double beta = alpha, eta = 0.0, u0 = 0.0, sig = 1.0;
+    int h = 0;  // outside 2^-240 .. 2^240: the exponent of ||x||
     double nx2 = fma(alpha, alpha, s2);
     if (s2 > 0.0 && nx2 < DBL_MAX) {
       const int ex = exp_field(nx2) - 1023;
       if (abs(ex) > 480) {
-        const int h = ex >> 1;
+        h = ex >> 1;
         sig = __hiloint2double((1023 - h) << 20, 0);
-        isig = __hiloint2double((1023 + h) << 20, 0);
         nx2 = nx2 * sig * sig;
         alpha *= sig;
       }
@@ -903,7 +906,8 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
       scal[4] = ue;
       scal[5] = -(ue * eta);
       scal[6] = sig;
-      scal[7] = beta * isig;
+      if (h != 0) beta *= __hiloint2double((1023 + h) << 20, 0);
+      scal[7] = beta;
     }
     __syncwarp();
     if (lane == 0) tc::mbar_arrive(&sbar);
