@@ -80,21 +80,20 @@ __device__ __forceinline__ double warp_sum(double v) {
 // lanes' significands are aligned to the largest exponent (9 guard bits below its last place), cut
 // into 26-bit limbs and added with redux.sync.  The result is within 1/8 unit in the last place of
 // the largest addend plus one rounding, closer than a tree of FP64 adds, and costs one FP64
-// instruction (a conversion) instead of five.  Non-finite addends take the FP64 tree (NaN and Inf
-// propagate); a result below the normal range is 0, one above it infinite.
+// instruction (a conversion) instead of five.  Non-finite addends, and such that a sum of 32 may leave the
+// range, take the FP64 tree (NaN and Inf propagate); a result below the normal range is 0.
+constexpr uint32_t kFxTop = 0x7f8;  // the largest exponent field the integer sum takes is one less
 __device__ __forceinline__ double fx_scaled(long long t, uint32_t top) {  // t 2^(top - 1075 - 9 + 5)
   const double d = __ll2double_rn(t);
   const int he = __double2hiint(d), ef = ((he >> 20) & 0x7ff) + (int)top - 1079;
-  const bool over = ef >= 0x7ff, in = t != 0 && ef > 0;  // (selects: a branch here is on every sum's path)
-  const int hi = over ? (he & (int)0x80000000) | 0x7ff00000 : he + (((int)top - 1079) << 20);
-  return __hiloint2double(in ? hi : 0, in && !over ? __double2loint(d) : 0);
+  return t != 0 && ef > 0 ? __hiloint2double(he + (((int)top - 1079) << 20), __double2loint(d)) : 0.0;
 }
 __device__ __forceinline__ double warp_sum_fx(double v) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
   const uint32_t e0 = (hi >> 20) & 0x7ffu;
   const uint32_t ex = max(e0, 1u);
   const uint32_t top = __reduce_max_sync(0xffffffffu, ex);
-  if (top == 0x7ffu) return warp_sum(v);
+  if (top >= kFxTop) return warp_sum(v);
   const uint32_t sh = min(top - ex, 63u);
   const uint32_t mh = (hi & 0xfffffu) | (e0 ? 0x100000u : 0u);
   const unsigned long long mant = ((((unsigned long long)mh << 32) | lo) << 9) >> sh;
@@ -298,9 +297,10 @@ __global__ void __launch_bounds__(256) chol_inv_smem_kernel(int n, const double*
 // units of 128 outputs (two threads each) so that a few tiles still spread over the SMs.
 // The factor of a tile (tile_factor): LDL^T by columns with the same row operations applied to the
 // identity, one thread per (row, column mod 8), one CTA barrier per column; the chain of a column is
-// its FMA, the reciprocal of the pivot (an FP32 seed and 3 FP64 instructions; a division for pivots at
-// the ends of the FP64 range) and one product.  The square roots are taken at the end, for all 32 pivots
-// in one go.
+// its FMA, the reciprocal of the pivot (an FP32 seed and 3 FP64 instructions) and one product.  The
+// square roots are taken at the end, for all 32 pivots in one go.  Those want pivots and reciprocals
+// that are normal: where A(0, 0) lies outside 2^-400 .. 2^400, A is scaled by a power of four on entry and the results
+// on exit (the pivots of a matrix that can be factored are within its condition number of each other).
 // info: 0, or j + 1 for the first column j whose pivot is not positive (L and L^-1 are then not
 // written in full).
 // Measured (cold, one call; before: a barrier per phase, the diagonal tile on one CTA, L^-1 after the
@@ -312,9 +312,6 @@ struct TileSmem {
   double col[2][CB], mul[2][CB], piv[CB], rs[CB];
   int bad;
 };
-
-// (behind a call: inlined, its code would stand in every unrolled column)
-__device__ __noinline__ double div_f64(double a, double b) { return a / b; }
 
 // Factor tile (K, K) of M (column-major n x n, lower triangle) into T.L and T.D; T.bad = 0, or j + 1
 // for the first pivot j that is not positive and finite.  256 threads.
@@ -336,9 +333,7 @@ __device__ __forceinline__ void tile_factor(TileSmem& T, const double* M, int n,
       if (w == jw) {
         const double d = __shfl_sync(0xffffffffu, a[jq], j);
         const bool good = d > 0.0 && d < DBL_MAX;
-        const double p = good ? d : 1.0;
-        // (rcp_h3 wants d and 1 / d normal)
-        const double m = (unsigned)(exp_field(p) - 3) <= 2040u ? a[jq] * rcp_h3(p) : div_f64(a[jq], p);
+        const double m = a[jq] * rcp_h3(good ? d : 1.0);
         T.col[buf][i] = a[jq];
         T.mul[buf][i] = m;
         T.L[i][j] = a[jq];
@@ -366,7 +361,7 @@ __device__ __forceinline__ void tile_factor(TileSmem& T, const double* M, int n,
     }
   }
   __syncthreads();
-  if (w == 0) T.rs[i] = exp_field(T.piv[i]) != 0 ? rsqrt_h3(T.piv[i]) : rsqrt(T.piv[i]);
+  if (w == 0) T.rs[i] = rsqrt_h3(T.piv[i]);
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -402,10 +397,13 @@ __global__ void __launch_bounds__(256) chol_inv_blocked_kernel(int n, const doub
   auto put = [&](double* M, int i, int j, double v) {
     if (i < n && j < n) __stcg(M + (size_t)j * n + i, v);
   };
+  // 2^-h A is factored (h even); 0 but at the ends of the range
+  const int f0 = exp_field(A[0]), e0 = f0 == 0x7ff ? 0 : f0 - 1023, h = abs(e0) > 400 ? e0 & ~1 : 0;
   // L = lower(A), Linv = I
   for (size_t e = (size_t)r * blockDim.x + tid; e < nn; e += (size_t)P * blockDim.x) {
     const size_t j = e / n, i = e - j * n;
-    __stcg(L + e, i >= j ? A[e] : 0.0);
+    const double v = i >= j ? A[e] : 0.0;
+    __stcg(L + e, h != 0 ? ldexp(v, -h) : v);
     __stcg(Linv + e, i == j ? 1.0 : 0.0);
   }
   grid.sync();
@@ -477,6 +475,13 @@ __global__ void __launch_bounds__(256) chol_inv_blocked_kernel(int n, const doub
       __syncthreads();
     }
     grid.sync();
+  }
+  if (h != 0) {
+    grid.sync();
+    for (size_t e = (size_t)r * blockDim.x + tid; e < nn; e += (size_t)P * blockDim.x) {
+      __stcg(L + e, ldexp(__ldcg(L + e), h / 2));
+      __stcg(Linv + e, ldexp(__ldcg(Linv + e), -h / 2));
+    }
   }
   if (r == 0 && tid == 0) *info = 0;
 }
@@ -674,8 +679,9 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_smem_kernel(int n, const 
 // a (from the owner of column k + 1): every CTA then forms t, w and the next pivot column
 // x' = a - u w_0 - w u_0 for itself, all from the same bits, so nobody waits for an owner again.  One
 // pass over the owned columns applies the rank-2 update and forms the next products.
-// eta^2 and the products with it are formed on their own, which holds for ||x|| in 2^-240 .. 2^240.  Outside, u and
-// t are multiplied by the power of two nearest to 1 / ||x|| (and eta by its inverse square), which leaves u w^T as it is.
+// eta^2 and the products with it are formed on their own, which holds for ||x|| = |beta| in 2^-240 .. 2^240.  Outside
+// (far_exp), u and t are multiplied by a power of two near 1 / ||x|| (and eta by its inverse square), which leaves
+// u w^T as it is.
 // Exchange: CL = true, one thread-block cluster: q by st.async, a by one bulk copy per CTA, both
 // completing bytes on the receiver's mbarrier.  CL = false, a cooperative grid: 16-byte packets
 // {low word, tag, high word, tag} through L2 (xg: 4 n packets, zeroed), polled by the thread that
@@ -688,6 +694,8 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_smem_kernel(int n, const 
 // Every wait is bounded: on a timeout *err is set to 2 and all CTAs leave.
 // Warps 0-7: rows and columns; warp 8: the scalars.  Outputs as tridiag_smem_kernel, with H(:, k) = u
 // and tau = eta (the same reflector, whatever the power of two).
+__device__ __forceinline__ bool far_exp(double beta) { return (unsigned)(exp_field(beta) - 783) > 480u; }
+
 constexpr int TX_THREADS = 288;
 constexpr int TX_ROWS = 4;  // rows per thread: n <= 1024
 
@@ -734,7 +742,8 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
                                                                  int* err) {
   extern __shared__ double sm_raw[];
   __shared__ __align__(8) uint64_t qbar[2], sbar;
-  // scal: beta, eta, -eta^2 / 2, u_0, u_0 eta, -u_0 eta^2 (of the scaled u), the power of two, beta unscaled
+  // scal: beta, then of the scaled u eta, -eta^2 / 2, u_0, u_0 eta, -u_0 eta^2; where far_exp(beta), the power of two
+  // and beta times it
   __shared__ double red[8], scal[8];
   __shared__ int abort_flag[2];
   const int P = gridDim.x, r = blockIdx.x;  // (a cluster launch is one cluster)
@@ -877,37 +886,39 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
     double s2 = 0.0;
     for (int i = k + 2 + lane; i < n; i += 32) s2 = fma(X[i], X[i], s2);
     s2 = warp_sum_fx(s2);
-    double alpha = X[k + 1];
-    double beta = alpha, eta = 0.0, u0 = 0.0, sig = 1.0;
-    int h = 0;  // outside 2^-240 .. 2^240: the exponent of ||x||
-    double nx2 = fma(alpha, alpha, s2);
-    if (s2 > 0.0 && nx2 < DBL_MAX) {
-      const int ex = exp_field(nx2) - 1023;
-      if (abs(ex) > 480) {
-        h = ex >> 1;
-        sig = __hiloint2double((1023 - h) << 20, 0);
-        nx2 = nx2 * sig * sig;
-        alpha *= sig;
-      }
+    const double alpha = X[k + 1];
+    double beta = alpha, eta = 0.0, u0 = 0.0;
+    const double nx2 = fma(alpha, alpha, s2);
+    auto reflect = [&](double al, double nn) {
       // eta = 1 / (||x||^2 + |alpha| ||x||) = (1 / ||x||) / (||x|| + |alpha|)
-      const double ri = rsqrt_h3(nx2), nx = nx2 * ri, g = nx + fabs(alpha);
-      beta = -copysign(nx, alpha);
-      u0 = copysign(g, alpha);  // alpha - beta
+      const double ri = rsqrt_h3(nn), nx = nn * ri, g = nx + fabs(al);
+      beta = -copysign(nx, al);
+      u0 = copysign(g, al);  // alpha - beta
       eta = ri * rcp_h3(g);
+    };
+    const bool some = s2 > 0.0 && nx2 < DBL_MAX;
+    if (some) {
+      reflect(alpha, nx2);
     } else if (s2 != 0.0) {
       beta = eta = u0 = __longlong_as_double(0x7ff8000000000000LL);  // overflow of ||x||^2, or a NaN in x
     }
+    if (lane == 0) scal[0] = beta;
+    if (far_exp(beta)) {
+      const int h = some ? exp_field(beta) - 1023 : 0;
+      const double sig = __hiloint2double((1023 - h) << 20, 0);
+      if (some) reflect(alpha * sig, nx2 * sig * sig);
+      if (lane == 0) {
+        scal[6] = sig;
+        scal[7] = beta;
+      }
+    }
     const double ue = u0 * eta;
     if (lane == 0) {
-      scal[0] = beta;
       scal[1] = eta;
       scal[2] = -0.5 * (eta * eta);
       scal[3] = u0;
       scal[4] = ue;
       scal[5] = -(ue * eta);
-      scal[6] = sig;
-      if (h != 0) beta *= __hiloint2double((1023 + h) << 20, 0);
-      scal[7] = beta;
     }
     __syncwarp();
     if (lane == 0) tc::mbar_arrive(&sbar);
@@ -986,9 +997,11 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
         }
         ok = tc::mbar_wait(&sbar, (uint32_t)(k & 1)) && ok;
         if (!ok) abort_flag[b] = 1;
-        const double beta = scal[0], eta = scal[1], mh = scal[2], u0 = scal[3], ue = scal[4], f0 = scal[5];
-        const double sig = scal[6];
-        if (__double2hiint(sig) != 0x3ff00000) {  // not 1
+        const double eta = scal[1], mh = scal[2], u0 = scal[3], ue = scal[4], f0 = scal[5];
+        double beta = scal[0];
+        if (far_exp(beta)) {
+          const double sig = scal[6];
+          beta = scal[7];
 #pragma unroll
           for (int j = 0; j < TX_ROWS; ++j) {
             xr[j] *= sig;
@@ -1042,7 +1055,7 @@ __global__ void __launch_bounds__(TX_THREADS) tridiag_xch_kernel(int n, const do
                   H[(size_t)k * n + i] = u[j];
                   if (i == k + 1) {
                     d[k + 1] = x;  // a_0 - 2 u_0 w_0: the next diagonal entry
-                    e[k] = scal[7];
+                    e[k] = scal[0];
                     tau[k] = eta;
                   }
                   if (k + 3 == n && i == n - 1) e[n - 2] = x;
@@ -1731,7 +1744,8 @@ __device__ __forceinline__ double warp_sum4_fx(const double (&v)[4], int lane) {
       top = tp;
     }
   }
-  if (top == 0x7ffu) return __longlong_as_double(0x7ff8000000000000LL);  // a non-finite addend
+  // (a non-finite addend, or one above 2^1016, which reflectors of norm up to 2^241 and unit vectors do not make)
+  if (top >= kFxTop) return __longlong_as_double(0x7ff8000000000000LL);
   return fx_scaled(t, top);
 }
 
