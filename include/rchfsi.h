@@ -107,8 +107,9 @@ typedef enum {
   RCHFSI_EIG_SYEVD = 0,  /* divide and conquer (cuSOLVER) */
   RCHFSI_EIG_JACOBI = 1, /* parallel cyclic Jacobi, one cooperative kernel, tolerance 1e-14 */
   RCHFSI_EIG_TRIDIAG = 2 /* this library's Householder tridiagonalisation (one thread-block cluster or
-                            cooperative grid), Sturm bisection and inverse iteration with Gram-Schmidt in
-                            clusters of numerically equal eigenvalues; falls back to RCHFSI_EIG_SYEVD for an
+                            cooperative grid), Sturm multisection with secant steps and twisted
+                            factorisations, inverse iteration with Gram-Schmidt in clusters of
+                            numerically equal eigenvalues; falls back to RCHFSI_EIG_SYEVD for an
                             order above 3072 or a cluster of more than 256 equal eigenvalues */
 } rchfsi_eig_mode;
 

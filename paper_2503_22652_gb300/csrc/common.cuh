@@ -210,7 +210,8 @@ void shift_diag_by_trace_f64(cudaStream_t s, int n, double* A, int lda, double f
 // Cholesky G = L L^T and L^-1 (small_eig.cu): A (n x n, col-major) destroyed; L, Linv lower triangular.
 int cholesky_inverse_f64(cudaStream_t s, int n, double* A, double* L, double* Linv, int* d_info, int num_sms,
                          DevBuf<double>& scratch);
-// Symmetric eigensolver (small_eig.cu: Householder tridiagonalisation, bisection, inverse iteration):
+// Symmetric eigensolver (small_eig.cu: Householder tridiagonalisation, Sturm multisection and twisted factorisations,
+// inverse iteration for clusters):
 // M destroyed; V (column-major eigenvectors) and evals ascending.  Returns false when it declines the
 // problem (order > 3072).  Enqueues only: *d_flag, read by the caller once the stream is synchronised, is
 // 0, 1 (V and evals are not valid: a cluster of close eigenvalues too large for inverse iteration) or 2

@@ -8,8 +8,7 @@
 // product is then 28 slice products A_c^(s) X_c^(t), s + t <= 6, each a 128 x BN x 128 tcgen05 MMA;
 // the products of one level L = s + t sum to an integer that FP32 holds exactly (levels <= 5; the
 // last level, weight 2^-48, at most one unit off), so the 7 level accumulators live in TMEM and are
-// folded once per tile, in float-float (a 2^-48 relative rounding per cell contribution, the order
-// of an FP64 dot product's own rounding over the 125 terms of a cell row).
+// folded once per tile into two 64-bit integers, exactly.
 //
 // The cell contributions are summed in 64-bit fixed point: entry (d, j) holds V with value
 // V 2^(E_d + ex_j + H - 62), E_d the largest row exponent of the cell rows that reach dof d and H
@@ -31,10 +30,10 @@
 //   warps 2-3  gather: 16-byte cp.async, eight lanes per row, of the rows' 64 columns of each slice
 //              plane into the MN-major 128-byte-swizzled image X_c^(t), slice by slice as the
 //              previous item releases them (slice 0, freed last, alternates between two images);
-//   warps 4-19 epilogue (four per TMEM lane quarter, 16 columns each): folds level L into a
-//              float-float (hi, lo) pair as soon as pass L is done and frees its block, then
-//              converts to the fixed-point grid by integer arithmetic and scatters with 64-bit
-//              integer atomics while the next item's MMAs run.
+//   warps 4-19 epilogue (four per TMEM lane quarter, 16 columns each): folds level L into the
+//              integers (levels 0-2 and 3-6) as soon as pass L is done and frees its block, then
+//              shifts both to the fixed-point grid, rounding each, and scatters their sum with
+//              64-bit integer atomics while the next item's MMAs run.
 // Every mbarrier wait is bounded; on a timeout the kernel raises the error flag and unwinds.
 #include "fe.cuh"
 #include "oz_digits.cuh"

@@ -11,15 +11,15 @@
 // 7 for the group and one spare, rotated so that the next group's first writes go to blocks in the
 // order they are freed; warps 2-17 (four per TMEM lane quarter, 16 columns each) fold level L of a
 // group as soon as the group's pass L is done: tcgen05.ld and one 64-bit multiply-add into exact integer
-// accumulators.  The final value, two conversions scaled by exponent arithmetic and one FP64 add, is stored (or, with split-K, written as a partial and summed by a
-// second kernel) while the next item's MMAs run.  The host splits K only as far as the items fill the
-// CTAs.
+// accumulators.  The final value, two conversions scaled by exponent arithmetic and one FP64 add, is stored
+// (or, with split-K, written as a partial and summed by a second kernel) while the next item's MMAs run.
+// The host splits K only as far as the items fill the CTAs.
 // Bound: issue of the 128 x 64 x 16 MMAs by one warp beside 16 busy epilogue warps.  A pass runs its A tile (16 K
 // values) against all its B slices before the next, with the tile kept in the collector: 35 clocks per MMA alone
 // instead of 48 (shared-memory reads of A).  Measured per MMA in the kernel: 86 clocks with stages of whole 32-wide
 // chunks, 87 with a ring and an arrival barrier per slice, 68 with the arrivals merged into five per chunk (a wait
-// that finds its data there still costs about 130 clocks).  262144 x 600 x 600: 6.79 -> 5.50 ms, the Gram matrix of
-// 600 columns of 262144 4.03 -> 3.25 ms.
+// that finds its data there still costs about 130 clocks), 57 with the levels folded in integers.  262144 x 600 x 600:
+// 6.79 -> 4.6 ms, the Gram matrix of 600 columns of 262144 4.03 -> 2.75 ms.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -36,10 +36,10 @@ namespace {
 constexpr int S = kOzSlices;
 constexpr int BM = 128;
 constexpr int KC = 64;            // K tile of the slicing kernel (K is padded to a multiple of it)
-// Chunks accumulated in TMEM before a drain: 2 x 64 = 128 K terms per exact FP32 sum (each term a
-// product of two integer slices, |t_s t_r| <= 2^16, so every partial sum stays below 2^23).
 constexpr int KCH = 64;           // K chunk of the products: one 128-byte row of BF16 per slice
-constexpr int GROUP = 2;          // chunks per exact accumulation group (2 x 64 = 128 K terms)
+// Chunks accumulated in TMEM before a drain: 2 x 64 = 128 K terms per exact FP32 sum (bounds of the sums: oz_gemm.cuh).
+constexpr int GROUP = 2;
+constexpr int kMaxSplitChunks = 1 << 14;  // 2^20 K terms: what the epilogue's integers hold exactly
 constexpr int kARing = 8;         // A slices in flight (a power of two)
 constexpr int kBRing = 8;         // B slices 6 .. 1 in flight (a power of two); slice 0 alternates between two slots
 constexpr int kPassRing = 16;     // barriers of finished passes: more than the passes the producer runs ahead
@@ -516,8 +516,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int64_t it = blockIdx.x; it < p.items && ok; it += G) {
       const OzItem wi = oz_item(p, it);
       const int ngroups = (chunks_of(wi.split) + GROUP - 1) / GROUP;
-      // sum_L D_L 2^(48 - 8 L) = top 2^32 + low over all groups, exact in 64-bit integers (D_L below 2^24, up to
-      // 2^11 groups): a conversion and one wide multiply-add per level and column
+      // sum_L D_L 2^(48 - 8 L) = top 2^32 + low over all groups (at most kMaxSplitChunks / GROUP), exact in 64-bit
+      // integers: a conversion and one wide multiply-add per level and column
       long long top[16], low[16];
 #pragma unroll
       for (int u = 0; u < 16; ++u) top[u] = low[u] = 0;
@@ -744,7 +744,7 @@ void oz_gemm(cudaStream_t s, int num_sms, const OzOperand& A, const OzOperand& B
   // persistent CTAs over (tile, K split) items: split K only as far as the items then fill the CTAs
   double eff = 0.0;
   int nsplit = choose_split(kept, nchunks, num_sms, &eff);
-  nsplit = std::max(nsplit, (nchunks + (1 << 14) - 1) >> 14);  // the epilogue's integers hold 2^22 K terms
+  nsplit = std::max(nsplit, (nchunks + kMaxSplitChunks - 1) / kMaxSplitChunks);
   const int per = (nchunks + nsplit - 1) / nsplit;
   nsplit = (nchunks + per - 1) / per;
   const CUtensorMap ma = slice_map(A, BM);

@@ -11,10 +11,12 @@
 //     group of 128 K terms the sum of level L is an integer below 2^24 for L <= 5 and the FP32
 //     tensor-core accumulation of those levels is exact; the last level (weight 2^-48) could in the
 //     worst case lose one unit, an error below 2^-72 of the product, far under FP64 rounding;
-//   * each group's levels are combined as sum_L D_L 2^-8L into a float-float (hi, lo) accumulator
-//     (TwoSum), and C(i,j) = 2^(e_i + f_j - 16) (hi + lo) is formed in FP64 at the end.
-// The result carries ~2^-48 relative rounding per chunk combination, comparable to an FP64 GEMM's
-// own rounding for the shapes used here.
+//   * the levels of all groups are added in two 64-bit integers, exactly: top = sum D_L 2^(16 - 8 L) over L <= 2,
+//     low = sum D_L 2^(48 - 8 L) over L >= 3.  Per group |D_0|, |D_1| <= 2^23, |D_2| < 2^23.4, |D_3| < 2^23.6 and
+//     |D_6| < 2^24.2, so |top| < 2^39.01 and |low| < 2^47.7; over at most 2^20 K terms (2^13 groups; K is split
+//     beyond that) |top| stays below 2^53, exact in FP64, and |low| below 2^61;
+//   * C(i,j) = 2^(e_i + f_j - 64) (top 2^32 + low): two conversions, scaled by exponent arithmetic, and one FP64 add.
+// What is left out, the levels above 6 and the digits past the seventh, is below 2^-38 of a unit of D_0 per K term.
 #pragma once
 #include "common.cuh"
 
