@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(256) chol_inv_smem_kernel(int n, const double*
 // identity, one thread per (row, column mod 8), one CTA barrier per column; the chain of a column is
 // its FMA, the reciprocal of the pivot (an FP32 seed and 3 FP64 instructions) and one product.  The
 // square roots are taken at the end, for all 32 pivots in one go.  Those want pivots and reciprocals
-// that are normal: where A(0, 0) lies outside 2^-400 .. 2^400, A is scaled by a power of four on entry and the results
-// on exit (the pivots of a matrix that can be factored are within its condition number of each other).
+// that are normal: where A(0, 0) lies outside 2^-800 .. 2^800, A is scaled by 2^200 or 2^-200 on entry and the
+// results on exit.
 // info: 0, or j + 1 for the first column j whose pivot is not positive (L and L^-1 are then not
 // written in full).
 // Measured, one call: N = 60 60 us, N = 240 233 us, N = 600 0.78 ms.
@@ -398,8 +398,8 @@ __global__ void __launch_bounds__(256) chol_inv_blocked_kernel(int n, const doub
   auto put = [&](double* M, int i, int j, double v) {
     if (i < n && j < n) __stcg(M + (size_t)j * n + i, v);
   };
-  // 2^-h A is factored (h even); 0 but at the ends of the range
-  const int f0 = exp_field(A[0]), e0 = f0 == 0x7ff ? 0 : f0 - 1023, h = abs(e0) > 400 ? e0 & ~1 : 0;
+  // 2^-h A is factored; 0 but at the ends of the range
+  const int e0 = exp_field(A[0]) - 1023, h = e0 < -800 ? -200 : e0 > 800 ? 200 : 0;
   // L = lower(A), Linv = I
   for (size_t e = (size_t)r * blockDim.x + tid; e < nn; e += (size_t)P * blockDim.x) {
     const size_t j = e / n, i = e - j * n;

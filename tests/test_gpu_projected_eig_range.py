@@ -81,3 +81,15 @@ def test_gram_matrices_at_the_ends_of_the_range(power, mode):
     s.set_dense(np.ldexp(A, power), B=np.ldexp(B, power))
     _, ev = s.rayleigh_ritz(np.eye(N))
     assert np.abs(ev - ref).max() <= 50 * N * max(np.finfo(float).eps, 2.0 ** (-1074 - power)) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("powers", [(-1000, 0), (0, -1000), (-1000, 90), (900, -60), (-60, 900)])
+def test_graded_gram_matrices(powers):
+    """A diagonal B of two scales far apart, either first: the pivots are its entries, exact."""
+    N = 40
+    d = np.where(np.arange(N) < N // 2, 2.0 ** powers[0], 2.0 ** powers[1])
+    lam = np.linspace(1.0, 2.0, N)
+    s = Solver(N, nev=1, block=N, rr_mode="fp64")
+    s.set_dense(np.diag(d * lam), B=np.diag(d))
+    _, ev = s.rayleigh_ritz(np.eye(N))
+    assert np.abs(ev - lam).max() <= 50 * N * np.finfo(float).eps * 2.0
